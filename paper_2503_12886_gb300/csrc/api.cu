@@ -264,6 +264,7 @@ int prologue(rgba_ctx_t ctx, const rgba_batch *b, void *ws, size_t ws_bytes, voi
     finish_layout(call.p.L, cap);
     call.ws = static_cast<unsigned char *>(ws);
     call.c = make_ctx(call.p.L, call.ws, b);
+    call.c.masked = call.p.max_n <= kMaskedN;
     call.s = static_cast<cudaStream_t>(stream);
     cudaError_t e = cudaSetDevice(ctx->device);
     if (e != cudaSuccess) return cuda_fail(e, "cudaSetDevice");

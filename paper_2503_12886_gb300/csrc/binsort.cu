@@ -5,7 +5,8 @@
 // Design: the per-tile counts come out of the preprocess kernel (atomics whose return values
 // give each Gaussian its slot in up to 8 tiles), a three-phase scan (per-CTA partials, one CTA
 // over the partials, per-CTA writes) turns them into list offsets and a work list, a scatter
-// kernel drops (depth << 32 | index) keys into their tile's segment (by
+// kernel drops (depth << 32 | index) keys, with a mask of the pixel blocks each splat reaches in
+// the low byte of the index word, into their tile's segment (by
 // slot, or by a cursor atomic for larger rectangles), and one CTA per non-empty tile sorts its
 // list, with the key compressed to (depth - segment minimum) << 32 | index: in shared memory by
 // one bucket pass on the top depth bits and a placement of every key by its rank in its bucket,
@@ -200,7 +201,64 @@ __global__ void __launch_bounds__(kScanTile) k_scan_write(Ctx c) {
 
 constexpr int kScatterThreads = 128;
 
+// The region where a splat reaches alpha 1/255: the ellipse a dx^2 + 2 b dx dy + c dy^2 <= s,
+// s = -2 alpha_cut(o), around (u, v).
+struct Reach {
+    bool none, all;  // never reaches it; too elongated to bound tightly
+    float u, v, ia, b, det, as, ys, hy;
+};
+
+// The square roots and quotients are the hardware's approximate ones: the widening below covers
+// their few ulp many times over.
+__device__ __forceinline__ float sqrt_fast(float x) {
+    float y;
+    asm("sqrt.approx.ftz.f32 %0, %1;" : "=f"(y) : "f"(x));
+    return y;
+}
+
+// s is widened by 2 % and each block by 0.05 px, so that whatever is excluded fails the per-pixel
+// FP32 test with room to spare: that test's power is off by at most a few 2^-24 (a dx^2 + c dy^2),
+// which on the ellipse is a few 2^-24 s / (1 - b^2 / ac). Beyond ac / det = 10^4 (a splat a hundred
+// times longer than wide) neither bound is trusted and every block is taken.
+__device__ __forceinline__ Reach reach_of(const float4 &r0, const float2 &r1) {
+    Reach e;
+    const float a = r0.z, b = r0.w, c = r1.x, tau = alpha_cut(r1.y);
+    const float det = a * c - b * b;
+    e.none = !(tau < 0.0f && det > 0.0f);
+    e.all = !(a * c < 1e4f * det);
+    const float s = -2.04f * tau, id = __fdividef(1.0f, det);
+    e.u = r0.x;
+    e.v = r0.y;
+    e.ia = __fdividef(1.0f, a);
+    e.b = b;
+    e.det = det;
+    e.as = a * s;
+    e.hy = sqrt_fast(e.as * id);
+    const float hx = sqrt_fast(s * c * id);
+    e.ys = -__fdividef(b, c) * hx;  // dy where the ellipse is furthest right (minus it: furthest left)
+    return e;
+}
+
+// The x extent [xl, xr] of the ellipse over pixel-centre rows y .. y + 3, widened (empty: xl > xr).
+// The right end over the rows is where dy is closest to ys, the left end closest to -ys.
+__device__ __forceinline__ void reach_rows(const Reach &e, float y, float &xl, float &xr) {
+    const float d0 = y - 0.05f - e.v, d1 = y + 3.05f - e.v;
+    xl = 1.0f;
+    xr = -1.0f;
+    if (d0 > e.hy || d1 < -e.hy) return;
+    const float yr = fminf(fmaxf(e.ys, d0), d1), yl = fminf(fmaxf(-e.ys, d0), d1);
+    xr = e.u + 0.05f + (sqrt_fast(fmaxf(0.0f, e.as - e.det * yr * yr)) - e.b * yr) * e.ia;
+    xl = e.u - 0.05f - (sqrt_fast(fmaxf(0.0f, e.as - e.det * yl * yl)) + e.b * yl) * e.ia;
+}
+
+// One thread per (frame, Gaussian): drops its key into the list of every tile of its rectangle,
+// with the tile's block mask. The masks cost one ellipse extent per four pixel rows of the
+// rectangle and two compares per block; computed here they are paid once per (Gaussian, tile),
+// where every compositing warp of a tile (eight, forwards and again backwards) would test every
+// entry of its list. TW: the tile width (16 or 8).
+template <int TW>
 __global__ void __launch_bounds__(kScatterThreads) k_scatter(Ctx c) {
+    constexpr int TH = kTilePix / TW, NBX = TW / 8, BANDS = TH / 4;
     pdl_enter();
     if (c.cnt->overflow) return;
     const int b = blockIdx.y;
@@ -208,21 +266,25 @@ __global__ void __launch_bounds__(kScatterThreads) k_scatter(Ctx c) {
     const int i = blockIdx.x * blockDim.x + threadIdx.x;
     if (i >= f.n) return;
     const long long r = f.rec_base + i;
+    // every load of the record at once (few Gaussians are culled)
     const ushort4 rc = c.rects[r];
-    if (rc.z <= rc.x || rc.w <= rc.y) return;
     const unsigned bits = __float_as_uint(c.depth[r]);
-    const unsigned long long key = ((unsigned long long)bits << 32) | (unsigned)i;
+    const float4 r0 = c.records[r * 3];
+    const float2 r1 = *reinterpret_cast<const float2 *>(c.records + r * 3 + 1);
+    const uint4 *rp = reinterpret_cast<const uint4 *>(c.ranks + r * kRankSlots);
+    const uint4 q0 = rp[0], q1 = rp[1];
+    if (rc.z <= rc.x || rc.w <= rc.y) return;
     const int w = rc.z - rc.x, area = w * (rc.w - rc.y);
-    if (area <= kRankSlots) {  // slots recorded by the preprocess: no atomics
-        const uint4 *rp = reinterpret_cast<const uint4 *>(c.ranks + r * kRankSlots);
-        const uint4 r0 = rp[0], r1 = rp[1];
-        const unsigned rk[kRankSlots] = {r0.x, r0.y, r0.z, r0.w, r1.x, r1.y, r1.z, r1.w};
-        const unsigned *ts = c.tile_start + f.tile_base + (long long)rc.y * f.tiles_x + rc.x;
-        int ox = 0, off = 0;  // slot q is tile (rc.x + ox, rc.y + q / w), off its offset from ts
+    const bool ranked = area <= kRankSlots;  // slots recorded by the preprocess: no atomics
+    unsigned rk[kRankSlots] = {q0.x, q0.y, q0.z, q0.w, q1.x, q1.y, q1.z, q1.w};
+    const unsigned *ts = c.tile_start + f.tile_base;
+    if (ranked) {  // every list start in flight while the masks are computed
+        const unsigned *t0 = ts + (long long)rc.y * f.tiles_x + rc.x;
+        int ox = 0, off = 0;  // slot q is tile (rc.x + ox, rc.y + q / w), off its offset from t0
 #pragma unroll
         for (int q = 0; q < kRankSlots; ++q) {
             if (q < area) {
-                c.keys[ts[off] + rk[q]] = key;
+                rk[q] += __ldg(t0 + off);
                 ++off;
                 if (++ox == w) {
                     ox = 0;
@@ -230,15 +292,36 @@ __global__ void __launch_bounds__(kScatterThreads) k_scatter(Ctx c) {
                 }
             }
         }
-        return;
     }
-    unsigned *cur = c.cursor + (r & (kSubCounters - 1));
-    for (int ty = rc.y; ty < rc.w; ++ty)
+    const Reach e = reach_of(r0, r1);
+    unsigned *cur = c.cursor + (size_t)f.tile_base * kSubCounters + (r & (kSubCounters - 1));
+    for (int ty = rc.y; ty < rc.w; ++ty) {
+        float xl[BANDS], xr[BANDS];
+#pragma unroll
+        for (int k = 0; k < BANDS; ++k) reach_rows(e, (float)(ty * TH + 4 * k) + 0.5f, xl[k], xr[k]);
         for (int tx = rc.x; tx < rc.z; ++tx) {
-            const long long gt = f.tile_base + (long long)ty * f.tiles_x + tx;
-            const unsigned pos = c.tile_start[gt] + atomicAdd(cur + gt * kSubCounters, 1u);
-            c.keys[pos] = key;
+            unsigned mask = 0u;
+#pragma unroll
+            for (int k = 0; k < BANDS; ++k)
+#pragma unroll
+                for (int q = 0; q < NBX; ++q) {
+                    const float x0 = (float)(tx * TW + 8 * q) + 0.5f;
+                    if (xr[k] >= x0 && xl[k] <= x0 + 7.0f) mask |= 1u << (k * NBX + q);
+                }
+            if (e.all) mask = 0xffu;
+            if (e.none) mask = 0u;
+            const long long t = (long long)ty * f.tiles_x + tx;
+            unsigned pos;
+            if (ranked) {  // the slots in tile order: take the first, move the others up
+                pos = rk[0];
+#pragma unroll
+                for (int q = 0; q + 1 < kRankSlots; ++q) rk[q] = rk[q + 1];
+            } else {
+                pos = ts[t] + atomicAdd(cur + t * kSubCounters, 1u);
+            }
+            c.keys[pos] = ((unsigned long long)bits << 32) | pack_low(c.masked, (unsigned)i, mask);
         }
+    }
 }
 
 // Asynchronous 8-byte copy global -> shared (both addresses 8-byte aligned), completed by
@@ -473,13 +556,14 @@ __device__ unsigned long long *bucket_sort(unsigned long long *a, unsigned long 
 // keys again fit in the same shared memory: a shared-memory atomic per
 // key gives its bucket and its slot, a scan the bucket starts, each key's position goes to its
 // bucket's run in s_pos, and every key counts the smaller keys of its bucket (read through the
-// positions) and writes its Gaussian index straight to its rank in the tile's list `out`.
+// positions) and writes its Gaussian index and block mask straight to its rank in the tile's lists
+// `out` and `out_mask`.
 // Returns false when some bucket is longer than kBucketRun (its keys are then not written; the
 // caller sorts the whole segment again another way).
 __device__ bool bucket_sort_pos(const unsigned long long *a, int L, unsigned d0, int db,
                                 unsigned *s_hist /* >= 2^kBucketBits + kSortWarps, zeroed */,
-                                unsigned short *s_rank, unsigned short *s_pos, unsigned *s_long,
-                                unsigned *__restrict__ out) {
+                                unsigned short *s_rank, unsigned short *s_pos, unsigned *s_long, bool masked,
+                                unsigned *__restrict__ out, unsigned char *__restrict__ out_mask) {
     constexpr int NB = 1 << kBucketBits, PER = NB / kSortThreads;
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
     const int bshift = max(0, db - kBucketBits);
@@ -522,14 +606,16 @@ __device__ bool bucket_sort_pos(const unsigned long long *a, int L, unsigned d0,
         }
         int rank = 0;
         for (int q = lo; q < hi; ++q) rank += a[s_pos[q]] < k;
-        out[lo + rank] = (unsigned)k;
+        out[lo + rank] = low_index(masked, (unsigned)k);
+        out_mask[lo + rank] = low_mask(masked, (unsigned)k);
     }
     __syncthreads();
     return *s_long == 0u;
 }
 
 // Persistent: CTAs take (frame, tile) segments from the LPT-ordered work list. A key is
-// (depth, Gaussian index); it is compressed to (depth - min depth) << 32 | index. A segment of
+// (depth, Gaussian index), "index" standing here for the word that also holds the block mask below
+// the index; it is compressed to (depth - min depth) << 32 | index. A segment of
 // up to kRadixCap keys is sorted in shared memory by bucket_sort (one bucket pass, then each
 // bucket by the full key), one of up to kMidCap keys by bucket_sort_pos (the same with 2-byte
 // positions in place of moved keys). A longer one is radix-sorted in place in global memory
@@ -583,6 +669,7 @@ __global__ void __launch_bounds__(kSortThreads) k_tile_sort(Ctx c) {
             w3 = atomicAdd(&c.cnt->next_sort, 1u);
         }
         const unsigned long long *g = c.keys + st;
+        unsigned char *masks = c.list_masks(st);  // over the list's keys, once nobody reads them
         const bool in_smem = L <= (unsigned)kRadixCap;
         const bool mid = !in_smem && L <= (unsigned)kMidCap;  // the position bucket sort
         unsigned dmin = 0xffffffffu, dmax = 0u, imax = 0u;
@@ -627,7 +714,8 @@ __global__ void __launch_bounds__(kSortThreads) k_tile_sort(Ctx c) {
         unsigned long long *res = nullptr;  // stays null when the keys' indices are already written
         bool done = false;
         if (mid) {
-            done = bucket_sort_pos(s_keys, (int)L, d0, db, s_cnt, s_rank_mid, s_pos_mid, &s_long, c.sorted + st);
+            done = bucket_sort_pos(s_keys, (int)L, d0, db, s_cnt, s_rank_mid, s_pos_mid, &s_long, c.masked,
+                                   c.sorted + st, masks);
             __syncthreads();  // every thread has read the flag before it is cleared
             if (!done) {      // a crowded bucket: sort the segment in global memory below
                 if (threadIdx.x == 0) s_long = 0u;
@@ -645,7 +733,9 @@ __global__ void __launch_bounds__(kSortThreads) k_tile_sort(Ctx c) {
                 res = radix_sort<true>(res, other, (int)L, 32, 32 + db, s_cnt, s_rank);
             }
         } else {
-            compress(a, g);
+            // a crowded list of the position sort is still whole in shared memory; its place in
+            // global memory already holds some of its masks
+            compress(a, mid ? s_keys : g);
             res = radix_sort<false>(a, bb, (int)L, 32, 32 + db, s_cnt, nullptr);
             // ties: a run keeps its depth under any reordering, so run starts found by other
             // threads do not change while a run is being ordered
@@ -674,8 +764,17 @@ __global__ void __launch_bounds__(kSortThreads) k_tile_sort(Ctx c) {
                 res = radix_sort<false>(res, other, (int)L, 32, 32 + db, s_cnt, nullptr);
             }
         }
+        if (res == g) {  // the masks go over this buffer: finish from the other one
+            for (unsigned e = threadIdx.x; e < L; e += blockDim.x) a[e] = res[e];
+            __syncthreads();
+            res = a;
+        }
         if (res)
-            for (unsigned e = threadIdx.x; e < L; e += blockDim.x) c.sorted[st + e] = (unsigned)res[e];
+            for (unsigned e = threadIdx.x; e < L; e += blockDim.x) {
+                const unsigned low = (unsigned)res[e];
+                c.sorted[st + e] = low_index(c.masked, low);
+                masks[e] = low_mask(c.masked, low);
+            }
         __syncthreads();
         if (threadIdx.x == 0) {
             s_cur = w1 < n_work ? 1u : 0u;
@@ -716,7 +815,7 @@ size_t scan_aux_bytes(long long T) {
 cudaError_t launch_scatter(const Ctx &c, int max_n, cudaStream_t s) {
     if (c.B == 0 || max_n == 0) return cudaSuccess;
     dim3 grid((max_n + kScatterThreads - 1) / kScatterThreads, c.B);
-    return launch_pdl(k_scatter, grid, dim3(kScatterThreads), 0, s, c);
+    return launch_pdl(c.tw == 16 ? k_scatter<16> : k_scatter<8>, grid, dim3(kScatterThreads), 0, s, c);
 }
 
 cudaError_t launch_tile_sort(const Ctx &c, int sms, cudaStream_t s) {

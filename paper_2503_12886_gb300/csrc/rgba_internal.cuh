@@ -122,6 +122,27 @@ struct Layout {
     int max_n_pad;
 };
 
+// A list entry carries the pixel blocks (8 x 4 pixels, 8 to a tile) its splat can reach: bit k is
+// set unless the splat stays below alpha 1/255 at every pixel of block k, so a compositing warp
+// picks its block's entries from one byte each, without touching the others' records. The masks are
+// made where a Gaussian's tiles are enumerated (k_scatter) and travel through the sort in the low
+// byte of the key's index word, below the index, so that they never decide an order; the sort
+// leaves them at one byte per entry at the start of the list's own (by then consumed) key segment.
+// Models of more than 2^24 Gaussians need the whole word for the index: their lists' masks are all
+// ones.
+constexpr long long kMaskedN = 1LL << 24;
+__device__ __forceinline__ unsigned pack_low(bool masked, unsigned idx, unsigned mask) {
+    return masked ? (idx << 8) | mask : idx;
+}
+__device__ __forceinline__ unsigned low_index(bool masked, unsigned low) { return masked ? low >> 8 : low; }
+__device__ __forceinline__ unsigned char low_mask(bool masked, unsigned low) {
+    return masked ? (unsigned char)low : (unsigned char)0xffu;
+}
+
+// -ln(255 o): alpha = o e^power is below 1/255 exactly when power is below this. One definition for
+// the masks and for the compositing, so that they cut at the same value.
+__device__ __forceinline__ float alpha_cut(float o) { return -__logf(255.0f * o); }
+
 // Everything a kernel needs to find its data (passed by value).
 struct Ctx {
     const ModelInfo *models;
@@ -143,14 +164,20 @@ struct Ctx {
     float4 *cache;     // [R][3]
     float *grad2d;     // [R][12]
     unsigned long long *keys;
-    unsigned long long *keys2;  // [cap]: second buffer of the global-memory radix passes
+    unsigned long long *keys2;  // [cap]: second buffer of the sort of long lists
     unsigned *sorted;
+    // keys carry a pixel-block mask (pack_low): every model has at most kMaskedN Gaussians
+    bool masked;
     float *dpsi_part;
     unsigned *ranks;   // [R][kRankSlots]: slot of the Gaussian in each tile of its rectangle
     float *depth;      // [R]: view-space depth of each kept record (the scatter's sort key)
     long long R, T, cap;
     int B, M, k_stride, tw, th;
     int loss_frames;       // the loss is averaged over this many frames (>= B)
+    // the block masks of the list that starts at entry st
+    __device__ __forceinline__ unsigned char *list_masks(unsigned st) const {
+        return reinterpret_cast<unsigned char *>(keys + st);
+    }
 };
 
 // Programmatic dependent launch (Hopper/Blackwell): a kernel launched with launch_pdl may be
