@@ -327,8 +327,8 @@ int rgba_profile_read(rgba_ctx_t ctx, rgba_profile *out);
  * accounting: how many list entries the kernels evaluated and how many of those blend.
  * Synchronous; out: host. */
 typedef struct {
-    int64_t fwd_staged;  /* list entries the forward's pixel-block warps staged */
-    int64_t fwd_hits;    /* (list entry, 8x4 pixel block) pairs whose alpha box meets the block */
+    int64_t fwd_staged;  /* list entries whose masks the forward's pixel-block warps scanned */
+    int64_t fwd_hits;    /* (list entry, 8x4 pixel block) pairs whose mask has the block */
     int64_t fwd_visits;  /* hits at which some pixel of the block passes the cutoffs (the entry
                             is then composited at the block) */
     int64_t fwd_blends;  /* (pixel, entry) pairs the forward blended */

@@ -10,9 +10,8 @@
 // slot, or by a cursor atomic for larger rectangles), and one CTA per non-empty tile sorts its
 // list, with the key compressed to (depth - segment minimum) << 32 | index: in shared memory by
 // one bucket pass on the top depth bits and a placement of every key by its rank in its bucket,
-// or, for long segments, through L2 by a stable LSD radix sort over the depth bits and a pass
-// that orders runs of equal depth by index. Because the key carries the index, the result is
-// unique.
+// or, for long segments, by the same bucket pass with the keys in L2; buckets too crowded for it
+// fall back to a stable LSD radix sort. Because the key carries the index, the result is unique.
 #include "rgba_internal.cuh"
 
 namespace rgba {
@@ -613,17 +612,92 @@ __device__ bool bucket_sort_pos(const unsigned long long *a, int L, unsigned d0,
     return *s_long == 0u;
 }
 
+constexpr int kStreamBits = 14;  // buckets of the sort of long lists, in the key area of the others
+constexpr int kStreamLoads = 8;  // keys per thread in flight in its sweeps
+static_assert((4 << kStreamBits) <= kRadixCap * 16, "bucket counts fit the key area");
+
+// Calls f(key) for the L keys at g, kStreamLoads of each thread's loads in flight at once.
+template <typename F>
+__device__ __forceinline__ void sweep(const unsigned long long *g, int L, F f) {
+    for (int e0 = threadIdx.x; e0 < L; e0 += kStreamLoads * kSortThreads) {
+        unsigned long long k[kStreamLoads];
+#pragma unroll
+        for (int u = 0; u < kStreamLoads; ++u) {
+            const int e = e0 + u * kSortThreads;
+            k[u] = e < L ? g[e] : 0ull;
+        }
+#pragma unroll
+        for (int u = 0; u < kStreamLoads; ++u)
+            if (e0 + u * kSortThreads < L) f(k[u]);
+    }
+}
+
+// Sort of a list too long for shared memory: the same bucket pass with the keys in global memory
+// (L2) and only the bucket counts in shared memory. One sweep counts the 2^kStreamBits buckets of
+// the depth spread, a scan turns the counts into starts, a second sweep moves every key to its
+// bucket's run in tmp (a shared-memory atomic gives the place; any order within the bucket), and a
+// third ranks each key among its bucket's (a few neighbours in tmp) and writes its index and mask.
+// Every sweep keeps kStreamLoads loads per thread in flight; a list of 24,000 keys takes three
+// sweeps instead of the radix sort's four passes of two dependent sweeps each with a warp-wide digit
+// match per key. Returns false, with nothing written, when some bucket is longer than kBucketRun.
+__device__ bool bucket_sort_stream(const unsigned long long *g, unsigned long long *tmp, int L, unsigned d0, int db,
+                                   unsigned *s_cnt /* [2^kStreamBits] */, unsigned *s_sum /* [kSortWarps] */,
+                                   bool masked, unsigned *__restrict__ out, unsigned char *__restrict__ out_mask) {
+    constexpr int NB = 1 << kStreamBits, PER = NB / kSortThreads;
+    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+    const int bshift = max(0, db - kStreamBits);
+    auto bucket = [&](unsigned long long k) { return ((unsigned)(k >> 32) - d0) >> bshift; };
+    for (int i = tid; i < NB; i += kSortThreads) s_cnt[i] = 0u;
+    __syncthreads();
+    sweep(g, L, [&](unsigned long long k) { atomicAdd(&s_cnt[bucket(k)], 1u); });
+    __syncthreads();
+    // exclusive scan of the counts; warp w owns buckets [w NB/W, (w+1) NB/W) and walks them 32 at a
+    // time (neighbouring lanes, neighbouring banks)
+    unsigned longest = 0u, run = 0u;
+    for (int i = 0; i < PER; ++i) {
+        unsigned *p = s_cnt + warp * (PER * 32) + 32 * i + lane;
+        const unsigned v = *p;
+        unsigned x = v;
+#pragma unroll
+        for (int o = 1; o < 32; o <<= 1) {
+            const unsigned y = __shfl_up_sync(0xffffffffu, x, o);
+            if (lane >= o) x += y;
+        }
+        *p = run + x - v;
+        run += __shfl_sync(0xffffffffu, x, 31);
+        longest = max(longest, v);
+    }
+    if (lane == 0) s_sum[warp] = run;
+    if (__syncthreads_or(longest > (unsigned)kBucketRun)) return false;
+    unsigned off = 0u;
+    for (int w = 0; w < warp; ++w) off += s_sum[w];
+    for (int i = 0; i < PER; ++i) s_cnt[warp * (PER * 32) + 32 * i + lane] += off;
+    __syncthreads();
+    sweep(g, L, [&](unsigned long long k) { tmp[atomicAdd(&s_cnt[bucket(k)], 1u)] = k; });
+    __syncthreads();  // s_cnt[b] is now the end of bucket b; the keys at g are no longer needed
+    sweep(tmp, L, [&](unsigned long long k) {
+        const unsigned b = bucket(k);
+        const int lo = b ? (int)s_cnt[b - 1] : 0, hi = (int)s_cnt[b];
+        int rank = lo;
+        for (int q = lo; q < hi; ++q) rank += tmp[q] < k;
+        out[rank] = low_index(masked, (unsigned)k);
+        out_mask[rank] = low_mask(masked, (unsigned)k);
+    });
+    return true;
+}
+
 // Persistent: CTAs take (frame, tile) segments from the LPT-ordered work list. A key is
 // (depth, Gaussian index), "index" standing here for the word that also holds the block mask below
 // the index; it is compressed to (depth - min depth) << 32 | index. A segment of
 // up to kRadixCap keys is sorted in shared memory by bucket_sort (one bucket pass, then each
 // bucket by the full key), one of up to kMidCap keys by bucket_sort_pos (the same with 2-byte
-// positions in place of moved keys). A longer one is radix-sorted in place in global memory
-// (mostly L2) on the depth bits only, which leaves runs of equal depth in list order, and a tie
-// pass orders each such run by index (insertion sort by the run's first thread). A bucket longer
-// than kBucketRun or a run longer than kTieRun sends the segment to a full-key sort: radix passes
-// on the index bits, then on the depth bits (a segment of bucket_sort_pos goes to the global-memory
-// sort).
+// positions in place of moved keys). A longer one is sorted by bucket_sort_stream with its keys in
+// global memory (mostly L2). A bucket longer than kBucketRun sends a segment of bucket_sort to a
+// full-key radix sort (index bits, then depth bits), and a longer one to a radix sort in global memory
+// on the depth bits only, which leaves runs of equal depth in list order; a tie pass orders each such
+// run by index (insertion sort by the run's first thread), a run longer than kTieRun the full key.
+// Long lists through L2 by buckets instead of radix passes: a batch of 15 frames of five avatars
+// with lists of up to 23,803 keys 475 -> 147 us, 64 frames of eight avatars (24,502) 500 -> 268 us.
 // The sort is bound by round trips to memory, so none of them waits on another: thread 0 claims
 // work items three ahead and, one stage per item, loads the claimed item's tile id and then its
 // list bounds while the CTA sorts the current segment; a segment that fits in shared memory
@@ -679,13 +753,16 @@ __global__ void __launch_bounds__(kSortThreads) k_tile_sort(Ctx c) {
             asm volatile("cp.async.wait_all;" ::: "memory");
             __syncthreads();
         }
-        for (unsigned e = threadIdx.x; e < L; e += blockDim.x) {
-            const unsigned long long k = in_smem || mid ? s_keys[e] : g[e];
+        auto widen = [&](unsigned long long k) {
             const unsigned d = (unsigned)(k >> 32), i = (unsigned)k;
             dmin = min(dmin, d);
             dmax = max(dmax, d);
             imax = max(imax, i);
-        }
+        };
+        if (in_smem || mid)
+            for (unsigned e = threadIdx.x; e < L; e += blockDim.x) widen(s_keys[e]);
+        else
+            sweep(g, (int)L, widen);
         for (int o = 16; o > 0; o >>= 1) {
             dmin = min(dmin, __shfl_xor_sync(0xffffffffu, dmin, o));
             dmax = max(dmax, __shfl_xor_sync(0xffffffffu, dmax, o));
@@ -721,6 +798,9 @@ __global__ void __launch_bounds__(kSortThreads) k_tile_sort(Ctx c) {
                 if (threadIdx.x == 0) s_long = 0u;
                 __syncthreads();
             }
+        } else if (!in_smem) {
+            done = bucket_sort_stream(g, c.keys2 + st, (int)L, d0, db, reinterpret_cast<unsigned *>(s_keys), s_cnt,
+                                      c.masked, c.sorted + st, masks);
         }
         if (done) {
         } else if (in_smem) {
