@@ -405,7 +405,7 @@ int do_gauss_bwd(rgba_ctx_t ctx, Call &k, const FusedAdam *fa) {
             max_ka = std::max(max_ka, m.k * m.A);
             any_bound = any_bound || m.n_faces > 0;
         }
-        if ((e = launch_gauss_bwd(k.c, k.p.max_chunks, k.p.max_k, max_ka, fa, any_bound, k.s)) != cudaSuccess)
+        if ((e = launch_gauss_bwd(k.c, k.p.max_chunks, k.p.max_nb, k.p.max_k, max_ka, fa, any_bound, k.s)) != cudaSuccess)
             return cuda_fail(e, "gauss bwd");
     }
     if (k.c.grad_psi) {

@@ -1,6 +1,6 @@
 // Backward through the projection (EWA splatting, activations) and the linear blend (Eq. 1).
 //
-//   k_gauss_bwd  one CTA per 32 Gaussians of one model, lane = Gaussian, frames 16 at a time:
+//   k_gauss_bwd  one CTA per 32 Gaussians of one model, lane = Gaussian, frames 8 or 16 at a time:
 //                first, per (frame, Gaussian), the 2-D gradients dL/d(u, v, conic, opacity,
 //                colour) from the compositing backward's sums -> dL/dG_b over the 14 channels
 //                (chain rule through conic inversion, J W Sigma W^T J^T, R diag(s^2) R^T,
@@ -23,215 +23,124 @@ namespace {
 
 constexpr int kBwdThreads = 256;
 
-// The backward needs no bit-exact replay of the forward decisions (those come from the
-// records), only fp32 values to the gradient tolerance, so it uses the hardware's fast
-// reciprocal, reciprocal square root and exponential.
-struct Fwd {
-    float p[3], qn[4], il, s[3], R[3][3], M[3][3], J[2][3], rx, ry, ipz;
-    bool clx, cly;
-    float A, B, C, det;
-};
-
-// BOUND: Rt [12] = TBN matrix row-major (columns T, B, N), then t (the identity and zero for an
-// unbound model of a batch that also has bound ones); the Gaussian is mapped from tangent space
-// by x = R x_T + t, covariance R Sigma R^T. !BOUND: no mapping (Rt is not read).
-template <bool BOUND>
-__device__ __forceinline__ void recompute(const float v[10], const float *V, int W, int H, const float *Rt, Fwd &f) {
-    float xm[3];
-#pragma unroll
-    for (int c = 0; c < 3; ++c)
-        xm[c] = BOUND ? Rt[3 * c] * v[0] + Rt[3 * c + 1] * v[1] + Rt[3 * c + 2] * v[2] + Rt[9 + c] : v[c];
-#pragma unroll
-    for (int j = 0; j < 3; ++j) f.p[j] = V[4 * j] * xm[0] + V[4 * j + 1] * xm[1] + V[4 * j + 2] * xm[2] + V[4 * j + 3];
-#pragma unroll
-    for (int m = 0; m < 3; ++m) f.s[m] = __expf(v[7 + m]);
-    f.il = rsqrtf(v[3] * v[3] + v[4] * v[4] + v[5] * v[5] + v[6] * v[6]);
-#pragma unroll
-    for (int m = 0; m < 4; ++m) f.qn[m] = v[3 + m] * f.il;
-    const float w = f.qn[0], x = f.qn[1], y = f.qn[2], z = f.qn[3];
-    f.R[0][0] = 1.f - 2.f * (y * y + z * z);
-    f.R[0][1] = 2.f * (x * y - w * z);
-    f.R[0][2] = 2.f * (x * z + w * y);
-    f.R[1][0] = 2.f * (x * y + w * z);
-    f.R[1][1] = 1.f - 2.f * (x * x + z * z);
-    f.R[1][2] = 2.f * (y * z - w * x);
-    f.R[2][0] = 2.f * (x * z - w * y);
-    f.R[2][1] = 2.f * (y * z + w * x);
-    f.R[2][2] = 1.f - 2.f * (x * x + y * y);
-    float Sg[3][3];
-#pragma unroll
-    for (int i = 0; i < 3; ++i)
-#pragma unroll
-        for (int j = 0; j < 3; ++j) {
-            float a = 0.f;
-#pragma unroll
-            for (int m = 0; m < 3; ++m) a += f.R[i][m] * f.s[m] * f.s[m] * f.R[j][m];
-            Sg[i][j] = a;
-        }
-    if (BOUND) {
-        float P[3][3];
-#pragma unroll
-        for (int i = 0; i < 3; ++i)
-#pragma unroll
-            for (int j = 0; j < 3; ++j) P[i][j] = Rt[3 * i] * Sg[0][j] + Rt[3 * i + 1] * Sg[1][j] + Rt[3 * i + 2] * Sg[2][j];
-#pragma unroll
-        for (int i = 0; i < 3; ++i)
-#pragma unroll
-            for (int j = 0; j < 3; ++j) Sg[i][j] = P[i][0] * Rt[3 * j] + P[i][1] * Rt[3 * j + 1] + P[i][2] * Rt[3 * j + 2];
-    }
-    float Tm[3][3];
-#pragma unroll
-    for (int i = 0; i < 3; ++i)
-#pragma unroll
-        for (int j = 0; j < 3; ++j) Tm[i][j] = V[4 * i] * Sg[0][j] + V[4 * i + 1] * Sg[1][j] + V[4 * i + 2] * Sg[2][j];
-#pragma unroll
-    for (int i = 0; i < 3; ++i)
-#pragma unroll
-        for (int j = 0; j < 3; ++j) f.M[i][j] = Tm[i][0] * V[4 * j] + Tm[i][1] * V[4 * j + 1] + Tm[i][2] * V[4 * j + 2];
-    const float fx = V[12], fy = V[13], pz = f.p[2];
-    const float limx = 1.3f * __fdividef(0.5f * W, fx), limy = 1.3f * __fdividef(0.5f * H, fy);
-    f.ipz = __frcp_rn(pz);
-    const float rx = f.p[0] * f.ipz, ry = f.p[1] * f.ipz;
-    f.clx = rx > limx || rx < -limx;
-    f.cly = ry > limy || ry < -limy;
-    f.rx = fminf(limx, fmaxf(-limx, rx));
-    f.ry = fminf(limy, fmaxf(-limy, ry));
-    f.J[0][0] = fx * f.ipz;
-    f.J[0][1] = 0.f;
-    f.J[0][2] = -fx * f.rx * f.ipz;
-    f.J[1][0] = 0.f;
-    f.J[1][1] = fy * f.ipz;
-    f.J[1][2] = -fy * f.ry * f.ipz;
-    float S2[2][2];
-#pragma unroll
-    for (int i = 0; i < 2; ++i)
-#pragma unroll
-        for (int j = 0; j < 2; ++j) {
-            float a = 0.f;
-#pragma unroll
-            for (int p = 0; p < 3; ++p)
-#pragma unroll
-                for (int q = 0; q < 3; ++q) a += f.J[i][p] * f.M[p][q] * f.J[j][q];
-            S2[i][j] = a;
-        }
-    f.A = S2[0][0] + 0.3f;
-    f.B = S2[0][1];
-    f.C = S2[1][1] + 0.3f;
-    f.det = f.A * f.C - f.B * f.B;
-}
-
-// dG[14]: gradient w.r.t. the blended channels of one (frame, Gaussian). g2: the compositing
-// backward's sums over the pixels that blend the Gaussian, S = (S1, S2, S3, S4, S5, S0) of
+// The gradient of one (frame, Gaussian) with respect to its 14 blended channels, from the
+// compositing backward's sums over the pixels that blend it: S = (S1, S2, S3, S4, S5, S0) of
 // g (dx, dy, dx^2, dx dy, dy^2, 1) with g = dL/dpower and (dx, dy) = pixel centre - mean, then
 // dL/d(r, g, b). As power = -(a dx^2 + c dy^2) / 2 - b dx dy and alpha = o e^power:
 // dL/du = a S1 + b S2, dL/dv = b S1 + c S2, dL/d(a, b, c) = (-S3 / 2, -S4, -S5 / 2) and
-// dL/do = S0 / o, with the conic (a, b, c) = Sigma'^-1 recomputed here.
+// dL/do = S0 / o, with the conic Q = (a, b, c) = Sigma'^-1 recomputed here.
+//
+// The 2-D covariance is kept as a product of thin factors, Sigma' = U diag(s^2) U^T + 0.3 I with
+// U = T R and T = J W (2 x 3), so that no 3 x 3 product is formed on the way back either:
+//   G = dL/dSigma' = -Q dL/dQ Q,   dL/ds_m^2 = (U^T G U)_mm,   X = dL/dU = 2 G U diag(s^2),
+//   dL/dR = T^T X,   dL/dT = X R^T,   dL/dJ = dL/dT W^T.
+// That is about 300 operations where the 3 x 3 covariances and their adjoints took about 900.
+// The backward needs no bit-exact replay of the forward decisions (those come from the
+// records), only fp32 values to the gradient tolerance, so it uses the hardware's fast
+// reciprocal, reciprocal square root and exponential.
+//
+// v: mean(3), quaternion(4), log-scale(3); V: the frame's parameters; lim: the Jacobian clamp
+// bounds 1.3 tan(fov / 2) in x and y. BOUND: Rt [12] = TBN matrix row-major (columns T, B, N), then t
+// (the identity and zero for an unbound model of a batch that also has bound ones); the Gaussian
+// is mapped from tangent space by x = Rt x_T + t, which makes W the view rotation times Rt. !BOUND:
+// no mapping (Rt is not read).
 template <bool BOUND>
-__device__ __forceinline__ void chain(const float v[10], float op, const float *V, int W, int H,
+__device__ __forceinline__ void chain(const float v[10], float op, const float *V, const float *lim,
                                       const float *Rt, const float g2[9], float dG[kNch]) {
-    Fwd f;
-    recompute<BOUND>(v, V, W, H, Rt, f);
-    const float A = f.A, B = f.B, C = f.C, D = f.det, iD = __frcp_rn(D), iD2 = iD * iD;
+    float W[3][3], p[3];
+#pragma unroll
+    for (int j = 0; j < 3; ++j) {
+#pragma unroll
+        for (int c = 0; c < 3; ++c)
+            W[j][c] = BOUND ? V[4 * j] * Rt[c] + V[4 * j + 1] * Rt[3 + c] + V[4 * j + 2] * Rt[6 + c] : V[4 * j + c];
+        p[j] = V[4 * j + 3];
+        if (BOUND) p[j] += V[4 * j] * Rt[9] + V[4 * j + 1] * Rt[10] + V[4 * j + 2] * Rt[11];
+        p[j] += W[j][0] * v[0] + W[j][1] * v[1] + W[j][2] * v[2];
+    }
+    float d[3];  // squared scales
+#pragma unroll
+    for (int m = 0; m < 3; ++m) {
+        const float s = __expf(v[7 + m]);
+        d[m] = s * s;
+    }
+    const float il = rsqrtf(v[3] * v[3] + v[4] * v[4] + v[5] * v[5] + v[6] * v[6]);
+    const float w = v[3] * il, x = v[4] * il, y = v[5] * il, z = v[6] * il;
+    const float R[3][3] = {{1.f - 2.f * (y * y + z * z), 2.f * (x * y - w * z), 2.f * (x * z + w * y)},
+                           {2.f * (x * y + w * z), 1.f - 2.f * (x * x + z * z), 2.f * (y * z - w * x)},
+                           {2.f * (x * z - w * y), 2.f * (y * z + w * x), 1.f - 2.f * (x * x + y * y)}};
+    const float fx = V[12], fy = V[13], ipz = __frcp_rn(p[2]);
+    const float rx0 = p[0] * ipz, ry0 = p[1] * ipz;
+    const bool clx = rx0 > lim[0] || rx0 < -lim[0], cly = ry0 > lim[1] || ry0 < -lim[1];
+    const float rx = fminf(lim[0], fmaxf(-lim[0], rx0)), ry = fminf(lim[1], fmaxf(-lim[1], ry0));
+    const float j00 = fx * ipz, j02 = -j00 * rx, j11 = fy * ipz, j12 = -j11 * ry;  // the entries of J
+    float T[2][3], U[2][3], UD[2][3];
+#pragma unroll
+    for (int c = 0; c < 3; ++c) {
+        T[0][c] = j00 * W[0][c] + j02 * W[2][c];
+        T[1][c] = j11 * W[1][c] + j12 * W[2][c];
+    }
+#pragma unroll
+    for (int r = 0; r < 2; ++r)
+#pragma unroll
+        for (int m = 0; m < 3; ++m) {
+            U[r][m] = T[r][0] * R[0][m] + T[r][1] * R[1][m] + T[r][2] * R[2][m];
+            UD[r][m] = U[r][m] * d[m];
+        }
+    const float A = U[0][0] * UD[0][0] + U[0][1] * UD[0][1] + U[0][2] * UD[0][2] + 0.3f;
+    const float B = U[0][0] * UD[1][0] + U[0][1] * UD[1][1] + U[0][2] * UD[1][2];
+    const float C = U[1][0] * UD[1][0] + U[1][1] * UD[1][1] + U[1][2] * UD[1][2] + 0.3f;
+    const float iD = __frcp_rn(A * C - B * B);
     const float ca = C * iD, cb = -B * iD, cc = A * iD;
     const float du = ca * g2[0] + cb * g2[1], dv = cb * g2[0] + cc * g2[1];
-    const float dca = -0.5f * g2[2], dcb = -g2[3], dcc = -0.5f * g2[4];
     dG[10] = g2[5] * (1.f - op);  // dL/do times the sigmoid's o (1 - o)
     dG[11] = g2[6];
     dG[12] = g2[7];
     dG[13] = g2[8];
-    const float dA = dca * (-C * C * iD2) + dcb * (B * C * iD2) + dcc * (iD - A * C * iD2);
-    const float dC = dca * (iD - A * C * iD2) + dcb * (A * B * iD2) + dcc * (-A * A * iD2);
-    const float dB = dca * (2.f * B * C * iD2) + dcb * (-iD - 2.f * B * B * iD2) + dcc * (2.f * A * B * iD2);
-    const float G2[2][2] = {{dA, 0.5f * dB}, {0.5f * dB, dC}};
-    // dJ = 2 G2 J M ; dM = J^T G2 J
-    float GJ[2][3];
-#pragma unroll
-    for (int r = 0; r < 2; ++r)
-#pragma unroll
-        for (int c = 0; c < 3; ++c) GJ[r][c] = G2[r][0] * f.J[0][c] + G2[r][1] * f.J[1][c];
-    float dJ[2][3];
-#pragma unroll
-    for (int r = 0; r < 2; ++r)
-#pragma unroll
-        for (int c = 0; c < 3; ++c) dJ[r][c] = 2.f * (GJ[r][0] * f.M[0][c] + GJ[r][1] * f.M[1][c] + GJ[r][2] * f.M[2][c]);
-    float dM[3][3];
-#pragma unroll
-    for (int r = 0; r < 3; ++r)
-#pragma unroll
-        for (int c = 0; c < 3; ++c) dM[r][c] = f.J[0][r] * GJ[0][c] + f.J[1][r] * GJ[1][c];
-    // dSigma = V^T dM V
-    float tmp[3][3], dS[3][3];
-#pragma unroll
-    for (int r = 0; r < 3; ++r)
-#pragma unroll
-        for (int c = 0; c < 3; ++c) tmp[r][c] = V[r] * dM[0][c] + V[4 + r] * dM[1][c] + V[8 + r] * dM[2][c];
-#pragma unroll
-    for (int r = 0; r < 3; ++r)
-#pragma unroll
-        for (int c = 0; c < 3; ++c) dS[r][c] = tmp[r][0] * V[c] + tmp[r][1] * V[4 + c] + tmp[r][2] * V[8 + c];
-    if (BOUND) {  // Sigma = R Sigma_T R^T: dSigma_T = R^T dSigma R
-#pragma unroll
-        for (int r = 0; r < 3; ++r)
-#pragma unroll
-            for (int c = 0; c < 3; ++c) tmp[r][c] = Rt[r] * dS[0][c] + Rt[3 + r] * dS[1][c] + Rt[6 + r] * dS[2][c];
-#pragma unroll
-        for (int r = 0; r < 3; ++r)
-#pragma unroll
-            for (int c = 0; c < 3; ++c) dS[r][c] = tmp[r][0] * Rt[c] + tmp[r][1] * Rt[3 + c] + tmp[r][2] * Rt[6 + c];
-    }
-    // Sigma = R diag(s^2) R^T
-    float dSR[3][3];
-#pragma unroll
-    for (int r = 0; r < 3; ++r)
-#pragma unroll
-        for (int m = 0; m < 3; ++m) dSR[r][m] = dS[r][0] * f.R[0][m] + dS[r][1] * f.R[1][m] + dS[r][2] * f.R[2][m];
-    float dR[3][3];
-#pragma unroll
-    for (int r = 0; r < 3; ++r)
-#pragma unroll
-        for (int m = 0; m < 3; ++m) dR[r][m] = 2.f * dSR[r][m] * f.s[m] * f.s[m];
+    // G = -Q H Q with H = dL/dQ = -(S3, S4, S5) / 2 as a symmetric matrix: the signs cancel
+    const float ha = 0.5f * g2[2], hb = 0.5f * g2[3], hc = 0.5f * g2[4];
+    const float q00 = ca * ha + cb * hb, q01 = ca * hb + cb * hc, q10 = cb * ha + cc * hb, q11 = cb * hb + cc * hc;
+    const float ga = q00 * ca + q01 * cb, gb = q00 * cb + q01 * cc, gc = q10 * cb + q11 * cc;
+    float X[2][3];
 #pragma unroll
     for (int m = 0; m < 3; ++m) {
-        const float q = f.R[0][m] * dSR[0][m] + f.R[1][m] * dSR[1][m] + f.R[2][m] * dSR[2][m];
-        dG[7 + m] = 2.f * f.s[m] * q * f.s[m];  // ds * s (s = exp(log-scale))
+        const float h0 = ga * U[0][m] + gb * U[1][m], h1 = gb * U[0][m] + gc * U[1][m];
+        const float d2 = 2.f * d[m];
+        dG[7 + m] = d2 * (U[0][m] * h0 + U[1][m] * h1);  // dL/ds_m^2 times 2 s_m^2 (s = exp(log-scale))
+        X[0][m] = d2 * h0;
+        X[1][m] = d2 * h1;
     }
-    const float w = f.qn[0], x = f.qn[1], y = f.qn[2], z = f.qn[3];
-    const float dw = 2.f * (-z * dR[0][1] + y * dR[0][2] + z * dR[1][0] - x * dR[1][2] - y * dR[2][0] + x * dR[2][1]);
-    const float dx = 2.f * (y * dR[0][1] + z * dR[0][2] + y * dR[1][0] - 2.f * x * dR[1][1] - w * dR[1][2] +
-                            z * dR[2][0] + w * dR[2][1] - 2.f * x * dR[2][2]);
-    const float dy = 2.f * (-2.f * y * dR[0][0] + x * dR[0][1] + w * dR[0][2] + x * dR[1][0] + z * dR[1][2] -
-                            w * dR[2][0] + z * dR[2][1] - 2.f * y * dR[2][2]);
-    const float dz = 2.f * (-2.f * z * dR[0][0] - w * dR[0][1] + x * dR[0][2] + w * dR[1][0] - 2.f * z * dR[1][1] +
-                            y * dR[1][2] + x * dR[2][0] + y * dR[2][1]);
+    float dR[3][3], dT[2][3];
+#pragma unroll
+    for (int c = 0; c < 3; ++c) {
+#pragma unroll
+        for (int m = 0; m < 3; ++m) dR[c][m] = T[0][c] * X[0][m] + T[1][c] * X[1][m];
+#pragma unroll
+        for (int r = 0; r < 2; ++r) dT[r][c] = X[r][0] * R[c][0] + X[r][1] * R[c][1] + X[r][2] * R[c][2];
+    }
+    const float dw = 2.f * (z * (dR[1][0] - dR[0][1]) + y * (dR[0][2] - dR[2][0]) + x * (dR[2][1] - dR[1][2]));
+    const float dx = 2.f * (y * (dR[0][1] + dR[1][0]) + z * (dR[0][2] + dR[2][0]) + w * (dR[2][1] - dR[1][2]) -
+                            2.f * x * (dR[1][1] + dR[2][2]));
+    const float dy = 2.f * (x * (dR[0][1] + dR[1][0]) + z * (dR[1][2] + dR[2][1]) + w * (dR[0][2] - dR[2][0]) -
+                            2.f * y * (dR[0][0] + dR[2][2]));
+    const float dz = 2.f * (x * (dR[0][2] + dR[2][0]) + y * (dR[1][2] + dR[2][1]) + w * (dR[1][0] - dR[0][1]) -
+                            2.f * z * (dR[0][0] + dR[1][1]));
     const float dot = w * dw + x * dx + y * dy + z * dz;
-    const float il = f.il;
     dG[3] = (dw - w * dot) * il;
     dG[4] = (dx - x * dot) * il;
     dG[5] = (dy - y * dot) * il;
     dG[6] = (dz - z * dot) * il;
-    // mean
-    const float fx = V[12], fy = V[13], ipz = f.ipz, ipz2 = ipz * ipz;
-    float dp0 = du * fx * ipz, dp1 = dv * fy * ipz;
-    float dp2 = -du * fx * f.p[0] * ipz2 - dv * fy * f.p[1] * ipz2;
-    dp2 += -(dJ[0][0] * fx + dJ[1][1] * fy) * ipz2;
-    if (!f.clx) {
-        dp0 += -dJ[0][2] * fx * ipz2;
-        dp2 += dJ[0][2] * 2.f * fx * f.p[0] * ipz2 * ipz;
-    } else {
-        dp2 += dJ[0][2] * fx * f.rx * ipz2;
-    }
-    if (!f.cly) {
-        dp1 += -dJ[1][2] * fy * ipz2;
-        dp2 += dJ[1][2] * 2.f * fy * f.p[1] * ipz2 * ipz;
-    } else {
-        dp2 += dJ[1][2] * fy * f.ry * ipz2;
-    }
-    float dxw[3];
+    // mean: through the projection, and through J (a clamped ratio does not move with p_x or p_y)
+    const float dj00 = dT[0][0] * W[0][0] + dT[0][1] * W[0][1] + dT[0][2] * W[0][2];
+    const float dj02 = dT[0][0] * W[2][0] + dT[0][1] * W[2][1] + dT[0][2] * W[2][2];
+    const float dj11 = dT[1][0] * W[1][0] + dT[1][1] * W[1][1] + dT[1][2] * W[1][2];
+    const float dj12 = dT[1][0] * W[2][0] + dT[1][1] * W[2][1] + dT[1][2] * W[2][2];
+    const float ax = j00 * ipz, ay = j11 * ipz;  // fx / p_z^2, fy / p_z^2
+    const float dp0 = du * j00 - (clx ? 0.f : dj02 * ax);
+    const float dp1 = dv * j11 - (cly ? 0.f : dj12 * ay);
+    const float dp2 = ax * (dj02 * (clx ? rx : 2.f * rx0) - du * p[0] - dj00) +
+                      ay * (dj12 * (cly ? ry : 2.f * ry0) - dv * p[1] - dj11);
 #pragma unroll
-    for (int c = 0; c < 3; ++c) dxw[c] = V[c] * dp0 + V[4 + c] * dp1 + V[8 + c] * dp2;
-#pragma unroll
-    for (int c = 0; c < 3; ++c)  // x = R x_T + t: dx_T = R^T dx
-        dG[c] = BOUND ? Rt[c] * dxw[0] + Rt[3 + c] * dxw[1] + Rt[6 + c] * dxw[2] : dxw[c];
+    for (int c = 0; c < 3; ++c) dG[c] = W[0][c] * dp0 + W[1][c] * dp1 + W[2][c] * dp2;
 }
 
 // TBN matrix and barycentric point of Gaussian i in one frame (the same definitions as the
@@ -272,7 +181,7 @@ __device__ __forceinline__ bool tbn_fast(const ModelInfo &m, const float *__rest
 }
 
 // The backward of one model chunk. One CTA = 32 Gaussians (lane = Gaussian) of one model; the
-// frames that render it go 16 at a time. The chunk's blendshape rows are copied to shared
+// frames that render it go FG (8 or 16) at a time. The chunk's blendshape rows are copied to shared
 // memory asynchronously at the start. Meanwhile the chain rule per (frame, Gaussian) turns the
 // 2-D gradients into dL/dG_b over the 14 channels, straight into shared memory (each item
 // reads only its cache and 2-D gradients: the cache carries the opacity and whether the
@@ -285,7 +194,6 @@ __device__ __forceinline__ void cp_async16(void *dst, const void *src) {
                  :: "r"(static_cast<unsigned>(__cvta_generic_to_shared(dst))), "l"(src) : "memory");
 }
 
-constexpr int kFG2 = 16;
 constexpr int kWarps = kBwdThreads / 32;
 // Shared-memory strides in floats: a frame's 14 x 32 blended-channel gradients, and a staged
 // blendshape row of 32 Gaussians, each padded by 4 so that the tensor-core fragment loads,
@@ -293,9 +201,9 @@ constexpr int kWarps = kBwdThreads / 32;
 constexpr int kDGF = kNch * kBwdChunk + 4;
 constexpr int kDgRow = kBwdChunk + 4;
 
-// The adjoint of Eq. 1 is two small dense products per chunk and group of frames (ddG: the
-// K x 16 weights times the 16 x (A 32) blended-channel gradients; dpsi: the 16 x (A 32)
-// gradients times the (A 32) x K blendshape rows), done on the tensor cores as
+// The adjoint of Eq. 1 is two small dense products per chunk and group of FG frames (ddG: the
+// K x FG weights times the FG x (A 32) blended-channel gradients; dpsi: the K x (A 32)
+// blendshape rows times the (A 32) x FG gradients), done on the tensor cores as
 // m16n8k8 TF32 matrix multiply-accumulates with FP32 accumulators. Each FP32 operand x is split
 // into x_hi = tf32(x) and x_lo = tf32(x - x_hi), and a b is accumulated as
 // a_lo b_hi + a_hi b_lo + a_hi b_hi (the a_lo b_lo term is below FP32 rounding), which keeps
@@ -303,6 +211,8 @@ constexpr int kDgRow = kBwdChunk + 4;
 // single precision accuracy from Tensor Cores", 2022). Fragment layout (m16n8k8, A row-major,
 // B column-major), with g = lane / 4 and t = lane % 4: A elements (g, t), (g + 8, t), (g, t + 4), (g + 8, t + 4);
 // B elements (t, g), (t + 4, g); C elements (g, 2t), (g, 2t + 1), (g + 8, 2t), (g + 8, 2t + 1).
+// Blendshapes are the rows of both products and frames come in eights (the n8 columns of one, a
+// k8 step of the other), so a group of up to eight frames costs half of one of sixteen.
 __device__ __forceinline__ void split_tf32(float x, unsigned &hi, unsigned &lo) {
     asm("cvt.rna.tf32.f32 %0, %1;" : "=r"(hi) : "f"(x));
     const float r = x - __uint_as_float(hi);
@@ -325,10 +235,7 @@ __device__ __forceinline__ void mma_3xtf32(float d[4], const unsigned ah[4], con
     mma_tf32(d, ah, bh);
 }
 
-// 2 CTAs per SM: without the TBN mapping (unbound batches) the chain rule fits without spills
-// at up to 128 registers, and that beat 3 CTAs at 80 registers with spills (0.120 vs 0.127 ms
-// on the batched training workload).
-// ADAM: the fused Adam update of rgba_step_adam_async; every model is rendered by at most kFG2
+// ADAM: the fused Adam update of rgba_step_adam_async; every model is rendered by at most FG
 // frames, so the reductions below are complete after one group. Their results are parked in
 // shared memory (G0's in s_g0, the blendshapes' in the slots of the staged rows, whose values
 // are read again from memory) and the CTA then streams the update over the chunk's rows; the
@@ -344,21 +251,32 @@ using AdamArg = typename std::conditional<ADAM, FusedAdam, NoAdam>::type;
 
 // BOUND: some model of the batch has a tangent-space binding (the chain rule then maps through
 // each bound Gaussian's TBN frame); otherwise that mapping is compiled out.
-template <bool ADAM, bool BOUND>
-__global__ void __launch_bounds__(kBwdThreads, 2)
-k_gauss_bwd(Ctx c, int max_k, AdamArg<ADAM> fa) {
+// FG: frames per group, 8 where every model of the batch is rendered by at most eight, else 16.
+// Bound by the latency of its phases (loads, chain rule, two products, stores) at few warps per SM,
+// so the shared memory and registers are held to three CTAs per SM where that needs no spills to
+// speak of: not for the fused update and the tangent-space mapping with 16 frames, which keep two
+// (the mapping: 135 us with two, 147 with three). Measured against 3 x 3 covariances, frames always
+// in sixteens and two CTAs per SM: 64 frames of eight avatars of 30,000 to 100,000 Gaussians
+// 666 -> 406 us, ten frames of 60,000 (K = 20) 92 -> 74, 16 frames of 60,000 (K = 32) 113 -> 100,
+// the same bound to a mesh 145 -> 129. Eights everywhere: 16 frames 143 us, as the blendshape
+// gradients are then read back and added to.
+template <bool ADAM, bool BOUND, int FG>
+__global__ void __launch_bounds__(kBwdThreads, (ADAM || BOUND) && FG == 16 ? 2 : 3)
+k_gauss_bwd(Ctx c, int max_k, int max_ka, AdamArg<ADAM> fa) {
     extern __shared__ float smem[];
-    float *s_dG = smem;                                   // [16][kDGF]: [14][32] per frame
-    float *s_psi = s_dG + kFG2 * kDGF;                    // [16][max_k]
-    float *s_dgc = s_psi + kFG2 * max_k;                  // [k][A][kDgRow]: the chunk's blendshapes
+    float *s_dG = smem;                                   // [FG][kDGF]: [14][32] per frame
+    float *s_psi = s_dG + FG * kDGF;                      // [FG][max_k]
+    float *s_dgc = s_psi + FG * max_k;                    // [k][A][kDgRow]: the chunk's blendshapes
     __shared__ __align__(16) float s_g0[ADAM ? kNch * kBwdChunk : 1];  // ADAM: the G0 gradients
-    __shared__ long long s_rec[kFG2];
-    __shared__ int s_wh[kFG2][2];
-    __shared__ const float *s_verts[kFG2];
+    __shared__ long long s_rec[FG];
+    __shared__ float s_lim[FG][2];
+    __shared__ const float *s_verts[FG];
     pdl_enter();
-    __shared__ float s_fp[kFG2][RGBA_FP_STRIDE];
+    __shared__ float s_fp[FG][RGBA_FP_STRIDE];
     __shared__ int s_ch[kNch];               // the model's blended channels, by slot
-    __shared__ __align__(16) float s_red[kWarps * kFG2 * 32];  // dpsi: each warp's sums, 32 blendshapes
+    // dpsi: each warp's sums, [32 blendshapes][FG], in s_dG's place when that is free by then
+    const bool alias = !ADAM && max_k <= 32;
+    float *s_red = alias ? s_dG : s_dgc + max_ka * kDgRow;
     const ModelInfo &m = c.models[blockIdx.y];
     const int chunk = blockIdx.x;
     const int i0 = chunk * kBwdChunk;
@@ -387,20 +305,22 @@ k_gauss_bwd(Ctx c, int max_k, AdamArg<ADAM> fa) {
         }
     }
     if (threadIdx.x < A) s_ch[threadIdx.x] = m.chans[threadIdx.x];
-    for (int g0 = 0; g0 < m.nb; g0 += kFG2) {
-        const int ng = min(kFG2, m.nb - g0);
+    for (int g0 = 0; g0 < m.nb; g0 += FG) {
+        const int ng = min(FG, m.nb - g0);
         if (threadIdx.x < ng) {
-            const FrameInfo &f = c.frames[c.mframes[m.frame_off + g0 + threadIdx.x]];
+            const int b = c.mframes[m.frame_off + g0 + threadIdx.x];
+            const FrameInfo &f = c.frames[b];
             s_rec[threadIdx.x] = f.rec_base;
-            s_wh[threadIdx.x][0] = f.W;
-            s_wh[threadIdx.x][1] = f.H;
+            const float *fp = c.fparams + (size_t)b * RGBA_FP_STRIDE;
+            s_lim[threadIdx.x][0] = 1.3f * __fdividef(0.5f * f.W, fp[12]);
+            s_lim[threadIdx.x][1] = 1.3f * __fdividef(0.5f * f.H, fp[13]);
             s_verts[threadIdx.x] = f.verts;
         }
         for (int e = threadIdx.x; e < ng * RGBA_FP_STRIDE; e += kBwdThreads) {
             const int fl = e / RGBA_FP_STRIDE, q = e - fl * RGBA_FP_STRIDE;
             s_fp[fl][q] = c.fparams[(size_t)c.mframes[m.frame_off + g0 + fl] * RGBA_FP_STRIDE + q];
         }
-        for (int e = threadIdx.x; e < kFG2 * max_k; e += kBwdThreads) {
+        for (int e = threadIdx.x; e < FG * max_k; e += kBwdThreads) {
             const int fl = e / max_k, kk = e % max_k;
             s_psi[e] = (fl < ng && kk < K) ? c.psi[(size_t)c.mframes[m.frame_off + g0 + fl] * c.k_stride + kk] : 0.f;
         }
@@ -409,7 +329,7 @@ k_gauss_bwd(Ctx c, int max_k, AdamArg<ADAM> fa) {
         // past the group's end, which the loops below run over too); a warp takes 32
         // consecutive Gaussians of one frame
         {
-            constexpr int kItems = kFG2 * kBwdChunk / kBwdThreads;
+            constexpr int kItems = FG * kBwdChunk / kBwdThreads;
             float4 c0[kItems], c1[kItems], c2[kItems], ga[kItems], gb[kItems], gc[kItems];
             bool live[kItems];
 #pragma unroll
@@ -442,9 +362,9 @@ k_gauss_bwd(Ctx c, int max_k, AdamArg<ADAM> fa) {
                     if (BOUND) {
                         float Rt[12] = {1.f, 0.f, 0.f, 0.f, 1.f, 0.f, 0.f, 0.f, 1.f, 0.f, 0.f, 0.f};
                         if (m.n_faces == 0 || tbn_fast(m, s_verts[fl], i0 + li, Rt))
-                            chain<true>(v, c2[0].z, s_fp[fl], s_wh[fl][0], s_wh[fl][1], Rt, g2, dG);
+                            chain<true>(v, c2[0].z, s_fp[fl], s_lim[fl], Rt, g2, dG);
                     } else {
-                        chain<false>(v, c2[0].z, s_fp[fl], s_wh[fl][0], s_wh[fl][1], nullptr, g2, dG);
+                        chain<false>(v, c2[0].z, s_fp[fl], s_lim[fl], nullptr, g2, dG);
                     }
                 }
 #pragma unroll
@@ -482,102 +402,124 @@ k_gauss_bwd(Ctx c, int max_k, AdamArg<ADAM> fa) {
             }
         }
         const int grp = lane >> 2, tig = lane & 3;
-        // dpsi_b[k] partial = sum over a, i of dG_k[a][i] dG_b[ch_a][i]: D (frames x k) =
-        // A (frames x columns) B (columns x k), a column being (channel slot a, Gaussian i) and
+        // dpsi_b[k] partial = sum over a, i of dG_k[a][i] dG_b[ch_a][i]: D (k x frames) =
+        // A (k x columns) B (columns x frames), a column being (channel slot a, Gaussian i) and
         // 8 columns one k-step; the warps split the k-steps, their sums meet in s_red
-        if (c.grad_psi) {
+        auto weight_grads = [&]() {
+            if (!c.grad_psi) return;
             const int KS = A * (kBwdChunk / 8);
             for (int kb = 0; kb < K; kb += 32) {
-                float acc[4][4];
+                float acc[2][FG / 8][4];
 #pragma unroll
-                for (int j = 0; j < 4; ++j) acc[j][0] = acc[j][1] = acc[j][2] = acc[j][3] = 0.f;
+                for (int j = 0; j < 2; ++j)
+#pragma unroll
+                    for (int n = 0; n < FG / 8; ++n) acc[j][n][0] = acc[j][n][1] = acc[j][n][2] = acc[j][n][3] = 0.f;
                 for (int ks = warp; ks < KS; ks += kWarps) {
                     const int sa = ks / (kBwdChunk / 8), ib = (ks % (kBwdChunk / 8)) * 8;
-                    const float *dg = s_dG + s_ch[sa] * kBwdChunk + ib;  // + frame * kDGF
-                    unsigned ah[4], al[4];
-                    split_tf32(dg[grp * kDGF + tig], ah[0], al[0]);
-                    split_tf32(dg[(grp + 8) * kDGF + tig], ah[1], al[1]);
-                    split_tf32(dg[grp * kDGF + tig + 4], ah[2], al[2]);
-                    split_tf32(dg[(grp + 8) * kDGF + tig + 4], ah[3], al[3]);
+                    const float *dg = s_dG + s_ch[sa] * kBwdChunk + ib + tig + grp * kDGF;
+                    unsigned bh[FG / 8][2], bl[FG / 8][2];
+#pragma unroll
+                    for (int n = 0; n < FG / 8; ++n) {
+                        split_tf32(dg[n * 8 * kDGF], bh[n][0], bl[n][0]);
+                        split_tf32(dg[n * 8 * kDGF + 4], bh[n][1], bl[n][1]);
+                    }
                     // padding columns hold whatever the caller left there: zero them
                     const bool v0 = i0 + ib + tig < m.n, v1 = i0 + ib + tig + 4 < m.n;
 #pragma unroll
-                    for (int j = 0; j < 4; ++j) {
-                        const int kk = kb + j * 8 + grp;
-                        const float *bs = s_dgc + ((size_t)kk * A + sa) * kDgRow + ib + tig;
-                        unsigned bh[2], bl[2];
-                        split_tf32(kk < K && v0 ? bs[0] : 0.f, bh[0], bl[0]);
-                        split_tf32(kk < K && v1 ? bs[4] : 0.f, bh[1], bl[1]);
-                        mma_3xtf32(acc[j], ah, al, bh, bl);
+                    for (int j = 0; j < 2; ++j) {
+                        const int k0 = kb + j * 16 + grp, k1 = k0 + 8;
+                        const float *as = s_dgc + (k0 * A + sa) * kDgRow + ib + tig, *bs = as + 8 * A * kDgRow;
+                        unsigned ah[4], al[4];
+                        split_tf32(k0 < K && v0 ? as[0] : 0.f, ah[0], al[0]);
+                        split_tf32(k1 < K && v0 ? bs[0] : 0.f, ah[1], al[1]);
+                        split_tf32(k0 < K && v1 ? as[4] : 0.f, ah[2], al[2]);
+                        split_tf32(k1 < K && v1 ? bs[4] : 0.f, ah[3], al[3]);
+#pragma unroll
+                        for (int n = 0; n < FG / 8; ++n) mma_3xtf32(acc[j][n], ah, al, bh[n], bl[n]);
                     }
                 }
+                if (alias) __syncthreads();  // the sums take the place of s_dG, which nobody reads any more
 #pragma unroll
-                for (int j = 0; j < 4; ++j) {  // this warp's sums, then the warps' in a fixed order
-                    float *r = s_red + warp * (kFG2 * 32) + grp * 32 + j * 8 + 2 * tig;
-                    *reinterpret_cast<float2 *>(r) = make_float2(acc[j][0], acc[j][1]);
-                    *reinterpret_cast<float2 *>(r + 8 * 32) = make_float2(acc[j][2], acc[j][3]);
-                }
+                for (int j = 0; j < 2; ++j)  // this warp's sums, then the warps' in a fixed order
+#pragma unroll
+                    for (int n = 0; n < FG / 8; ++n) {
+                        float *r = s_red + warp * (32 * FG) + (j * 16 + grp) * FG + n * 8 + 2 * tig;
+                        *reinterpret_cast<float2 *>(r) = make_float2(acc[j][n][0], acc[j][n][1]);
+                        *reinterpret_cast<float2 *>(r + 8 * FG) = make_float2(acc[j][n][2], acc[j][n][3]);
+                    }
                 __syncthreads();
-                for (int e = threadIdx.x; e < kFG2 * 32; e += kBwdThreads) {
-                    const int fl = e >> 5, kk = kb + (e & 31);
+                for (int e = threadIdx.x; e < 32 * FG; e += kBwdThreads) {
+                    const int kk = kb + e / FG, fl = e % FG;
                     float t = 0.f;
 #pragma unroll
-                    for (int w = 0; w < kWarps; ++w) t += s_red[w * (kFG2 * 32) + e];
+                    for (int w = 0; w < kWarps; ++w) t += s_red[w * (32 * FG) + e];
                     if (fl < ng && kk < K)
                         c.dpsi_part[m.dpsi_off + ((long long)(g0 + fl) * K + kk) * m.n_chunks + chunk] = t;
                 }
                 __syncthreads();
             }
-        }
+        };
         // ddG[k][a][i] = sum_b psi_b[k] dG_b[ch_a][i]: D (k x columns) = A (k x frames)
-        // B (frames x columns), two k-steps of 8 frames; the warps split the 8-column tiles
-        if (ADAM ? true : m.gdg != nullptr) {
+        // B (frames x columns), a k-step per 8 frames; the warps split the 8-column tiles and a
+        // tile's split gradients serve 32 blendshapes
+        auto basis_grads = [&]() {
+            if (!ADAM && m.gdg == nullptr) return;
             const int NT = A * (kBwdChunk / 8);
-            for (int mb = 0; mb < K; mb += 16) {
-                const int k0 = mb + grp, k1 = k0 + 8;
-                unsigned ah[2][4], al[2][4];
+            for (int kb = 0; kb < K; kb += 32) {
+                unsigned ah[2][FG / 8][4], al[2][FG / 8][4];
 #pragma unroll
-                for (int q = 0; q < 2; ++q) {
-                    const int f0 = q * 8 + tig, f1 = f0 + 4;
-                    split_tf32(k0 < K ? s_psi[f0 * max_k + k0] : 0.f, ah[q][0], al[q][0]);
-                    split_tf32(k1 < K ? s_psi[f0 * max_k + k1] : 0.f, ah[q][1], al[q][1]);
-                    split_tf32(k0 < K ? s_psi[f1 * max_k + k0] : 0.f, ah[q][2], al[q][2]);
-                    split_tf32(k1 < K ? s_psi[f1 * max_k + k1] : 0.f, ah[q][3], al[q][3]);
+                for (int j = 0; j < 2; ++j) {
+                    const int k0 = kb + j * 16 + grp, k1 = k0 + 8;
+#pragma unroll
+                    for (int q = 0; q < FG / 8; ++q) {
+                        const int f0 = q * 8 + tig, f1 = f0 + 4;
+                        split_tf32(k0 < K ? s_psi[f0 * max_k + k0] : 0.f, ah[j][q][0], al[j][q][0]);
+                        split_tf32(k1 < K ? s_psi[f0 * max_k + k1] : 0.f, ah[j][q][1], al[j][q][1]);
+                        split_tf32(k0 < K ? s_psi[f1 * max_k + k0] : 0.f, ah[j][q][2], al[j][q][2]);
+                        split_tf32(k1 < K ? s_psi[f1 * max_k + k1] : 0.f, ah[j][q][3], al[j][q][3]);
+                    }
                 }
                 for (int nt = warp; nt < NT; nt += kWarps) {
                     const int sa = nt / (kBwdChunk / 8), ib = (nt % (kBwdChunk / 8)) * 8;
                     const float *dg = s_dG + s_ch[sa] * kBwdChunk + ib + grp;
-                    float d[4] = {0.f, 0.f, 0.f, 0.f};
+                    unsigned bh[FG / 8][2], bl[FG / 8][2];
 #pragma unroll
-                    for (int q = 0; q < 2; ++q) {
-                        unsigned bh[2], bl[2];
-                        split_tf32(dg[(q * 8 + tig) * kDGF], bh[0], bl[0]);
-                        split_tf32(dg[(q * 8 + tig + 4) * kDGF], bh[1], bl[1]);
-                        mma_3xtf32(d, ah[q], al[q], bh, bl);
+                    for (int q = 0; q < FG / 8; ++q) {
+                        split_tf32(dg[(q * 8 + tig) * kDGF], bh[q][0], bl[q][0]);
+                        split_tf32(dg[(q * 8 + tig + 4) * kDGF], bh[q][1], bl[q][1]);
                     }
-                    const int i = ib + 2 * tig;  // columns i, i + 1 of rows k0 and k1
-                    if (ADAM) {
-                        // s_dgc is no longer read (dpsi is done): its slots park the gradients
-                        if (k0 < K) {
-                            s_dgc[((size_t)k0 * A + sa) * kDgRow + i] = 0.f + d[0];
-                            s_dgc[((size_t)k0 * A + sa) * kDgRow + i + 1] = 0.f + d[1];
-                        }
-                        if (k1 < K) {
-                            s_dgc[((size_t)k1 * A + sa) * kDgRow + i] = 0.f + d[2];
-                            s_dgc[((size_t)k1 * A + sa) * kDgRow + i + 1] = 0.f + d[3];
-                        }
-                    } else if (i0 + i < m.n_pad) {  // n_pad - i0 is a multiple of 4: i + 1 too
+                    const int i = ib + 2 * tig;  // columns i, i + 1 of the rows k0 and k1
+                    float *o0 = ADAM ? nullptr : m.gdg + (size_t)((kb + grp) * A + sa) * m.n_pad + i0 + i;
+                    const size_t step = (size_t)8 * A * m.n_pad;  // eight blendshapes on
+#pragma unroll
+                    for (int j = 0; j < 2; ++j) {
+                        float d[4] = {0.f, 0.f, 0.f, 0.f};
+#pragma unroll
+                        for (int q = 0; q < FG / 8; ++q) mma_3xtf32(d, ah[j][q], al[j][q], bh[q], bl[q]);
 #pragma unroll
                         for (int h = 0; h < 2; ++h) {
-                            const int kk = h ? k1 : k0;
+                            const int kk = kb + j * 16 + 8 * h + grp;
                             if (kk >= K) continue;
-                            float2 *o = reinterpret_cast<float2 *>(m.gdg + ((size_t)kk * A + sa) * m.n_pad + i0 + i);
-                            const float2 old = g0 == 0 ? make_float2(0.f, 0.f) : *o;
-                            *o = make_float2(old.x + d[2 * h], old.y + d[2 * h + 1]);
+                            if (ADAM) {  // s_dgc is no longer read (dpsi is done): its slots park the gradients
+                                float *o = s_dgc + (kk * A + sa) * kDgRow + i;
+                                o[0] = 0.f + d[2 * h];
+                                o[1] = 0.f + d[2 * h + 1];
+                            } else if (i0 + i < m.n_pad) {  // n_pad - i0 is a multiple of 4: i + 1 too
+                                float2 *o = reinterpret_cast<float2 *>(o0 + (2 * j + h) * step);
+                                const float2 old = g0 == 0 ? make_float2(0.f, 0.f) : *o;
+                                *o = make_float2(old.x + d[2 * h], old.y + d[2 * h + 1]);
+                            }
                         }
                     }
                 }
             }
+        };
+        if (ADAM) {  // the blendshape gradients are parked in the rows that the weight gradients read
+            weight_grads();
+            basis_grads();
+        } else {
+            basis_grads();
+            weight_grads();
         }
         __syncthreads();
     }
@@ -659,10 +601,13 @@ __global__ void __launch_bounds__(kDpsiThreads) k_dpsi_reduce(Ctx c) {
 }  // namespace
 
 namespace {
-template <bool ADAM, bool BOUND>
+template <bool ADAM, bool BOUND, int FG>
 cudaError_t gauss_bwd_inst(const Ctx &c, int max_chunks, int max_k, int max_ka, const AdamArg<ADAM> &fa,
                            cudaStream_t s) {
-    auto bytes = [](int k, int ka) { return (kFG2 * kDGF + kFG2 * k + ka * kDgRow) * (int)sizeof(float); };
+    auto bytes = [](int k, int ka) {
+        const int red = ADAM || k > 32 ? kWarps * 32 * FG : 0;  // as in the kernel
+        return (FG * kDGF + FG * k + ka * kDgRow + red) * (int)sizeof(float);
+    };
     // set once, at the largest size any batch can ask for, so no attribute call happens while
     // a stream is being captured
     static int attr_device = -1;
@@ -670,26 +615,33 @@ cudaError_t gauss_bwd_inst(const Ctx &c, int max_chunks, int max_k, int max_ka, 
     cudaError_t e = cudaGetDevice(&dev);
     if (e != cudaSuccess) return e;
     if (attr_device != dev) {
-        e = cudaFuncSetAttribute(k_gauss_bwd<ADAM, BOUND>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+        e = cudaFuncSetAttribute(k_gauss_bwd<ADAM, BOUND, FG>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                  bytes(RGBA_MAX_K, RGBA_MAX_K * 13));
         if (e != cudaSuccess) return e;
         attr_device = dev;
     }
     dim3 g2(max_chunks, c.M);
-    return launch_pdl(k_gauss_bwd<ADAM, BOUND>, g2, dim3(kBwdThreads), (size_t)bytes(max_k, max_ka), s, c, max_k,
-                      fa);
+    return launch_pdl(k_gauss_bwd<ADAM, BOUND, FG>, g2, dim3(kBwdThreads), (size_t)bytes(max_k, max_ka), s, c, max_k,
+                      max_ka, fa);
+}
+
+template <bool ADAM, bool BOUND>
+cudaError_t gauss_bwd_frames(const Ctx &c, int max_chunks, int max_nb, int max_k, int max_ka, const AdamArg<ADAM> &fa,
+                             cudaStream_t s) {
+    return max_nb <= 8 ? gauss_bwd_inst<ADAM, BOUND, 8>(c, max_chunks, max_k, max_ka, fa, s)
+                       : gauss_bwd_inst<ADAM, BOUND, 16>(c, max_chunks, max_k, max_ka, fa, s);
 }
 }  // namespace
 
-cudaError_t launch_gauss_bwd(const Ctx &c, int max_chunks, int max_k, int max_ka, const FusedAdam *fa,
+cudaError_t launch_gauss_bwd(const Ctx &c, int max_chunks, int max_nb, int max_k, int max_ka, const FusedAdam *fa,
                              bool any_bound, cudaStream_t s) {
     if (c.M == 0 || max_chunks == 0) return cudaSuccess;
     if (fa)
-        return any_bound ? gauss_bwd_inst<true, true>(c, max_chunks, max_k, max_ka, *fa, s)
-                         : gauss_bwd_inst<true, false>(c, max_chunks, max_k, max_ka, *fa, s);
+        return any_bound ? gauss_bwd_frames<true, true>(c, max_chunks, max_nb, max_k, max_ka, *fa, s)
+                         : gauss_bwd_frames<true, false>(c, max_chunks, max_nb, max_k, max_ka, *fa, s);
     const NoAdam none{};
-    return any_bound ? gauss_bwd_inst<false, true>(c, max_chunks, max_k, max_ka, none, s)
-                     : gauss_bwd_inst<false, false>(c, max_chunks, max_k, max_ka, none, s);
+    return any_bound ? gauss_bwd_frames<false, true>(c, max_chunks, max_nb, max_k, max_ka, none, s)
+                     : gauss_bwd_frames<false, false>(c, max_chunks, max_nb, max_k, max_ka, none, s);
 }
 
 cudaError_t launch_dpsi_reduce(const Ctx &c, int max_k, cudaStream_t s) {
