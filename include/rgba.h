@@ -329,8 +329,8 @@ int rgba_profile_read(rgba_ctx_t ctx, rgba_profile *out);
 typedef struct {
     int64_t fwd_staged;  /* list entries whose masks the forward's pixel-block warps scanned */
     int64_t fwd_hits;    /* (list entry, 8x4 pixel block) pairs whose mask has the block */
-    int64_t fwd_visits;  /* hits at which some pixel of the block passes the cutoffs (the entry
-                            is then composited at the block) */
+    int64_t fwd_visits;  /* hits at which some pixel of the block blends the entry (bwd: takes a
+                            gradient of it) */
     int64_t fwd_blends;  /* (pixel, entry) pairs the forward blended */
     int64_t bwd_staged;  /* the same counts for the backward's reverse walk */
     int64_t bwd_hits;

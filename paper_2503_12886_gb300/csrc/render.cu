@@ -5,13 +5,17 @@
 // many warps and no warp ever waits at a CTA barrier. A block is 8 x 4 pixels, one per lane.
 //
 // Every list entry comes with a byte that says which of the tile's eight blocks its splat can
-// reach (made once per (Gaussian, tile) by the scatter). A warp scans its tile's list 64 entries
-// at a time, keeps those whose bit for its block is set in a queue of its own, and stages 32 S of
-// the queued entries at a time: each lane loads the records of S of them (one step ahead of the
-// compositing) and writes them, in the form the pixel loop reads, to the warp's shared-memory
-// slots. The warp then visits the slots in list order (in reverse in the backward): it evaluates
-// the power at every pixel, skips the entry when no lane passes the cutoff, and otherwise runs
-// the pixel step without branches (lanes that do not take part keep their state). The forward
+// reach (made once per (Gaussian, tile) by the scatter). A warp scans its tile's list 128 entries
+// at a time, four mask bytes per lane, and queues the positions whose bit for its block is set. It
+// stages 32 S of the queued entries at a time: each lane loads the records of S of them (one step
+// ahead of the compositing, the Gaussian indices two), tests which half of the block (4 x 4 pixels) the splat
+// reaches and writes the entry, in the form the pixel loop reads, to the shared-memory slots of those
+// halves. The two halves of the warp then walk their own slots side by side, in list order (in
+// reverse in the backward): on 16 frames of 512 x 512 (N = 60,000) a quarter of the splats that meet a
+// block miss one of its halves, which leaves 9 % fewer steps after the fuller half of each stage. The
+// pixel step has no branches (lanes that do not take part keep their state; skipping an entry that no
+// pixel takes saved less than the vote and the broken-up schedule cost), so that several entries' steps
+// overlap, and the power is evaluated for two entries at a time in packed FP32. The forward
 // stops once every pixel of the block is saturated.
 //
 // Per pixel, with d = pixel centre - mean:
@@ -23,6 +27,7 @@
 // (1 - alpha). Per-Gaussian gradient sums are formed 16 entries at a time with the warp turned
 // round: lanes hold entries instead of pixels and add up their rows of a shared-memory matrix
 // that the visits filled; the sums reach global memory as atomic reductions.
+#include "reach.cuh"
 #include "rgba_internal.cuh"
 
 namespace rgba {
@@ -40,17 +45,29 @@ __device__ __forceinline__ int find_frame(const Ctx &c, long long t) {
     return lo;
 }
 
-// power = -(a dx^2 + c dy^2)/2 - b dx dy = dx ((-a/2) dx + (-b) dy) + (-c/2) dy dy, from a staged
-// entry's (u, v, -a/2, -b) and -c/2. Both kernels evaluate through this function and cut with
-// skip(), so their decisions agree bit for bit.
-__device__ __forceinline__ float power_of(float dx, float dy, const float4 &A, float hc) {
-    return __fmaf_rn(dx, __fmaf_rn(A.z, dx, __fmul_rn(A.w, dy)), __fmul_rn(__fmul_rn(hc, dy), dy));
+// power = -(a dx^2 + c dy^2)/2 - b dx dy = dx ((-a/2) dx + (-b) dy) + (-c/2) dy dy for a pair of staged
+// entries: A = (-u, -v), B = (-a/2, -b), hc = -c/2, one entry in each component. Both kernels evaluate
+// through this function and cut with skip(), so their decisions agree bit for bit.
+__device__ __forceinline__ float2 power_of(float pxc, float pyc, const float4 &A, const float4 &B, float2 hc) {
+    const float2 dx = __fadd2_rn(make_float2(pxc, pxc), make_float2(A.x, A.y));
+    const float2 dy = __fadd2_rn(make_float2(pyc, pyc), make_float2(A.z, A.w));
+    const float2 t = __ffma2_rn(make_float2(B.x, B.y), dx, __fmul2_rn(make_float2(B.z, B.w), dy));
+    return __ffma2_rn(dx, t, __fmul2_rn(__fmul2_rn(hc, dy), dy));
 }
 
 // the skip decision: a positive power (never, for a positive definite conic, but kept as the
 // definition) or alpha below 1/255 (alpha_cut): most pairs, the far tail of a splat, are rejected
 // before the exponential and before the colour is read
 __device__ __forceinline__ bool skip(float power, float tau) { return power > 0.0f || power < tau; }
+
+// e^x for the compositing, as 2^(x log2 e) on the hardware's base-2 exponential in its
+// flush-to-zero form: the general form guards against subnormal results with three more
+// instructions, and no weight that counts (alpha >= 1/255) is near that range.
+__device__ __forceinline__ float exp_ftz(float x) {
+    float y;
+    asm("ex2.approx.ftz.f32 %0, %1;" : "=f"(y) : "f"(__fmul_rn(x, 1.44269504088896341f)));
+    return y;
+}
 
 struct PixF {
     float pxc, pyc, T, C0, C1, C2;
@@ -66,7 +83,7 @@ struct PixF {
 // weight is 0). Returns the splatting weight alpha T at the pixel (0 when the entry does not
 // blend).
 __device__ __forceinline__ float composite(PixF &p, bool live, float power, const float4 &Cc, int pos) {
-    const float alpha = fminf(kAlphaMax, __fmul_rn(Cc.x, __expf(power)));
+    const float alpha = fminf(kAlphaMax, __fmul_rn(Cc.x, exp_ftz(power)));
     const float testT = p.T * (1.0f - alpha);
     const bool sat = testT < kTMin;
     p.done = p.done || (live && sat);
@@ -82,118 +99,200 @@ __device__ __forceinline__ float composite(PixF &p, bool live, float power, cons
 
 constexpr int kWarpsPerCta = 4;  // independent warps per CTA (they share nothing but the loss sum)
 
-// A warp's shared memory: the queue of entries that reach its block, and the staged slots
-// (32 S of them, and one past the end for the loop's look-ahead).
-//   a = (u, v, -a/2, -b)   q = (-c/2, tau, list position + 1, Gaussian index)   c = (opacity, r, g, b)
+// Two staged entries, slots 2 p and 2 p + 1, as the pixel loop reads them:
+//   A = (-u, -u', -v, -v')  B = (-a/2, -a'/2, -b, -b')  H = (-c/2, -c'/2, tau, tau')
+//   c = (opacity, r, g, b)  pos = list position + 1   idx = Gaussian index
+struct __align__(16) Pair {
+    float4 A, B, H, c[2];
+    int pos[2];
+    unsigned idx[2];
+};
+
+// A warp's shared memory: the queue of list positions that reach its block, and for each half of
+// the block its staged slots, up to 32 S (and a pair past the end for the loop's look-ahead). The
+// halves lie 64 bytes apart modulo the banks' 128, so that both halves' reads are one pass.
 template <int S>
 struct WarpMem {
-    static constexpr int kQueue = S > 2 ? 256 : 128;  // holds a stage's worth and one scan
-    float4 a[32 * S + 1], q[32 * S + 1], c[32 * S];
-    uint2 queue[kQueue];  // (list position + 1, Gaussian index)
+    static constexpr int kQueue = 256;  // holds a stage's worth and one scan
+    static_assert(32 * S - 1 + 128 <= kQueue, "queue");
+    static constexpr int kHalf = 16 * S * (int)sizeof(Pair) + 64;
+    __align__(16) unsigned char slots[kHalf + (16 * S + 1) * sizeof(Pair)];
+    unsigned queue[kQueue];
+    __device__ __forceinline__ Pair *half(int h) { return reinterpret_cast<Pair *>(slots + h * kHalf); }
+    __device__ __forceinline__ const Pair *half(int h) const { return reinterpret_cast<const Pair *>(slots + h * kHalf); }
 };
 
 // One compositing warp's view of a (tile, pixel block) item: the tile's list and the block.
 struct Walk {
     const unsigned *list;        // the tile's sorted Gaussian indices
-    const unsigned char *masks;  // and their block masks
+    const unsigned char *masks;  // and their block masks (8-byte aligned)
     int len;
     unsigned blk;
     const float4 *rec;  // the frame's render records
     float bx0, by0;     // the block's first pixel centre
+    bool masked;        // the lists carry masks
 };
 
-// The entries of list positions [lo, hi) that reach the block, front to back (DIR = 1) or back to
-// front (DIR = -1). scan() appends the hits among the next 64 entries to the queue; the 64 after
-// them are in flight meanwhile.
+// The entries of list positions [0, hi) that reach the block, front to back (DIR = 1) or back to
+// front (DIR = -1). A chunk is 128 list positions, four neighbouring ones per lane (their mask bytes
+// are one word); fill() appends a chunk's hits to the queue in walking order, with the words of the two
+// chunks after it in flight.
 template <int S, int DIR>
 struct Feed {
-    int lo, hi, at;       // entries not scanned yet: [at, hi) or [lo, at)
+    int hi, next, left;   // entries; the next chunk to load; chunks not scanned yet
     unsigned head, count; // the queue's first element and length
-    unsigned idx[2];      // the loaded entries: lane + 32 i past `at`
-    bool hit[2];
+    unsigned w0, w1;      // this lane's mask bytes of the next two chunks, as loaded: a warp waits for a
+                          // load at the first instruction that reads it, so nothing does before the scan
 
-    __device__ __forceinline__ void load(const Walk &w) {
+    // this lane's first list position of chunk k
+    static __device__ __forceinline__ int first(int k) {
         const int lane = threadIdx.x & 31;
-#pragma unroll
-        for (int i = 0; i < 2; ++i) {
-            const int e = DIR > 0 ? at + lane + 32 * i : at - 1 - lane - 32 * i;
-            const bool in = DIR > 0 ? e < hi : e >= lo;
-            hit[i] = in && ((w.masks[in ? e : lo] >> w.blk) & 1u);
-            idx[i] = in ? w.list[e] : 0u;
-        }
+        return k * 128 + 4 * (DIR > 0 ? lane : 31 - lane);
     }
-    __device__ __forceinline__ void start(const Walk &w, int lo_, int hi_) {
-        lo = lo_;
+    __device__ __forceinline__ unsigned load(const Walk &w) {
+        const int e = first(next);
+        next += DIR;
+        unsigned m = 0u;  // bytes past the list's end lie in its own key segment
+        if (e >= 0 && e < hi) m = *reinterpret_cast<const unsigned *>(w.masks + e);
+        return m;
+    }
+    __device__ __forceinline__ void start(const Walk &w, int hi_) {
         hi = hi_;
-        at = DIR > 0 ? lo : hi;
+        left = (hi + 127) / 128;
+        next = DIR > 0 ? 0 : left - 1;
         head = count = 0u;
-        load(w);
+        w0 = load(w);
+        w1 = load(w);
     }
-    __device__ __forceinline__ bool more() const { return DIR > 0 ? at < hi : at > lo; }
     // until the queue holds a stage's worth (or the list is done); returns the entries scanned
     __device__ __forceinline__ int fill(const Walk &w, WarpMem<S> &m) {
         constexpr unsigned Q = WarpMem<S>::kQueue - 1;
         const int lane = threadIdx.x & 31;
+        const unsigned lt = (1u << lane) - 1u;
         int scanned = 0;
-        while (count < 32u * S && more()) {
-            const unsigned b0 = __ballot_sync(0xffffffffu, hit[0]), b1 = __ballot_sync(0xffffffffu, hit[1]);
-            const unsigned lt = (1u << lane) - 1u, n0 = __popc(b0), tail = head + count;
-            const unsigned pos = DIR > 0 ? at + lane + 1 : at - lane;  // list position + 1
-            if (hit[0]) m.queue[(tail + __popc(b0 & lt)) & Q] = make_uint2(pos, idx[0]);
-            if (hit[1]) m.queue[(tail + n0 + __popc(b1 & lt)) & Q] = make_uint2(pos + DIR * 32, idx[1]);
-            count += n0 + __popc(b1);
-            scanned += DIR > 0 ? min(64, hi - at) : min(64, at - lo);
-            at += DIR * 64;
-            load(w);
+        while (count < 32u * S && left > 0) {
+            const int e = first(next - 2 * DIR);
+            unsigned hits = (w0 >> w.blk) & 0x01010101u;  // bit 8 i: byte i
+            if (hi - e < 4) hits = hi > e ? hits & ((1u << (8 * (hi - e))) - 1u) : 0u;
+            const unsigned n = __popc(hits);
+            const unsigned b0 = __ballot_sync(0xffffffffu, n & 1u), b1 = __ballot_sync(0xffffffffu, n & 2u),
+                           b2 = __ballot_sync(0xffffffffu, n & 4u);
+            unsigned at = head + count + __popc(b0 & lt) + 2u * __popc(b1 & lt) + 4u * __popc(b2 & lt);
+#pragma unroll
+            for (int i = 0; i < 4; ++i) {
+                const int k = DIR > 0 ? i : 3 - i;
+                if ((hits >> (8 * k)) & 1u) m.queue[at++ & Q] = (unsigned)(e + k + 1);
+            }
+            count += __popc(b0) + 2u * __popc(b1) + 4u * __popc(b2);
+            --left;
+            scanned += min(128, hi - (next - 2 * DIR) * 128);
+            w0 = w1;
+            w1 = load(w);
         }
         __syncwarp();
         return scanned;
     }
 };
 
-// The records of the next 32 S queued entries, on their way to the slots: lane l takes entries
-// l, l + 32, ...
+// Up to 32 S queued entries on their way to the slots: lane l takes entries l, l + 32, ... First
+// their list positions and Gaussian indices, a step later their records.
+template <int S>
+struct Ids {
+    unsigned pos[S], idx[S];
+    int n;  // entries
+};
 template <int S>
 struct Stage {
-    uint2 e[S];
+    Ids<S> id;
     float4 r0[S], r1[S];
     float r2[S];
-    int n;  // entries
 };
 
 template <int S, int DIR>
-__device__ __forceinline__ void load_stage(const Walk &w, const WarpMem<S> &m, Feed<S, DIR> &f, Stage<S> &g) {
+__device__ __forceinline__ void load_ids(const Walk &w, const WarpMem<S> &m, Feed<S, DIR> &f, Ids<S> &d) {
     const int lane = threadIdx.x & 31;
-    g.n = min((int)f.count, 32 * S);
+    d.n = min((int)f.count, 32 * S);
 #pragma unroll
     for (int s = 0; s < S; ++s) {
-        if (lane + 32 * s < g.n) {
-            g.e[s] = m.queue[(f.head + lane + 32 * s) & (WarpMem<S>::kQueue - 1)];
-            const float4 *r = w.rec + (size_t)g.e[s].y * 3;
+        if (lane + 32 * s < d.n) {
+            d.pos[s] = m.queue[(f.head + lane + 32 * s) & (WarpMem<S>::kQueue - 1)];
+            d.idx[s] = w.list[d.pos[s] - 1u];
+        }
+    }
+    f.head += d.n;
+    f.count -= d.n;
+}
+
+template <int S>
+__device__ __forceinline__ void load_stage(const Walk &w, const Ids<S> &d, Stage<S> &g) {
+    const int lane = threadIdx.x & 31;
+    g.id = d;
+#pragma unroll
+    for (int s = 0; s < S; ++s) {
+        if (lane + 32 * s < d.n) {
+            const float4 *r = w.rec + (size_t)d.idx[s] * 3;
             g.r0[s] = r[0];
             g.r1[s] = r[1];
             g.r2[s] = r[2].x;
         }
     }
-    f.head += g.n;
-    f.count -= g.n;
 }
 
+// Writes one entry to slot k of half h.
 template <int S>
-__device__ __forceinline__ void commit(const Stage<S> &g, WarpMem<S> &m) {
+__device__ __forceinline__ void put_slot(WarpMem<S> &m, int h, int k, const float4 &r0, const float4 &r1, float r2, float tau,
+                                         unsigned pos, unsigned idx) {
+    Pair &s = m.half(h)[k >> 1];
+    const int i = k & 1;
+    float *A = reinterpret_cast<float *>(&s.A) + i, *B = reinterpret_cast<float *>(&s.B) + i, *H = reinterpret_cast<float *>(&s.H) + i;
+    A[0] = -r0.x;
+    A[2] = -r0.y;
+    B[0] = -0.5f * r0.z;
+    B[2] = -r0.w;
+    H[0] = -0.5f * r1.x;
+    H[2] = tau;
+    s.c[i] = make_float4(r1.y, r1.z, r1.w, r2);
+    s.pos[i] = (int)pos;
+    s.idx[i] = idx;
+}
+
+// The staged entries into the slots of the halves they reach, in order; n[h] of half h. A half with
+// fewer is filled up, to an even number, with entries that no pixel takes. Returns the slots to walk;
+// reach[h]: the lanes whose (last) entry reaches half h.
+template <int S>
+__device__ __forceinline__ int commit(const Walk &w, const Stage<S> &g, WarpMem<S> &m, int n[2], unsigned reach[2]) {
     const int lane = threadIdx.x & 31;
+    const unsigned lt = (1u << lane) - 1u;
     __syncwarp();  // the previous stage's slots are no longer read
+    n[0] = n[1] = 0;
 #pragma unroll
     for (int s = 0; s < S; ++s) {
-        const int k = lane + 32 * s;
-        if (k < g.n) {
-            m.a[k] = make_float4(g.r0[s].x, g.r0[s].y, -0.5f * g.r0[s].z, -g.r0[s].w);
-            m.q[k] = make_float4(-0.5f * g.r1[s].x, alpha_cut(g.r1[s].y), __uint_as_float(g.e[s].x),
-                                 __uint_as_float(g.e[s].y));
-            m.c[k] = make_float4(g.r1[s].y, g.r1[s].z, g.r1[s].w, g.r2[s]);
+        bool left = false, right = false;
+        float tau = 0.f;
+        if (lane + 32 * s < g.id.n) {
+            const Reach e = reach_of(g.r0[s], make_float2(g.r1[s].x, g.r1[s].y));
+            float xl, xr;
+            reach_rows(e, w.by0, xl, xr);
+            tau = alpha_cut(g.r1[s].y);
+            const bool all = e.all || !w.masked, hit = xr >= w.bx0 && xl <= w.bx0 + 7.0f && !e.none;
+            left = all || (hit && xl <= w.bx0 + 3.0f);
+            right = all || (hit && xr >= w.bx0 + 4.0f);
         }
+        const unsigned bl = __ballot_sync(0xffffffffu, left), br = __ballot_sync(0xffffffffu, right);
+        if (left) put_slot(m, 0, n[0] + __popc(bl & lt), g.r0[s], g.r1[s], g.r2[s], tau, g.id.pos[s], g.id.idx[s]);
+        if (right) put_slot(m, 1, n[1] + __popc(br & lt), g.r0[s], g.r1[s], g.r2[s], tau, g.id.pos[s], g.id.idx[s]);
+        n[0] += __popc(bl);
+        n[1] += __popc(br);
+        reach[0] = bl;
+        reach[1] = br;
     }
+    const int top = (max(n[0], n[1]) + 1) & ~1;
+    const float4 z = make_float4(0.f, 0.f, 0.f, 0.f);
+#pragma unroll
+    for (int h = 0; h < 2; ++h)
+        for (int k = n[h] + lane; k < top; k += 32) put_slot(m, h, k, z, z, 0.f, __int_as_float(0x7f800000), 0u, 0u);
     __syncwarp();
+    return top;
 }
 
 // A fire-and-forget global float add.
@@ -206,42 +305,29 @@ __device__ __forceinline__ void red_add4(float *addr, float a, float b, float c,
     asm volatile("red.global.add.v4.f32 [%0], {%1, %2, %3, %4};" :: "l"(addr), "f"(a), "f"(b), "f"(c), "f"(d) : "memory");
 }
 
-// Sums over pixels for 16 slots at a time. The visit of slot j leaves one or two numbers per pixel
+// Sums over pixels for 16 slots at a time. The step of slot j leaves one or two numbers per pixel
 // (lane) in row j % 16 of a shared-memory matrix; after 16 slots the warp turns round: lane l takes
-// the entry of row l % 16 and the pixel rows 2 (l / 16) and 2 (l / 16) + 1 of the block, and adds up
-// its 16 pixels from 16-byte loads, two columns per packed FP32 instruction. Per visit that costs
+// slot l % 16 of half l / 16 and adds up that half's 16 pixels (the columns 16 (l / 16) ...) from 16-byte
+// loads, one pixel row at a time, two pixels per packed FP32 instruction. Per slot that costs
 // the stores and a sixteenth of about 150 instructions, where a shuffle reduction of nine sums
-// over the lanes takes about 45 and puts ten dependent shuffles into every visit. The rows are
+// over the lanes takes about 45 and puts ten dependent shuffles into every step. The rows are
 // padded to 36 floats so that the 16-byte loads of eight lanes fall in different banks.
 constexpr int kRows = 16;
 constexpr int kRowStride = 36;
 
-// The 16 pixel values of this lane's row and pixel rows, as pairs of neighbouring columns.
-__device__ __forceinline__ void row_pairs(const float *rows, int q, float2 v[4]) {
+// The four values of pixel row q of this lane's slot and half, as pairs of neighbouring columns.
+__device__ __forceinline__ void row_pairs(const float *rows, int q, float2 v[2]) {
     const int lane = threadIdx.x & 31;
-    const float4 *p = reinterpret_cast<const float4 *>(rows + (lane & 15) * kRowStride + 8 * (2 * (lane >> 4) + q));
-    const float4 a = p[0], b = p[1];
+    const float4 a = *reinterpret_cast<const float4 *>(rows + (lane & 15) * kRowStride + (lane & 16) + 4 * q);
     v[0] = make_float2(a.x, a.y);
     v[1] = make_float2(a.z, a.w);
-    v[2] = make_float2(b.x, b.y);
-    v[3] = make_float2(b.z, b.w);
 }
 
-// c += sum over the pairs of w times the block's per-pixel values `pix` (pixel row 2 (lane / 16) + q)
-__device__ __forceinline__ void add_dot(float2 &c, const float2 w[4], const float *pix, int q) {
-    const float4 *p = reinterpret_cast<const float4 *>(pix + 8 * (2 * ((threadIdx.x & 31) >> 4) + q));
-    const float4 a = p[0], b = p[1];
+// c += sum over the pairs of w times the pixels' values `pix` [32] (pixel row q of this lane's half)
+__device__ __forceinline__ void add_dot(float2 &c, const float2 w[2], const float *pix, int q) {
+    const float4 a = *reinterpret_cast<const float4 *>(pix + (threadIdx.x & 16) + 4 * q);
     c = __ffma2_rn(w[0], make_float2(a.x, a.y), c);
     c = __ffma2_rn(w[1], make_float2(a.z, a.w), c);
-    c = __ffma2_rn(w[2], make_float2(b.x, b.y), c);
-    c = __ffma2_rn(w[3], make_float2(b.z, b.w), c);
-}
-
-// Adds over both halves of the warp: lanes l and l + 16 hold the two halves of a block's pixels.
-template <int N>
-__device__ __forceinline__ void add_halves(float t[N]) {
-#pragma unroll
-    for (int i = 0; i < N; ++i) t[i] += __shfl_xor_sync(0xffffffffu, t[i], 16);
 }
 
 // Writes one finished pixel (colour over the background, T, contributor count) and, with a
@@ -286,9 +372,10 @@ __device__ __forceinline__ void finish_pixel(const Ctx &c, const FrameInfo &f, i
     }
 }
 
-// An empty tile's item: the background, T = 1, no contributors, eight pixels per lane.
+// An empty tile's item: the background, T = 1, no contributors, eight pixels per lane; four
+// neighbouring ones at a time where the frame's rows and the arrays allow 16-byte accesses (vec).
 template <int TW>
-__device__ __forceinline__ void empty_tile(const Ctx &c, long long t, float *img, float *T_final, int *n_contrib,
+__device__ __forceinline__ void empty_tile(const Ctx &c, long long t, bool vec, float *img, float *T_final, int *n_contrib,
                                            const float *target, int loss_kind, float *dl_dimg, float &loss_acc) {
     constexpr int TH = kTilePix / TW;
     const int lane = threadIdx.x & 31;
@@ -296,6 +383,38 @@ __device__ __forceinline__ void empty_tile(const Ctx &c, long long t, float *img
     const FrameInfo &f = c.frames[b];
     const int lt = (int)(t - f.tile_base);
     const int ty = lt / f.tiles_x, tx = lt - ty * f.tiles_x;
+    if (vec && ((f.W | f.pix_base) & 3) == 0) {
+        const float *bg = c.fparams + (size_t)b * RGBA_FP_STRIDE + 17;
+        const long long hw = (long long)f.W * f.H;
+        const float scale = 1.0f / (3.0f * (float)hw * (float)c.loss_frames);
+#pragma unroll
+        for (int k = 0; k < kTilePix / 128; ++k) {
+            const int p4 = 4 * lane + 128 * k, px = tx * TW + (p4 % TW), py = ty * TH + (p4 / TW);
+            if (px >= f.W || py >= f.H) continue;
+            const long long pix = (long long)py * f.W + px;
+#pragma unroll
+            for (int ch = 0; ch < 3; ++ch) {
+                const long long at = f.pix_base * 3 + ch * hw + pix;
+                const float o = fmaf(1.f, bg[ch], 0.f);
+                *reinterpret_cast<float4 *>(img + at) = make_float4(o, o, o, o);
+                if (target) {
+                    const float4 tg = *reinterpret_cast<const float4 *>(target + at);
+                    float g[4];
+                    const float dd[4] = {o - tg.x, o - tg.y, o - tg.z, o - tg.w};
+#pragma unroll
+                    for (int q = 0; q < 4; ++q) {
+                        const bool l1 = loss_kind == RGBA_LOSS_L1;
+                        loss_acc += (l1 ? fabsf(dd[q]) : 0.5f * (dd[q] * dd[q])) * scale;
+                        g[q] = l1 ? (dd[q] > 0.f ? scale : (dd[q] < 0.f ? -scale : 0.f)) : dd[q] * scale;
+                    }
+                    if (dl_dimg) *reinterpret_cast<float4 *>(dl_dimg + at) = make_float4(g[0], g[1], g[2], g[3]);
+                }
+            }
+            *reinterpret_cast<float4 *>(T_final + f.pix_base + pix) = make_float4(1.f, 1.f, 1.f, 1.f);
+            *reinterpret_cast<int4 *>(n_contrib + f.pix_base + pix) = make_int4(0, 0, 0, 0);
+        }
+        return;
+    }
 #pragma unroll 1
     for (int k = lane; k < kTilePix; k += 32) {
         const int px = tx * TW + (k % TW), py = ty * TH + (k / TW);
@@ -307,12 +426,29 @@ __device__ __forceinline__ void empty_tile(const Ctx &c, long long t, float *img
     }
 }
 
-// Compositing statistics of one warp (counting instances only): list entries scanned, entries
-// that reach the block by their mask, visits that evaluated an entry (one with some pixel past the
-// cutoffs; warp-uniform), and the (pixel, entry) pairs that blend or take a gradient (this lane's).
+// Compositing statistics of one warp (counting instances only, S = 1): list entries scanned, entries
+// that reach the block by their mask, visits that some pixel of the block takes (past the cutoffs;
+// warp-uniform), and the (pixel, entry) pairs that blend or take a gradient (this lane's). taken: the
+// stage's slots of each half that some pixel took.
 struct WalkStats {
     unsigned long long staged, hits, visits;
-    unsigned lanes;
+    unsigned lanes, taken[2];
+    // slots j and j + 1 of the stage: whether this lane's pixel takes them
+    __device__ __forceinline__ void step(int j, bool a, bool b) {
+        const unsigned va = __ballot_sync(0xffffffffu, a), vb = __ballot_sync(0xffffffffu, b);
+        taken[0] |= ((va & 0xffffu) ? 1u << j : 0u) | ((vb & 0xffffu) ? 2u << j : 0u);
+        taken[1] |= ((va >> 16) ? 1u << j : 0u) | ((vb >> 16) ? 2u << j : 0u);
+        lanes += (a ? 1u : 0u) + (b ? 1u : 0u);
+    }
+    // the stage's end; reach: the lanes whose staged entry went to each half's slots
+    __device__ __forceinline__ void stage(const unsigned reach[2]) {
+        const int lane = threadIdx.x & 31;
+        const unsigned lt = (1u << lane) - 1u;
+        bool v = false;
+        for (int h = 0; h < 2; ++h) v = v || (((reach[h] >> lane) & 1u) && ((taken[h] >> __popc(reach[h] & lt)) & 1u));
+        visits += __popc(__ballot_sync(0xffffffffu, v));
+        taken[0] = taken[1] = 0u;
+    }
 };
 
 // Shared memory of the colour initialisation's sums: the visits' weights and the block's target.
@@ -321,26 +457,25 @@ struct __align__(16) AccMem {
     float target[3 * 32];
 };
 
-// Adds the weights w and w times the target colour of 16 slots' entries (slot0 ...; bit e of
-// `visited`: row e holds a visit) to their records' first four accumulators in acc.
+// Adds the weights w and w times the target colour of the entries in slots slot0 ... slot0 + 15 of each half
+// (n[h] slots in all) to their records' first four accumulators in acc.
 template <int S>
-__device__ __forceinline__ void flush_acc(const AccMem &r, const WarpMem<S> &m, int slot0, unsigned visited, float *acc) {
-    const int lane = threadIdx.x & 31;
+__device__ __forceinline__ void flush_acc(const AccMem &r, const WarpMem<S> &m, int slot0, const int n[2], float *acc) {
+    const int lane = threadIdx.x & 31, h = lane >> 4, slot = slot0 + (lane & 15);
     __syncwarp();
     float2 s = make_float2(0.f, 0.f), c0 = s, c1 = s, c2 = s;
 #pragma unroll
-    for (int q = 0; q < 2; ++q) {
-        float2 v[4];
+    for (int q = 0; q < 4; ++q) {
+        float2 v[2];
         row_pairs(r.w, q, v);
-        s = __fadd2_rn(s, __fadd2_rn(__fadd2_rn(v[0], v[1]), __fadd2_rn(v[2], v[3])));
+        s = __fadd2_rn(s, __fadd2_rn(v[0], v[1]));
         add_dot(c0, v, r.target, q);
         add_dot(c1, v, r.target + 32, q);
         add_dot(c2, v, r.target + 64, q);
     }
-    float t[4] = {s.x + s.y, c0.x + c0.y, c1.x + c1.y, c2.x + c2.y};
-    add_halves<4>(t);
-    if (lane < 16 && ((visited >> lane) & 1u))
-        red_add4(acc + (size_t)__float_as_uint(m.q[slot0 + lane].w) * kG2Floats, t[0], t[1], t[2], t[3]);
+    const float t = s.x + s.y;
+    if (slot < (h ? n[1] : n[0]) && t > 0.f)  // else no pixel took the entry
+        red_add4(acc + (size_t)m.half(h)[slot >> 1].idx[slot & 1] * kG2Floats, t, c0.x + c0.y, c1.x + c1.y, c2.x + c2.y);
     __syncwarp();
 }
 
@@ -348,46 +483,50 @@ __device__ __forceinline__ void flush_acc(const AccMem &r, const WarpMem<S> &m, 
 // ACC: colour-initialisation accumulation into acc (see k_render_fwd).
 template <int S, bool ACC, bool STATS>
 __device__ __forceinline__ void fwd_walk(const Walk &w, WarpMem<S> &m, PixF &p, AccMem *am, float *acc, WalkStats &st) {
-    const int lane = threadIdx.x & 31;
+    const int lane = threadIdx.x & 31, h = lane >> 4;
     Feed<S, 1> f;
+    Ids<S> d;
     Stage<S> g;
-    f.start(w, 0, w.len);
+    f.start(w, w.len);
     int scanned = f.fill(w, m);
-    load_stage<S>(w, m, f, g);
-    while (g.n) {
+    load_ids<S>(w, m, f, d);
+    scanned += f.fill(w, m);
+    load_stage<S>(w, d, g);
+    load_ids<S>(w, m, f, d);
+    while (g.id.n) {
         if (STATS) st.staged += scanned;
         if (__all_sync(0xffffffffu, p.done)) break;
-        const int n = g.n;
-        commit<S>(g, m);
+        int n[2];
+        unsigned reach[2];
+        if (STATS) st.hits += g.id.n;
+        const int top = commit<S>(w, g, m, n, reach);
         scanned = f.fill(w, m);
-        load_stage<S>(w, m, f, g);
-        float4 A = m.a[0], Q = m.q[0];
-        for (int j0 = 0; j0 < n; j0 += kRows) {
-            unsigned visited = 0u;
-            const int j1 = min(n, j0 + kRows);
-#pragma unroll 4
-            for (int j = j0; j < j1; ++j) {
-                const float4 An = m.a[j + 1], Qn = m.q[j + 1];  // the next slot (any value past the last)
-                const float dx = __fsub_rn(p.pxc, A.x), dy = __fsub_rn(p.pyc, A.y);
-                const float power = power_of(dx, dy, A, Q.x);
-                const bool live = !p.done && !skip(power, Q.y);
-                if (STATS) ++st.hits;
-                if (__any_sync(0xffffffffu, live)) {  // else the colour is not even read
-                    const float wgt = composite(p, live, power, m.c[j], (int)__float_as_uint(Q.z));
-                    if (STATS) {
-                        ++st.visits;
-                        st.lanes += wgt > 0.0f ? 1u : 0u;
-                    }
-                    if (ACC) {
-                        am->w[(j - j0) * kRowStride + lane] = wgt;
-                        visited |= 1u << (j - j0);
-                    }
+        load_stage<S>(w, d, g);
+        load_ids<S>(w, m, f, d);
+        const Pair *s = m.half(h);
+        float4 A = s->A, B = s->B, H = s->H;
+        for (int j0 = 0; j0 < top; j0 += kRows) {
+            const int j1 = min(top, j0 + kRows);
+#pragma unroll 2
+            for (int j = j0; j < j1; j += 2, ++s) {
+                const float2 power = power_of(p.pxc, p.pyc, A, B, make_float2(H.x, H.y));
+                const float tau0 = H.z, tau1 = H.w;
+                A = s[1].A;  // the next pair (any value past the last)
+                B = s[1].B;
+                H = s[1].H;
+                const int2 pos = make_int2(s->pos[0], s->pos[1]);
+                const float4 ca = s->c[0], cb = s->c[1];
+                const float w0 = composite(p, !p.done && !skip(power.x, tau0), power.x, ca, pos.x);
+                const float w1 = composite(p, !p.done && !skip(power.y, tau1), power.y, cb, pos.y);
+                if (STATS) st.step(j, w0 > 0.f, w1 > 0.f);
+                if (ACC) {
+                    am->w[(j - j0) * kRowStride + lane] = w0;
+                    am->w[(j - j0 + 1) * kRowStride + lane] = w1;
                 }
-                A = An;
-                Q = Qn;
             }
-            if (ACC && visited) flush_acc<S>(*am, m, j0, visited, acc);
+            if (ACC) flush_acc<S>(*am, m, j0, n, acc);
         }
+        if (STATS) st.stage(reach);
     }
 }
 
@@ -399,14 +538,6 @@ struct PixB {
     int last;
 };
 
-// e^x for the compositing backward, as 2^(x log2 e) on the hardware's base-2 exponential in its
-// flush-to-zero form: the general form guards against subnormal results with three more
-// instructions, and no weight that counts (alpha >= 1/255) is near that range.
-__device__ __forceinline__ float exp_ftz(float x) {
-    float y;
-    asm("ex2.approx.ftz.f32 %0, %1;" : "=f"(y) : "f"(__fmul_rn(x, 1.44269504088896341f)));
-    return y;
-}
 __device__ __forceinline__ float rcp_ftz(float x) {
     float y;
     asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(y) : "f"(x));
@@ -446,35 +577,31 @@ struct __align__(16) GradMem {
     float dl[3 * 32];
 };
 
-// Adds the gradient sums of 16 slots' entries (slot0 ...; bit e of `visited`: row e holds a visit):
-// the sums over the block's pixels of g (dx, dy, dx^2, dx dy, dy^2, 1), (dx, dy) = pixel centre -
-// mean, and of w dL/dcolour, to the entries' 2-D gradient slots in g2. dy is one number per pixel
-// row, so the y moments come from the row sums. Each half of the warp adds half of the nine sums
-// as 16-byte reductions: scalar ones of the same sums are nine instead of three per entry.
+// Adds the gradient sums of the entries in slots slot0 ... slot0 + 15 of each half (n[h] slots in all):
+// the sums over the half's pixels of g (dx, dy, dx^2, dx dy, dy^2, 1), (dx, dy) = pixel centre -
+// mean, and of w dL/dcolour, to the entries' 2-D gradient slots in g2, as 16-byte reductions. dy is
+// one number per pixel row, so the y moments come from the row sums.
 template <int S>
 __device__ __forceinline__ void flush_grads(const GradMem &r, const WarpMem<S> &m, const Walk &w, int slot0,
-                                            unsigned visited, float *g2) {
-    const int lane = threadIdx.x & 31, e = lane & 15, h = lane >> 4;
+                                            const int n[2], float *g2) {
+    const int lane = threadIdx.x & 31, h = lane >> 4;
+    const bool mine = slot0 + (lane & 15) < (h ? n[1] : n[0]);
+    const int slot = mine ? slot0 + (lane & 15) : slot0;  // none: any other, its sums are not added
     __syncwarp();
-    const bool mine = (visited >> e) & 1u;
-    const int slot = mine ? slot0 + e : slot0;  // a slot not visited: any other, its sums are not added
-    const float2 uv = *reinterpret_cast<const float2 *>(&m.a[slot]);
-    float2 dx[4];
-#pragma unroll
-    for (int i = 0; i < 4; ++i) dx[i] = make_float2(w.bx0 + (float)(2 * i) - uv.x, w.bx0 + (float)(2 * i + 1) - uv.x);
+    const float *a = reinterpret_cast<const float *>(&m.half(h)[slot >> 1].A) + (slot & 1);
+    const float nu = a[0] + (w.bx0 + (float)(4 * h)), nv = a[2] + w.by0;  // first pixel centre - mean
+    const float2 dx[2] = {make_float2(nu, nu + 1.0f), make_float2(nu + 2.0f, nu + 3.0f)};
     float t[9];
     float2 c0 = make_float2(0.f, 0.f), c1 = c0, c2 = c0;
 #pragma unroll
-    for (int q = 0; q < 2; ++q) {
-        const float dy = w.by0 + (float)(2 * h + q) - uv.y;
-        float2 g[4], x[4];
+    for (int q = 0; q < 4; ++q) {
+        const float dy = nv + (float)q;
+        float2 g[2], x[2];
         row_pairs(r.d, q, g);
-#pragma unroll
-        for (int i = 0; i < 4; ++i) x[i] = __fmul2_rn(g[i], dx[i]);
-        const float2 r0 = __fadd2_rn(__fadd2_rn(g[0], g[1]), __fadd2_rn(g[2], g[3]));
-        const float2 r1 = __fadd2_rn(__fadd2_rn(x[0], x[1]), __fadd2_rn(x[2], x[3]));
-        const float2 r2 = __fadd2_rn(__ffma2_rn(x[0], dx[0], __fmul2_rn(x[1], dx[1])),
-                                     __ffma2_rn(x[2], dx[2], __fmul2_rn(x[3], dx[3])));
+        x[0] = __fmul2_rn(g[0], dx[0]);
+        x[1] = __fmul2_rn(g[1], dx[1]);
+        const float2 r0 = __fadd2_rn(g[0], g[1]), r1 = __fadd2_rn(x[0], x[1]);
+        const float2 r2 = __ffma2_rn(x[0], dx[0], __fmul2_rn(x[1], dx[1]));
         const float s0 = r0.x + r0.y, s1 = r1.x + r1.y, s2 = r2.x + r2.y, sy = dy * s0;
         t[0] = q ? t[0] + s1 : s1;
         t[1] = q ? t[1] + sy : sy;
@@ -490,15 +617,14 @@ __device__ __forceinline__ void flush_grads(const GradMem &r, const WarpMem<S> &
     t[6] = c0.x + c0.y;
     t[7] = c1.x + c1.y;
     t[8] = c2.x + c2.y;
-    add_halves<9>(t);
-    if (mine) {
-        float *dst = g2 + (size_t)__float_as_uint(m.q[slot].w) * kG2Floats;
-        if (h == 0) {
-            red_add4(dst, t[0], t[1], t[2], t[3]);
-        } else {
-            red_add4(dst + 4, t[4], t[5], t[6], t[7]);
-            red_add(dst + 8, t[8]);
-        }
+    unsigned any = 0u;  // all sums zero: no pixel took the entry
+#pragma unroll
+    for (int i = 0; i < 9; ++i) any |= __float_as_uint(t[i]);
+    if (mine && (any << 1)) {
+        float *dst = g2 + (size_t)m.half(h)[slot >> 1].idx[slot & 1] * kG2Floats;
+        red_add4(dst, t[0], t[1], t[2], t[3]);
+        red_add4(dst + 4, t[4], t[5], t[6], t[7]);
+        red_add(dst + 8, t[8]);
     }
     __syncwarp();
 }
@@ -506,53 +632,61 @@ __device__ __forceinline__ void flush_grads(const GradMem &r, const WarpMem<S> &
 // The reverse walk of one pixel block over list positions [0, top), top the block's largest
 // contributor count.
 template <int S, bool STATS>
-__device__ __forceinline__ void bwd_walk(const Walk &w, WarpMem<S> &m, GradMem &gm, PixB &p, float *g2, int top,
+__device__ __forceinline__ void bwd_walk(const Walk &w, WarpMem<S> &m, GradMem &gm, PixB &p, float *g2, int last,
                                          WalkStats &st) {
-    const int lane = threadIdx.x & 31;
-    if (top <= 0) return;
+    const int lane = threadIdx.x & 31, h = lane >> 4;
+    if (last <= 0) return;
     Feed<S, -1> f;
+    Ids<S> d;
     Stage<S> g;
-    f.start(w, 0, top);
+    f.start(w, last);
     int scanned = f.fill(w, m);
-    load_stage<S>(w, m, f, g);
-    while (g.n) {
-        if (STATS) st.staged += scanned;
-        const int n = g.n;
-        commit<S>(g, m);
-        scanned = f.fill(w, m);
-        load_stage<S>(w, m, f, g);
-        float4 A = m.a[0], Q = m.q[0];
-        for (int j0 = 0; j0 < n; j0 += kRows) {
-            unsigned visited = 0u;
-            const int j1 = min(n, j0 + kRows);
-#pragma unroll 2
-            for (int j = j0; j < j1; ++j) {
-                const float4 An = m.a[j + 1], Qn = m.q[j + 1];  // the next slot (any value past the last)
-                const float dx = __fsub_rn(p.pxc, A.x), dy = __fsub_rn(p.pyc, A.y);
-                const float power = power_of(dx, dy, A, Q.x);
-                const bool live = (int)__float_as_uint(Q.z) <= p.last && !skip(power, Q.y);
-                if (STATS) ++st.hits;
-                if (__any_sync(0xffffffffu, live)) {  // else the colour is not even read
-                    if (STATS) {
-                        ++st.visits;
-                        st.lanes += live ? 1u : 0u;
-                    }
-                    float dpow, wgt;
-                    accumulate(p, live, power, m.c[j], dpow, wgt);
-                    gm.d[(j - j0) * kRowStride + lane] = dpow;
-                    gm.w[(j - j0) * kRowStride + lane] = wgt;
-                    visited |= 1u << (j - j0);
-                }
-                A = An;
-                Q = Qn;
-            }
-            if (visited) flush_grads<S>(gm, m, w, j0, visited, g2);
+    load_ids<S>(w, m, f, d);
+    scanned += f.fill(w, m);
+    load_stage<S>(w, d, g);
+    load_ids<S>(w, m, f, d);
+    while (g.id.n) {
+        int n[2];
+        unsigned reach[2];
+        if (STATS) {
+            st.staged += scanned;
+            st.hits += g.id.n;
         }
+        const int top = commit<S>(w, g, m, n, reach);
+        scanned = f.fill(w, m);
+        load_stage<S>(w, d, g);
+        load_ids<S>(w, m, f, d);
+        const Pair *s = m.half(h);
+        float4 A = s->A, B = s->B, H = s->H;
+        for (int j0 = 0; j0 < top; j0 += kRows) {
+            const int j1 = min(top, j0 + kRows);
+#pragma unroll 2
+            for (int j = j0; j < j1; j += 2, ++s) {
+                const float2 power = power_of(p.pxc, p.pyc, A, B, make_float2(H.x, H.y));
+                const float tau0 = H.z, tau1 = H.w;
+                A = s[1].A;  // the next pair (any value past the last)
+                B = s[1].B;
+                H = s[1].H;
+                const int2 pos = make_int2(s->pos[0], s->pos[1]);
+                const float4 ca = s->c[0], cb = s->c[1];
+                const bool l0 = pos.x <= p.last && !skip(power.x, tau0), l1 = pos.y <= p.last && !skip(power.y, tau1);
+                if (STATS) st.step(j, l0, l1);
+                float d0, d1, w0, w1;
+                accumulate(p, l0, power.x, ca, d0, w0);
+                accumulate(p, l1, power.y, cb, d1, w1);
+                gm.d[(j - j0) * kRowStride + lane] = d0;
+                gm.d[(j - j0 + 1) * kRowStride + lane] = d1;
+                gm.w[(j - j0) * kRowStride + lane] = w0;
+                gm.w[(j - j0 + 1) * kRowStride + lane] = w1;
+            }
+            flush_grads<S>(gm, m, w, j0, n, g2);
+        }
+        if (STATS) st.stage(reach);
     }
 }
 
-// A (tile, pixel block) item: its frame, the block's pixel (one per lane: column lane % 8 of
-// row lane / 8 of the 8 x 4 block) and the walk over the tile's list.
+// A (tile, pixel block) item: its frame, the block's pixel (one per lane: the block's left 4 x 4 pixels
+// in the warp's first half, the right ones in the second, row by row) and the walk over the tile's list.
 template <int TW>
 __device__ __forceinline__ int block_item(const Ctx &c, unsigned item, int &px, int &py, Walk &w) {
     constexpr int TH = kTilePix / TW, NBX = TW / 8, NB = NBX * (TH / 4);
@@ -565,8 +699,8 @@ __device__ __forceinline__ int block_item(const Ctx &c, unsigned item, int &px, 
     const int lt = (int)(t - f.tile_base);
     const int ty = lt / f.tiles_x, tx = lt - ty * f.tiles_x;
     const int bx = tx * TW + (int)(blk % NBX) * 8, by = ty * TH + (int)(blk / NBX) * 4;
-    px = bx + (lane & 7);
-    py = by + (lane >> 3);
+    px = bx + ((lane >> 4) << 2) + (lane & 3);
+    py = by + ((lane >> 2) & 3);
     w.bx0 = (float)bx + 0.5f;
     w.by0 = (float)by + 0.5f;
     w.blk = blk;
@@ -575,6 +709,7 @@ __device__ __forceinline__ int block_item(const Ctx &c, unsigned item, int &px, 
     w.masks = c.list_masks(st);
     w.len = (int)(c.tile_start[t + 1] - st);
     w.rec = c.records + (size_t)f.rec_base * 3;
+    w.masked = c.masked;
     return b;
 }
 
@@ -603,18 +738,23 @@ __device__ __forceinline__ void flush_loss(const Ctx &c, float loss_acc, float *
     }
 }
 
-// Items: the pixel blocks of the non-empty tiles (work list order, heaviest tiles first), then
-// one item per empty tile, which the warp fills with the background eight pixels per lane.
+// Items: the pixel blocks of the non-empty tiles (work list order, heaviest tiles first), and one item per
+// empty tile, which the warp fills with the background. The empty tiles are spread evenly among the
+// blocks: they are bound by memory (44 bytes a pixel with a target) and most of a face-centred frame, so
+// they run in the shadow of the compositing instead of after it.
 // ACC (colour initialisation, Eq. 3): every blended entry also adds its splatting weight w and
 // w times the pixel's colour in acc_target to the record's first four 2-D gradient slots
 // (flush_acc: one 16-byte reduction per entry and pixel block).
 // STATS (the counting instance): also count the visits that evaluate an entry and the
 // (pixel, entry) pairs that blend, into the compositing statistics of the counters.
-// Bound by instruction issue, and by one warp's walk where few blocks have work. Against staging and
-// testing every list entry per block: 160 -> 127 us on 16 frames of 512 x 512 (N = 60,000), 123 ->
-// 72 us on one of 128 x 128, colour initialisation of ten frames 178 -> 107 us.
+// Bound by instruction issue (67 % of the slots), and by the walks of the heaviest blocks: six CTAs per SM
+// beat eight (more warps, each slower) except where far more blocks have work than fit. Whole-warp
+// entries with a vote per entry, then this: 127 -> 121 us on 16 frames of 512 x 512 (N = 60,000), 248 ->
+// 182 us with the avatar bound to a mesh, 233 -> 160 us on 15 frames of 256 to 1,024 pixels of five
+// avatars, 594 -> 520 us on 64 of eight, 66 -> 49 us on one of 128 x 128, colour initialisation of ten
+// frames 107 -> 98 us. Empty tiles after all blocks instead of among the lighter ones: 559 us on the 64.
 template <int TW, int S, bool ACC, bool STATS = false>
-__global__ void __launch_bounds__(32 * kWarpsPerCta)
+__global__ void __launch_bounds__(32 * kWarpsPerCta, ACC ? 4 : 6)
 k_render_fwd(Ctx c, float *__restrict__ img, float *__restrict__ T_final, int *__restrict__ n_contrib,
              const float *__restrict__ target, int loss_kind, float *__restrict__ dl_dimg,
              const float *__restrict__ acc_target) {
@@ -629,18 +769,31 @@ k_render_fwd(Ctx c, float *__restrict__ img, float *__restrict__ T_final, int *_
     AccMem *am = s_acc + (ACC ? wid : 0);
     const unsigned n_work = c.cnt->n_work, n_blocks = n_work * NB;
     const unsigned n_items = n_blocks + ((unsigned)c.T - n_work);
+    // the first items, one per resident warp, are the heaviest blocks; from there empty tiles per item,
+    // as a 32-bit fraction rounded up: e(i) = i frac / 2^32 of the next i items are empty tiles, and all
+    // of them together are exactly the empty tiles
+    const unsigned first = min(n_blocks, gridDim.x * kWarpsPerCta), rest = n_items - first;
+    const unsigned long long frac = (((unsigned long long)(n_items - n_blocks) << 32) + rest - 1) / max(rest, 1u);
+    const bool vec = ((reinterpret_cast<uintptr_t>(img) | reinterpret_cast<uintptr_t>(T_final) |
+                       reinterpret_cast<uintptr_t>(n_contrib) | reinterpret_cast<uintptr_t>(target) |
+                       reinterpret_cast<uintptr_t>(dl_dimg)) & 15) == 0;
     float loss_acc = 0.0f;
-    WalkStats st{0ull, 0ull, 0ull, 0u};  // STATS
+    WalkStats st{0ull, 0ull, 0ull, 0u, {0u, 0u}};  // STATS
     while (true) {
         unsigned item = 0;
         if (lane == 0) item = atomicAdd(&c.cnt->next_fwd, 1u);
         item = __shfl_sync(0xffffffffu, item, 0);
         if (item >= n_items) break;
-        if (item >= n_blocks) {  // an empty tile: background, T = 1, no contributors
-            empty_tile<TW>(c, c.work[n_work + (item - n_blocks)], img, T_final, n_contrib, target, loss_kind,
-                           dl_dimg, loss_acc);
+        unsigned e0 = 0u, e1 = 0u;
+        if (item >= first) {
+            e0 = (unsigned)(((item - first) * frac) >> 32);
+            e1 = (unsigned)(((item - first + 1ull) * frac) >> 32);
+        }
+        if (e1 != e0) {  // an empty tile: background, T = 1, no contributors
+            empty_tile<TW>(c, c.work[n_work + e0], vec, img, T_final, n_contrib, target, loss_kind, dl_dimg, loss_acc);
             continue;
         }
+        item -= e0;
         int px, py;
         const int b = block_item<TW>(c, item, px, py, w);
         const FrameInfo &f = c.frames[b];
@@ -669,14 +822,13 @@ k_render_fwd(Ctx c, float *__restrict__ img, float *__restrict__ T_final, int *_
 
 // STATS (the counting instance): also count the visits that evaluate an entry and the
 // (pixel, entry) pairs that take a gradient, into the compositing statistics of the counters.
-// Bound by instruction issue. 16 frames of 512 x 512 of a 60,000-Gaussian avatar, not yet fitted:
-// 301 -> 170 us (222 -> 117 M warp instructions) against staging every list entry per block and
-// reducing nine sums by shuffles at every visit; one 128 x 128 frame, where only 80 warps have work
-// and the length of one warp's walk is what counts: 182 -> 96 us. Six CTAs per SM (80 registers):
-// without the bound the row sums take 128 registers and the occupancy they cost eats the gain
-// (307 us).
+// Bound by instruction issue (65 % of the slots, 65 instructions per step of the two halves) and by the
+// walks of the heaviest blocks: four CTAs per SM (128 registers) beat five and six. Whole-warp entries with
+// a vote per entry, then this: 16 frames of 512 x 512 of a 60,000-Gaussian avatar, not yet fitted, 170 ->
+// 152 us, bound to a mesh 344 -> 256, 64 frames of eight avatars 644 -> 588; one 128 x 128 frame, where only
+// 80 warps have work and the length of one warp's walk is what counts, 94 -> 53 us.
 template <int TW, int S, bool STATS = false>
-__global__ void __launch_bounds__(32 * kWarpsPerCta, S == 1 ? 6 : 1)
+__global__ void __launch_bounds__(32 * kWarpsPerCta, 4)
 k_render_bwd(Ctx c, const float *__restrict__ dl_dimg, const float *__restrict__ T_final,
              const int *__restrict__ n_contrib) {
     constexpr int TH = kTilePix / TW, NB = (TW / 8) * (TH / 4);
@@ -688,7 +840,7 @@ k_render_bwd(Ctx c, const float *__restrict__ dl_dimg, const float *__restrict__
     Walk w;
     GradMem &gm = s_g[wid];
     const unsigned n_items = c.cnt->n_work * NB;
-    WalkStats st{0ull, 0ull, 0ull, 0u};  // STATS
+    WalkStats st{0ull, 0ull, 0ull, 0u, {0u, 0u}};  // STATS
     while (true) {
         unsigned item = 0;
         if (lane == 0) item = atomicAdd(&c.cnt->next_bwd, 1u);
@@ -759,12 +911,10 @@ cudaError_t fwd_dispatch(const Ctx &c, int grid, int sb, float *img, float *T, i
         return fwd_inst<16, 1, false, true>(c, grid, img, T, n, tg, lk, dl, acc_tg, s);
     if (c.tw == 16) {
         if (sb == 64) return fwd_inst<16, 1, ACC>(c, grid, img, T, n, tg, lk, dl, acc_tg, s);
-        if (sb == 128) return fwd_inst<16, 2, ACC>(c, grid, img, T, n, tg, lk, dl, acc_tg, s);
-        return fwd_inst<16, 3, ACC>(c, grid, img, T, n, tg, lk, dl, acc_tg, s);
+        return fwd_inst<16, 2, ACC>(c, grid, img, T, n, tg, lk, dl, acc_tg, s);
     }
     if (sb == 64) return fwd_inst<8, 1, ACC>(c, grid, img, T, n, tg, lk, dl, acc_tg, s);
-    if (sb == 128) return fwd_inst<8, 2, ACC>(c, grid, img, T, n, tg, lk, dl, acc_tg, s);
-    return fwd_inst<8, 3, ACC>(c, grid, img, T, n, tg, lk, dl, acc_tg, s);
+    return fwd_inst<8, 2, ACC>(c, grid, img, T, n, tg, lk, dl, acc_tg, s);
 }
 
 template <int TW, int S, bool STATS = false>
@@ -787,17 +937,13 @@ cudaError_t launch_render_fwd(const Ctx &c, int grid, int smem_batch, float *img
                                nullptr, stats, s);
 }
 
+// smem_batch: the backward stages 32 entries at a time whatever the staging size (its slots and row sums
+// take 37 KB per CTA; the forward's stages grow to 64 entries at 128 and 256).
 cudaError_t launch_render_bwd(const Ctx &c, int grid, int smem_batch, const float *dl_dimg,
                               const float *T_final, const int *n_contrib, bool stats, cudaStream_t s) {
     if (stats && c.tw == 16 && smem_batch == 64) return bwd_inst<16, 1, true>(c, grid, dl_dimg, T_final, n_contrib, s);
-    if (c.tw == 16) {
-        if (smem_batch == 64) return bwd_inst<16, 1>(c, grid, dl_dimg, T_final, n_contrib, s);
-        if (smem_batch == 128) return bwd_inst<16, 2>(c, grid, dl_dimg, T_final, n_contrib, s);
-        return bwd_inst<16, 3>(c, grid, dl_dimg, T_final, n_contrib, s);
-    }
-    if (smem_batch == 64) return bwd_inst<8, 1>(c, grid, dl_dimg, T_final, n_contrib, s);
-    if (smem_batch == 128) return bwd_inst<8, 2>(c, grid, dl_dimg, T_final, n_contrib, s);
-    return bwd_inst<8, 3>(c, grid, dl_dimg, T_final, n_contrib, s);
+    return c.tw == 16 ? bwd_inst<16, 1>(c, grid, dl_dimg, T_final, n_contrib, s)
+                      : bwd_inst<8, 1>(c, grid, dl_dimg, T_final, n_contrib, s);
 }
 
 }  // namespace rgba

@@ -103,8 +103,8 @@ struct Counters {
     unsigned done_bwd;    // every launch starts from zero without a memset
     // compositing statistics, counted only by the counting instances of the compositing kernels
     // (rgba_profile_enable(ctx, 2)); zeroed with the rest at the start of every preprocess
-    // per direction: list entries staged, box hits, (entry, pixel block) visits that evaluated
-    // the entry, (pixel, entry) pairs that blended (forward) or took a gradient (backward)
+    // per direction: list entries scanned, mask hits, (entry, pixel block) visits that some pixel takes,
+    // (pixel, entry) pairs that blended (forward) or took a gradient (backward)
     unsigned long long st_fwd[4];
     unsigned long long st_bwd[4];
 };
