@@ -8,10 +8,11 @@
 // kernel drops (depth << 32 | index) keys, with a mask of the pixel blocks each splat reaches in
 // the low byte of the index word, into their tile's segment (by
 // slot, or by a cursor atomic for larger rectangles), and one CTA per non-empty tile sorts its
-// list, with the key compressed to (depth - segment minimum) << 32 | index: in shared memory by
+// list: in shared memory by
 // one bucket pass on the top depth bits and a placement of every key by its rank in its bucket,
 // or, for long segments, by the same bucket pass with the keys in L2; buckets too crowded for it
-// fall back to a stable LSD radix sort. Because the key carries the index, the result is unique.
+// fall back to a stable LSD radix sort of the keys compressed to (depth - segment minimum) << 32 |
+// index. Because the key carries the index, the result is unique.
 #include "reach.cuh"
 #include "rgba_internal.cuh"
 
@@ -274,22 +275,16 @@ __global__ void __launch_bounds__(kScatterThreads) k_scatter(Ctx c) {
     }
 }
 
-// Asynchronous 8-byte copy global -> shared (both addresses 8-byte aligned), completed by
-// cp.async.wait_all.
-__device__ __forceinline__ void cp_async8(void *dst, const void *src) {
-    asm volatile("cp.async.ca.shared.global [%0], [%1], 8;"
-                 :: "r"(static_cast<unsigned>(__cvta_generic_to_shared(dst))), "l"(src) : "memory");
-}
-
 constexpr int kSortThreads = 512;
 constexpr int kSortWarps = kSortThreads / 32;
-constexpr int kRadixCap = 8192;                  // keys a segment may have for the shared-memory radix sort
-constexpr int kMidCap = 3 * kRadixCap / 2;       // keys a segment may have for the position bucket sort
-// the position sort's keys, ranks and positions fill the key area and rank array of the
-// shared-memory sort exactly, so the kernel needs no more shared memory than that one: a larger
-// footprint kept the next kernel's CTAs from starting on the SMs early and cost 0.12 ms per
-// training step in the captured graph
-static_assert(kMidCap * (8 + 2 + 2) <= kRadixCap * (2 * 8 + 2), "position sort fits the key area and rank array");
+// Shared memory of the sort: 96 KB, so that two CTAs share an SM. The bucket sort takes kSmemCap keys
+// and 2^kMaxBits 2-byte bucket counts; the radix sort kRadixCap keys twice, their ranks and the digit counts;
+// the sort of long lists 2^kStreamBits 4-byte bucket counts.
+constexpr int kSmemCap = 16 * kSortThreads;
+constexpr int kMaxBits = 14;
+constexpr int kRadixCap = 4544;
+constexpr int kSortSmem = kSmemCap * 8 + (2 << kMaxBits) + 16;
+static_assert(kRadixCap * (2 * 8 + 2) + (kSortWarps * 256 + kSortWarps) * 4 <= kSortSmem, "radix sort fits");
 constexpr int kDigitParts = kSortThreads / 256;  // threads sharing one digit's column of warp counts
 static_assert(kSortThreads % 256 == 0 && 32 % kDigitParts == 0, "whole digits per warp");
 
@@ -432,38 +427,74 @@ __device__ unsigned long long *radix_sort(unsigned long long *a, unsigned long l
 
 constexpr int kTieRun = 32;  // longest run of equal depths the tie pass orders by itself
 
-constexpr int kBucketBits = 12;  // buckets of the one-pass shared-memory sort
-constexpr int kBucketRun = 64;   // longest bucket the rank placement orders by itself
-static_assert((1 << kBucketBits) + kSortWarps <= kSortWarps * 256 + kSortWarps, "bucket counts fit the count area");
+constexpr int kBucketRun = 64;  // longest bucket the rank placement orders by itself
 
-// Sort of L <= kRadixCap compressed keys (depth - d0) << 32 | index in shared memory by the
-// top kBucketBits bits of the db-bit depth spread, then each bucket by the full key: one
-// shared-memory atomic per key gives its bucket and its slot in it, an exclusive scan of the
-// bucket counts the bucket starts, a scatter puts every key in its bucket (in any order
-// inside), and every key then counts the smaller keys of its bucket and moves to that rank
-// (keys are distinct: the index differs). Buckets are short (L keys over 2^kBucketBits
-// buckets), so the count costs little and is the same for every key of a bucket. A bucket
-// longer than kBucketRun sets *s_long and the keys are returned grouped by bucket for the
-// caller's fallback. Returns the buffer holding the result.
-__device__ unsigned long long *bucket_sort(unsigned long long *a, unsigned long long *b, int L, unsigned d0, int db,
-                                           unsigned *s_hist /* >= 2^kBucketBits + kSortWarps, zeroed */,
-                                           unsigned short *s_rank, unsigned *s_long) {
-    constexpr int NB = 1 << kBucketBits, PER = NB / kSortThreads;
-    static_assert(NB % kSortThreads == 0, "whole buckets per thread");
+// Sort of L <= KPT kSortThreads keys at g by one bucket pass: each thread keeps its KPT keys in registers,
+// a shared-memory atomic per key counts the 2^BITS buckets of the depth spread (two 16-bit counts to a
+// word) and gives the key its slot in its bucket, an exclusive scan turns the counts into starts, the
+// keys go to their bucket's run in s_keys (in any order inside), and every key there counts the smaller
+// keys of its bucket (keys are distinct: the index differs) and writes its Gaussian index and block
+// mask straight to its rank in the tile's lists `out` and `out_mask`. Per key that is one shared-memory
+// write and, with about two buckets per key, two or three reads in the last step: the
+// shared-memory passes over the keys are what bounds the sort of a list. Returns false, with nothing
+// written, when some bucket is longer than kBucketRun.
+template <int KPT, int BITS>
+__device__ __forceinline__ bool bucket_sort(const unsigned long long *g, int L, unsigned long long *s_keys, unsigned *s_cnt,
+                                            unsigned *s_sum /* [kSortWarps] */, unsigned *s_dmin, unsigned *s_dmax,
+                                            bool masked, unsigned *__restrict__ out, unsigned char *out_mask) {
+    constexpr int NW = 1 << (BITS - 1), PER = NW / kSortThreads;  // words, words per thread
+    static_assert(PER % 4 == 0, "whole 16-byte groups per thread");
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
-    const int bshift = max(0, db - kBucketBits);
-    // the bucket of a key: the top kBucketBits bits of its depth above the segment's minimum
-    auto bucket = [&](unsigned long long k) { return ((unsigned)(k >> 32) - d0) >> bshift; };
-    unsigned *wsum = s_hist + NB;
-    for (int e = tid; e < L; e += kSortThreads)
-        s_rank[e] = (unsigned short)atomicAdd(&s_hist[bucket(a[e])], 1u);
-    __syncthreads();
-    {  // exclusive scan of the bucket counts; thread t owns buckets [t PER, (t+1) PER)
-        unsigned v[PER], run = 0;
+    unsigned long long k[KPT];
 #pragma unroll
-        for (int q = 0; q < PER; ++q) {
-            v[q] = run;
-            run += s_hist[tid * PER + q];
+    for (int i = 0; i < KPT; ++i) k[i] = tid + i * kSortThreads < L ? g[tid + i * kSortThreads] : 0ull;
+    uint4 *cnt4 = reinterpret_cast<uint4 *>(s_cnt);
+#pragma unroll
+    for (int i = 0; i < PER / 4; ++i) cnt4[tid + i * kSortThreads] = make_uint4(0u, 0u, 0u, 0u);
+    unsigned dmin = 0xffffffffu, dmax = 0u;
+#pragma unroll
+    for (int i = 0; i < KPT; ++i)
+        if (tid + i * kSortThreads < L) {
+            dmin = min(dmin, (unsigned)(k[i] >> 32));
+            dmax = max(dmax, (unsigned)(k[i] >> 32));
+        }
+    dmin = __reduce_min_sync(0xffffffffu, dmin);
+    dmax = __reduce_max_sync(0xffffffffu, dmax);
+    if (lane == 0) {
+        atomicMin(s_dmin, dmin);
+        atomicMax(s_dmax, dmax);
+    }
+    __syncthreads();
+    const unsigned d0 = *s_dmin;
+    const int bshift = max(0, 32 - __clz(*s_dmax - d0) - BITS);
+    auto bucket = [&](unsigned long long key) { return ((unsigned)(key >> 32) - d0) >> bshift; };
+    unsigned slot[KPT / 4], crowd = 0u;  // slots below kBucketRun, a byte each
+#pragma unroll
+    for (int i = 0; i < KPT; ++i) {
+        unsigned s = 0u;
+        if (tid + i * kSortThreads < L) {
+            const unsigned b = bucket(k[i]), sh = 16u * (b & 1u);
+            s = (atomicAdd(&s_cnt[b >> 1], 1u << sh) >> sh) & 0xffffu;
+        }
+        crowd = max(crowd, s);
+        slot[i / 4] = (i & 3 ? slot[i / 4] : 0u) | s << (8 * (i & 3));
+    }
+    if (__syncthreads_or(crowd >= (unsigned)kBucketRun)) return false;
+    {  // exclusive scan of the counts; thread t owns words [t PER, (t + 1) PER)
+        unsigned w[PER], run = 0u;
+#pragma unroll
+        for (int i = 0; i < PER / 4; ++i) {
+            const uint4 q = cnt4[tid * (PER / 4) + i];
+            w[4 * i] = q.x;
+            w[4 * i + 1] = q.y;
+            w[4 * i + 2] = q.z;
+            w[4 * i + 3] = q.w;
+        }
+#pragma unroll
+        for (int i = 0; i < PER; ++i) {
+            const unsigned c0 = w[i] & 0xffffu, c1 = w[i] >> 16;
+            w[i] = run | ((run + c0) << 16);
+            run += c0 + c1;
         }
         unsigned x = run;
 #pragma unroll
@@ -471,101 +502,39 @@ __device__ unsigned long long *bucket_sort(unsigned long long *a, unsigned long 
             const unsigned y = __shfl_up_sync(0xffffffffu, x, o);
             if (lane >= o) x += y;
         }
-        if (lane == 31) wsum[warp] = x;
+        if (lane == 31) s_sum[warp] = x;
         __syncthreads();
         unsigned off = x - run;
 #pragma unroll
-        for (int q = 0; q < kSortWarps; ++q) off += q < warp ? wsum[q] : 0u;
+        for (int q = 0; q < kSortWarps; ++q) off += q < warp ? s_sum[q] : 0u;
+        off |= off << 16;  // both halves: no start exceeds kSmemCap
 #pragma unroll
-        for (int q = 0; q < PER; ++q) s_hist[tid * PER + q] = off + v[q];
+        for (int i = 0; i < PER / 4; ++i)
+            cnt4[tid * (PER / 4) + i] = make_uint4(w[4 * i] + off, w[4 * i + 1] + off, w[4 * i + 2] + off, w[4 * i + 3] + off);
+        if (tid == 0) s_cnt[NW] = (unsigned)L;  // the last bucket's end
     }
     __syncthreads();
-    for (int e = tid; e < L; e += kSortThreads) {
-        const unsigned long long k = a[e];
-        b[s_hist[bucket(k)] + s_rank[e]] = k;
-    }
+    const unsigned short *start = reinterpret_cast<const unsigned short *>(s_cnt);
+#pragma unroll
+    for (int i = 0; i < KPT; ++i)
+        if (tid + i * kSortThreads < L) s_keys[start[bucket(k[i])] + ((slot[i / 4] >> (8 * (i & 3))) & 0xffu)] = k[i];
     __syncthreads();
+#pragma unroll 2
     for (int p = tid; p < L; p += kSortThreads) {
-        const unsigned long long k = b[p];
-        const unsigned bk = bucket(k);
-        const int lo = (int)s_hist[bk], hi = bk + 1 < (unsigned)NB ? (int)s_hist[bk + 1] : L;
-        if (hi - lo > kBucketRun) {
-            *s_long = 1u;
-            continue;
-        }
-        int rank = 0;
-        for (int q = lo; q < hi; ++q) rank += b[q] < k;
-        a[lo + rank] = k;
+        const unsigned long long key = s_keys[p];
+        const unsigned b = bucket(key);
+        const int lo = start[b], hi = start[b + 1];
+        int rank = lo;
+        for (int q = lo; q < hi; ++q) rank += s_keys[q] < key;
+        out[rank] = low_index(masked, (unsigned)key);
+        out_mask[rank] = low_mask(masked, (unsigned)key);
     }
-    __syncthreads();
-    return *s_long ? b : a;  // b still holds every key for the fallback
+    return true;
 }
 
-// Sort of kRadixCap < L <= kMidCap keys held in shared memory as they are (a) by the same
-// one-pass bucketing, but moving 2-byte positions instead of 8-byte keys so that half as many
-// keys again fit in the same shared memory: a shared-memory atomic per
-// key gives its bucket and its slot, a scan the bucket starts, each key's position goes to its
-// bucket's run in s_pos, and every key counts the smaller keys of its bucket (read through the
-// positions) and writes its Gaussian index and block mask straight to its rank in the tile's lists
-// `out` and `out_mask`.
-// Returns false when some bucket is longer than kBucketRun (its keys are then not written; the
-// caller sorts the whole segment again another way).
-__device__ bool bucket_sort_pos(const unsigned long long *a, int L, unsigned d0, int db,
-                                unsigned *s_hist /* >= 2^kBucketBits + kSortWarps, zeroed */,
-                                unsigned short *s_rank, unsigned short *s_pos, unsigned *s_long, bool masked,
-                                unsigned *__restrict__ out, unsigned char *__restrict__ out_mask) {
-    constexpr int NB = 1 << kBucketBits, PER = NB / kSortThreads;
-    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
-    const int bshift = max(0, db - kBucketBits);
-    auto bucket = [&](unsigned long long k) { return ((unsigned)(k >> 32) - d0) >> bshift; };
-    unsigned *wsum = s_hist + NB;
-    for (int e = tid; e < L; e += kSortThreads)
-        s_rank[e] = (unsigned short)atomicAdd(&s_hist[bucket(a[e])], 1u);
-    __syncthreads();
-    {  // exclusive scan of the bucket counts; thread t owns buckets [t PER, (t+1) PER)
-        unsigned v[PER], run = 0;
-#pragma unroll
-        for (int q = 0; q < PER; ++q) {
-            v[q] = run;
-            run += s_hist[tid * PER + q];
-        }
-        unsigned x = run;
-#pragma unroll
-        for (int o = 1; o < 32; o <<= 1) {
-            const unsigned y = __shfl_up_sync(0xffffffffu, x, o);
-            if (lane >= o) x += y;
-        }
-        if (lane == 31) wsum[warp] = x;
-        __syncthreads();
-        unsigned off = x - run;
-#pragma unroll
-        for (int q = 0; q < kSortWarps; ++q) off += q < warp ? wsum[q] : 0u;
-#pragma unroll
-        for (int q = 0; q < PER; ++q) s_hist[tid * PER + q] = off + v[q];
-    }
-    __syncthreads();
-    for (int e = tid; e < L; e += kSortThreads) s_pos[s_hist[bucket(a[e])] + s_rank[e]] = (unsigned short)e;
-    __syncthreads();
-    for (int p = tid; p < L; p += kSortThreads) {
-        const unsigned long long k = a[s_pos[p]];
-        const unsigned bk = bucket(k);
-        const int lo = (int)s_hist[bk], hi = bk + 1 < (unsigned)NB ? (int)s_hist[bk + 1] : L;
-        if (hi - lo > kBucketRun) {
-            *s_long = 1u;
-            continue;
-        }
-        int rank = 0;
-        for (int q = lo; q < hi; ++q) rank += a[s_pos[q]] < k;
-        out[lo + rank] = low_index(masked, (unsigned)k);
-        out_mask[lo + rank] = low_mask(masked, (unsigned)k);
-    }
-    __syncthreads();
-    return *s_long == 0u;
-}
-
-constexpr int kStreamBits = 14;  // buckets of the sort of long lists, in the key area of the others
+constexpr int kStreamBits = 14;  // buckets of the sort of long lists
 constexpr int kStreamLoads = 8;  // keys per thread in flight in its sweeps
-static_assert((4 << kStreamBits) <= kRadixCap * 16, "bucket counts fit the key area");
+static_assert((4 << kStreamBits) <= kSortSmem, "bucket counts fit");
 
 // Calls f(key) for the L keys at g, kStreamLoads of each thread's loads in flight at once.
 template <typename F>
@@ -639,38 +608,36 @@ __device__ bool bucket_sort_stream(const unsigned long long *g, unsigned long lo
 
 // Persistent: CTAs take (frame, tile) segments from the LPT-ordered work list. A key is
 // (depth, Gaussian index), "index" standing here for the word that also holds the block mask below
-// the index; it is compressed to (depth - min depth) << 32 | index. A segment of
-// up to kRadixCap keys is sorted in shared memory by bucket_sort (one bucket pass, then each
-// bucket by the full key), one of up to kMidCap keys by bucket_sort_pos (the same with 2-byte
-// positions in place of moved keys). A longer one is sorted by bucket_sort_stream with its keys in
-// global memory (mostly L2). A bucket longer than kBucketRun sends a segment of bucket_sort to a
-// full-key radix sort (index bits, then depth bits), and a longer one to a radix sort in global memory
-// on the depth bits only, which leaves runs of equal depth in list order; a tie pass orders each such
-// run by index (insertion sort by the run's first thread), a run longer than kTieRun the full key.
-// Long lists through L2 by buckets instead of radix passes: a batch of 15 frames of five avatars
-// with lists of up to 23,803 keys 475 -> 147 us, 64 frames of eight avatars (24,502) 500 -> 268 us.
-// The sort is bound by round trips to memory, so none of them waits on another: thread 0 claims
-// work items three ahead and, one stage per item, loads the claimed item's tile id and then its
-// list bounds while the CTA sorts the current segment; a segment that fits in shared memory
-// arrives there by asynchronous copies, all in flight at once.
-__global__ void __launch_bounds__(kSortThreads) k_tile_sort(Ctx c) {
-    // [kRadixCap] x 2 keys, [kRadixCap] ranks, counts; the position sort uses the keys and ranks
-    // area as [kMidCap] keys, [kMidCap] ranks, [kMidCap] positions
-    extern __shared__ unsigned long long s_keys[];
-    unsigned short *s_rank = reinterpret_cast<unsigned short *>(s_keys + 2 * kRadixCap);
-    unsigned *s_cnt = reinterpret_cast<unsigned *>(s_rank + kRadixCap);
-    unsigned short *s_rank_mid = reinterpret_cast<unsigned short *>(s_keys + kMidCap);
-    unsigned short *s_pos_mid = s_rank_mid + kMidCap;
-    __shared__ unsigned s_cur, s_st, s_L, s_dmin, s_dmax, s_imax, s_long;
+// the index. A segment of up to kSmemCap keys is sorted by bucket_sort, with more keys per thread and
+// more buckets the longer it is, a longer one by bucket_sort_stream with its keys in
+// global memory (mostly L2). A bucket longer than kBucketRun sends a segment of up to kRadixCap keys to a
+// full-key radix sort in shared memory (index bits, then depth bits), and a longer one to a radix sort in
+// global memory on the depth bits only, which leaves runs of equal depth in list order; a tie pass orders
+// each such run by index (insertion sort by the run's first thread), a run longer than kTieRun the full key.
+// The radix sorts take keys compressed to (depth - min depth) << 32 | index.
+// Bound by the shared-memory passes over the keys and, for short lists, by the load and the barriers
+// between them, so two CTAs share an SM. Keys moved between two shared-memory buffers with 2^12 buckets
+// whatever the length (one CTA per SM, lists of 8,193 to 12,288 keys by positions), then this: one frame with lists
+// of up to 6,321 keys 35 -> 16 us, 15 frames of five avatars 145 -> 80, 16 frames 55 -> 43, ten frames 43 -> 31,
+// 64 frames of eight avatars with lists of up to 24,552 keys 268 -> 188. The same with one CTA of 1,024
+// threads: 14, 68, 49, 35 and 256 us. A list of 12,289 to 24,552 keys through L2 by buckets instead of radix passes:
+// 475 -> 147 us on the 15 frames.
+// Thread 0 claims work items three ahead and, one stage per item, loads the claimed item's tile id and
+// then its list bounds while the CTA sorts the current segment.
+__global__ void __launch_bounds__(kSortThreads, 2) k_tile_sort(Ctx c) {
+    extern __shared__ __align__(16) unsigned long long s_keys[];
+    unsigned *s_cnt = reinterpret_cast<unsigned *>(s_keys + kSmemCap);  // bucket_sort's counts
+    __shared__ unsigned s_cur, s_st, s_L, s_dmin, s_dmax, s_imax, s_long, s_sum[kSortWarps];
     pdl_enter();
     if (c.cnt->overflow) return;
     const unsigned n_work = c.cnt->n_work;
     // thread 0's pipeline: w1 / t1 the next item and its tile, w2 the item after it
     unsigned w1 = 0, t1 = 0, w2 = 0;
     if (threadIdx.x == 0) {
-        const unsigned w0 = atomicAdd(&c.cnt->next_sort, 1u);
-        w1 = atomicAdd(&c.cnt->next_sort, 1u);
-        w2 = atomicAdd(&c.cnt->next_sort, 1u);
+        // the first two items by CTA, the one with the longest list taking the shortest next
+        const unsigned w0 = blockIdx.x;
+        w1 = 2 * gridDim.x - 1 - w0;
+        w2 = 2 * gridDim.x + atomicAdd(&c.cnt->next_sort, 1u);
         const unsigned t0 = w0 < n_work ? c.work[w0] : 0u;
         t1 = w1 < n_work ? c.work[w1] : 0u;
         s_cur = w0 < n_work ? 1u : 0u;
@@ -691,121 +658,96 @@ __global__ void __launch_bounds__(kSortThreads) k_tile_sort(Ctx c) {
                 nend = c.tile_start[t1 + 1];
             }
             t2 = w2 < n_work ? c.work[w2] : 0u;
-            w3 = atomicAdd(&c.cnt->next_sort, 1u);
+            w3 = 2 * gridDim.x + atomicAdd(&c.cnt->next_sort, 1u);
         }
         const unsigned long long *g = c.keys + st;
+        unsigned *out = c.sorted + st;
         unsigned char *masks = c.list_masks(st);  // over the list's keys, once nobody reads them
-        const bool in_smem = L <= (unsigned)kRadixCap;
-        const bool mid = !in_smem && L <= (unsigned)kMidCap;  // the position bucket sort
-        unsigned dmin = 0xffffffffu, dmax = 0u, imax = 0u;
-        if (in_smem || mid) {
-            for (unsigned e = threadIdx.x; e < L; e += blockDim.x) cp_async8(s_keys + e, g + e);
-            for (int i = threadIdx.x; i < (1 << kBucketBits); i += blockDim.x) s_cnt[i] = 0u;  // bucket counts
-            asm volatile("cp.async.wait_all;" ::: "memory");
-            __syncthreads();
-        }
-        auto widen = [&](unsigned long long k) {
-            const unsigned d = (unsigned)(k >> 32), i = (unsigned)k;
-            dmin = min(dmin, d);
-            dmax = max(dmax, d);
-            imax = max(imax, i);
-        };
-        if (in_smem || mid)
-            for (unsigned e = threadIdx.x; e < L; e += blockDim.x) widen(s_keys[e]);
-        else
-            sweep(g, (int)L, widen);
-        for (int o = 16; o > 0; o >>= 1) {
-            dmin = min(dmin, __shfl_xor_sync(0xffffffffu, dmin, o));
-            dmax = max(dmax, __shfl_xor_sync(0xffffffffu, dmax, o));
-            imax = max(imax, __shfl_xor_sync(0xffffffffu, imax, o));
-        }
-        if ((threadIdx.x & 31) == 0) {
-            atomicMin(&s_dmin, dmin);
-            atomicMax(&s_dmax, dmax);
-            atomicMax(&s_imax, imax);
-        }
-        __syncthreads();
-        const unsigned d0 = s_dmin;
-        const int ib = 32 - __clz(s_imax);       // bits of the largest index (0 if 0)
-        const int db = 32 - __clz(s_dmax - d0);  // bits of the depth spread
-        unsigned long long *a = in_smem ? s_keys : c.keys2 + st;
-        unsigned long long *bb = in_smem ? s_keys + kRadixCap : c.keys + st;
-        // the radix passes take keys compressed to (depth - d0) << 32 | index (the order is the
-        // same); the bucket sort reads the keys as they are
-        auto compress = [&](unsigned long long *dst, const unsigned long long *src) {
-            for (unsigned e = threadIdx.x; e < L; e += blockDim.x) {
-                const unsigned long long k = src[e];
-                dst[e] = ((unsigned long long)((unsigned)(k >> 32) - d0) << 32) | (unsigned)k;
-            }
-            __syncthreads();
-        };
-        unsigned long long *res = nullptr;  // stays null when the keys' indices are already written
-        bool done = false;
-        if (mid) {
-            done = bucket_sort_pos(s_keys, (int)L, d0, db, s_cnt, s_rank_mid, s_pos_mid, &s_long, c.masked,
-                                   c.sorted + st, masks);
-            __syncthreads();  // every thread has read the flag before it is cleared
-            if (!done) {      // a crowded bucket: sort the segment in global memory below
-                if (threadIdx.x == 0) s_long = 0u;
-                __syncthreads();
-            }
-        } else if (!in_smem) {
-            done = bucket_sort_stream(g, c.keys2 + st, (int)L, d0, db, reinterpret_cast<unsigned *>(s_keys), s_cnt,
-                                      c.masked, c.sorted + st, masks);
-        }
-        if (done) {
+        const bool in_smem = L <= (unsigned)kSmemCap;
+        bool done;
+        if (L <= 4u * kSortThreads) {
+            done = bucket_sort<4, 12>(g, (int)L, s_keys, s_cnt, s_sum, &s_dmin, &s_dmax, c.masked, out, masks);
+        } else if (L <= 8u * kSortThreads) {
+            done = bucket_sort<8, 13>(g, (int)L, s_keys, s_cnt, s_sum, &s_dmin, &s_dmax, c.masked, out, masks);
         } else if (in_smem) {
-            res = bucket_sort(a, bb, (int)L, d0, db, s_cnt, s_rank, &s_long);
-            if (s_long) {  // a bucket too crowded for the fix-up: the full key by radix passes
-                compress(res, res);
-                unsigned long long *other = res == a ? bb : a;
-                res = radix_sort<true>(res, other, (int)L, 0, ib, s_cnt, s_rank);
-                other = res == a ? bb : a;
-                res = radix_sort<true>(res, other, (int)L, 32, 32 + db, s_cnt, s_rank);
-            }
+            done = bucket_sort<16, 14>(g, (int)L, s_keys, s_cnt, s_sum, &s_dmin, &s_dmax, c.masked, out, masks);
         } else {
-            // a crowded list of the position sort is still whole in shared memory; its place in
-            // global memory already holds some of its masks
-            compress(a, mid ? s_keys : g);
-            res = radix_sort<false>(a, bb, (int)L, 32, 32 + db, s_cnt, nullptr);
-            // ties: a run keeps its depth under any reordering, so run starts found by other
-            // threads do not change while a run is being ordered
-            for (unsigned e = threadIdx.x; e + 1 < L; e += blockDim.x) {
-                const unsigned dep = (unsigned)(res[e] >> 32);
-                if ((unsigned)(res[e + 1] >> 32) != dep || (e > 0 && (unsigned)(res[e - 1] >> 32) == dep))
-                    continue;
-                unsigned end = e + 2;
-                while (end < L && end - e <= (unsigned)kTieRun && (unsigned)(res[end] >> 32) == dep) ++end;
-                if (end - e > (unsigned)kTieRun) {
-                    s_long = 1u;
-                    continue;
-                }
-                for (unsigned i = e + 1; i < end; ++i) {
-                    const unsigned long long k = res[i];
-                    unsigned j = i;
-                    for (; j > e && res[j - 1] > k; --j) res[j] = res[j - 1];
-                    res[j] = k;
-                }
+            unsigned dmin = 0xffffffffu, dmax = 0u;
+            sweep(g, (int)L, [&](unsigned long long k) {
+                dmin = min(dmin, (unsigned)(k >> 32));
+                dmax = max(dmax, (unsigned)(k >> 32));
+            });
+            dmin = __reduce_min_sync(0xffffffffu, dmin);
+            dmax = __reduce_max_sync(0xffffffffu, dmax);
+            if ((threadIdx.x & 31) == 0) {
+                atomicMin(&s_dmin, dmin);
+                atomicMax(&s_dmax, dmax);
             }
             __syncthreads();
-            if (s_long) {
-                unsigned long long *other = res == a ? bb : a;
-                res = radix_sort<false>(res, other, (int)L, 0, ib, s_cnt, nullptr);
-                other = res == a ? bb : a;
-                res = radix_sort<false>(res, other, (int)L, 32, 32 + db, s_cnt, nullptr);
+            done = bucket_sort_stream(g, c.keys2 + st, (int)L, s_dmin, 32 - __clz(s_dmax - s_dmin),
+                                      reinterpret_cast<unsigned *>(s_keys), s_sum, c.masked, out, masks);
+        }
+        if (!done) {  // a crowded bucket; the keys at g are untouched and s_dmin, s_dmax set
+            unsigned imax = 0u;
+            sweep(g, (int)L, [&](unsigned long long k) { imax = max(imax, (unsigned)k); });
+            imax = __reduce_max_sync(0xffffffffu, imax);
+            if ((threadIdx.x & 31) == 0) atomicMax(&s_imax, imax);
+            const unsigned d0 = s_dmin;
+            const int db = 32 - __clz(s_dmax - d0);  // bits of the depth spread
+            const bool radix_smem = L <= (unsigned)kRadixCap;
+            unsigned long long *a = radix_smem ? s_keys : c.keys2 + st, *bb = radix_smem ? s_keys + kRadixCap : c.keys + st;
+            unsigned short *rank = reinterpret_cast<unsigned short *>(s_keys + 2 * kRadixCap);
+            unsigned *cnt = reinterpret_cast<unsigned *>(rank + kRadixCap);
+            for (unsigned e = threadIdx.x; e < L; e += blockDim.x) {
+                const unsigned long long k = g[e];
+                a[e] = ((unsigned long long)((unsigned)(k >> 32) - d0) << 32) | (unsigned)k;
             }
-        }
-        if (res == g) {  // the masks go over this buffer: finish from the other one
-            for (unsigned e = threadIdx.x; e < L; e += blockDim.x) a[e] = res[e];
             __syncthreads();
-            res = a;
-        }
-        if (res)
+            const int ib = 32 - __clz(s_imax);  // bits of the largest index (0 if 0)
+            unsigned long long *res;
+            if (radix_smem) {
+                res = radix_sort<true>(a, bb, (int)L, 0, ib, cnt, rank);
+                res = radix_sort<true>(res, res == a ? bb : a, (int)L, 32, 32 + db, cnt, rank);
+            } else {
+                res = radix_sort<false>(a, bb, (int)L, 32, 32 + db, cnt, nullptr);
+                // ties: a run keeps its depth under any reordering, so run starts found by other
+                // threads do not change while a run is being ordered
+                for (unsigned e = threadIdx.x; e + 1 < L; e += blockDim.x) {
+                    const unsigned dep = (unsigned)(res[e] >> 32);
+                    if ((unsigned)(res[e + 1] >> 32) != dep || (e > 0 && (unsigned)(res[e - 1] >> 32) == dep))
+                        continue;
+                    unsigned end = e + 2;
+                    while (end < L && end - e <= (unsigned)kTieRun && (unsigned)(res[end] >> 32) == dep) ++end;
+                    if (end - e > (unsigned)kTieRun) {
+                        s_long = 1u;
+                        continue;
+                    }
+                    for (unsigned i = e + 1; i < end; ++i) {
+                        const unsigned long long k = res[i];
+                        unsigned j = i;
+                        for (; j > e && res[j - 1] > k; --j) res[j] = res[j - 1];
+                        res[j] = k;
+                    }
+                }
+                __syncthreads();
+                if (s_long) {
+                    unsigned long long *other = res == a ? bb : a;
+                    res = radix_sort<false>(res, other, (int)L, 0, ib, cnt, nullptr);
+                    other = res == a ? bb : a;
+                    res = radix_sort<false>(res, other, (int)L, 32, 32 + db, cnt, nullptr);
+                }
+            }
+            if (res == g) {  // the masks go over this buffer: finish from the other one
+                for (unsigned e = threadIdx.x; e < L; e += blockDim.x) a[e] = res[e];
+                __syncthreads();
+                res = a;
+            }
             for (unsigned e = threadIdx.x; e < L; e += blockDim.x) {
                 const unsigned low = (unsigned)res[e];
-                c.sorted[st + e] = low_index(c.masked, low);
+                out[e] = low_index(c.masked, low);
                 masks[e] = low_mask(c.masked, low);
             }
+        }
         __syncthreads();
         if (threadIdx.x == 0) {
             s_cur = w1 < n_work ? 1u : 0u;
@@ -851,8 +793,7 @@ cudaError_t launch_scatter(const Ctx &c, int max_n, cudaStream_t s) {
 
 cudaError_t launch_tile_sort(const Ctx &c, int sms, cudaStream_t s) {
     static int attr_device = -1, per_sm = 1;
-    const int smem = 2 * kRadixCap * (int)sizeof(unsigned long long) + kRadixCap * (int)sizeof(unsigned short) +
-                     (kSortWarps * 256 + kSortWarps) * 4;
+    const int smem = kSortSmem;
     int dev = 0;
     cudaError_t e = cudaGetDevice(&dev);
     if (e != cudaSuccess) return e;
