@@ -35,7 +35,7 @@ struct Plan {
     std::vector<FrameInfo> frames;
     std::vector<int> mframes;
     Layout L{};
-    int max_n = 0, max_k = 1, max_chunks = 0, max_nb = 0;
+    int max_n = 0, max_k = 1, max_chunks = 0, max_nb = 0, max_tiles = 0;
 };
 
 // Host-side checks and tables; sizes of everything except the pair buffers.
@@ -116,6 +116,7 @@ int make_plan(const rgba_batch *b, Plan &p) {
         fi.H = fr.height;
         fi.tiles_x = (fr.width + tw - 1) / tw;
         fi.tiles_y = (fr.height + th - 1) / th;
+        p.max_tiles = std::max(p.max_tiles, fi.tiles_x * fi.tiles_y);
         fi.tile_base = (int)T;
         fi.rec_base = (int)R;
         fi.n = mi.n;
@@ -164,16 +165,15 @@ int make_plan(const rgba_batch *b, Plan &p) {
     L.models = take(sizeof(ModelInfo) * (size_t)M);
     L.frames = take(sizeof(FrameInfo) * (size_t)B);
     L.mframes = take(sizeof(int) * (size_t)B);
-    L.tile_count = take((size_t)tc_bytes(T));
+    L.tile_count = take(4 * (size_t)T);
     L.tile_start = take(4 * (size_t)(T + 1));
-    L.cursor = take(4 * (size_t)T * kSubCounters);
+    L.cursor = take(4 * (size_t)T);
     L.work = take(4 * (size_t)T);
     L.scan_aux = take(scan_aux_bytes(T));
     L.records = take(sizeof(float) * kRecFloats * (size_t)R);
     L.rects = take(8 * (size_t)R);
     L.cache = take(sizeof(float) * kCacheFloats * (size_t)R);
     L.grad2d = take(sizeof(float) * kG2Floats * (size_t)R);
-    L.ranks = take(4 * kRankSlots * (size_t)R);
     L.depth = take(4 * (size_t)R);
     L.pix_T = take(4 * (size_t)P);
     L.pix_n = take(4 * (size_t)P);
@@ -218,7 +218,6 @@ Ctx make_ctx(const Layout &L, unsigned char *ws, const rgba_batch *b) {
     c.grad_psi = b->grad_psi;
     c.cnt = reinterpret_cast<Counters *>(ws + L.counters);
     c.tile_count = reinterpret_cast<unsigned *>(ws + L.tile_count);
-    c.tc_mask = (unsigned)(tc_pow2(L.T) - 1);
     c.tile_start = reinterpret_cast<unsigned *>(ws + L.tile_start);
     c.cursor = reinterpret_cast<unsigned *>(ws + L.cursor);
     c.work = reinterpret_cast<unsigned *>(ws + L.work);
@@ -231,7 +230,6 @@ Ctx make_ctx(const Layout &L, unsigned char *ws, const rgba_batch *b) {
     c.keys2 = reinterpret_cast<unsigned long long *>(ws + L.keys2);
     c.sorted = reinterpret_cast<unsigned *>(ws + L.sorted);
     c.dpsi_part = reinterpret_cast<float *>(ws + L.dpsi_part);
-    c.ranks = reinterpret_cast<unsigned *>(ws + L.ranks);
     c.depth = reinterpret_cast<float *>(ws + L.depth);
     c.R = L.R;
     c.T = L.T;
@@ -322,7 +320,7 @@ int memset_async(void *p, size_t bytes, cudaStream_t s, const char *what) {
 
 int do_preprocess(rgba_ctx_t ctx, Call &k) {
     int rc;
-    const size_t count_bytes = (size_t)tc_bytes(k.p.L.T);
+    const size_t count_bytes = 4 * (size_t)k.p.L.T;
     {  // tables, counters and tile counts in one launch when the tables fit its parameters
         const Layout &L = k.p.L;
         PrologueArgs a{};
@@ -366,12 +364,13 @@ int do_preprocess(rgba_ctx_t ctx, Call &k) {
 int do_bin_sort(rgba_ctx_t ctx, Call &k) {
     cudaError_t e;
     {
-        StageScope sc(ctx, ST_SCAN, k.s, 3);
+        StageScope sc(ctx, ST_SCAN, k.s, 4);
+        if ((e = launch_count(k.c, k.p.max_n, k.p.max_tiles, k.s)) != cudaSuccess) return cuda_fail(e, "count");
         if ((e = launch_scan(k.c, k.s)) != cudaSuccess) return cuda_fail(e, "scan");
     }
     {
         StageScope sc(ctx, ST_SCATTER, k.s, 1);
-        if ((e = launch_scatter(k.c, k.p.max_n, k.s)) != cudaSuccess) return cuda_fail(e, "scatter");
+        if ((e = launch_scatter(k.c, k.p.max_n, k.p.max_tiles, k.s)) != cudaSuccess) return cuda_fail(e, "scatter");
     }
     StageScope sc(ctx, ST_SORT, k.s, 1);
     if ((e = launch_tile_sort(k.c, ctx->sms, k.s)) != cudaSuccess) return cuda_fail(e, "tile sort");

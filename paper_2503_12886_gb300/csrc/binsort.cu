@@ -2,17 +2,16 @@
 // the paper's renderer inherits it from 3DGS): every kept Gaussian is listed in every screen
 // tile of its rectangle and each (frame, tile) list is ordered by (depth bits, Gaussian index).
 //
-// Design: the per-tile counts come out of the preprocess kernel (atomics whose return values
-// give each Gaussian its slot in up to 8 tiles), a three-phase scan (per-CTA partials, one CTA
-// over the partials, per-CTA writes) turns them into list offsets and a work list, a scatter
+// Design: a kernel counts the rectangles' tiles, a three-phase scan (per-CTA
+// partials, one CTA over the partials, per-CTA writes) turns the counts into list offsets and a work list, a scatter
 // kernel drops (depth << 32 | index) keys, with a mask of the pixel blocks each splat reaches in
-// the low byte of the index word, into their tile's segment (by
-// slot, or by a cursor atomic for larger rectangles), and one CTA per non-empty tile sorts its
-// list: in shared memory by
-// one bucket pass on the top depth bits and a placement of every key by its rank in its bucket,
+// the low byte of the index word, into their tile's segment, and
+// one CTA per non-empty tile sorts its list: in shared memory by one bucket pass on the top depth bits and a placement of every key by its rank in its bucket,
 // or, for long segments, by the same bucket pass with the keys in L2; buckets too crowded for it
 // fall back to a stable LSD radix sort of the keys compressed to (depth - segment minimum) << 32 |
 // index. Because the key carries the index, the result is unique.
+#include <algorithm>
+
 #include "reach.cuh"
 #include "rgba_internal.cuh"
 
@@ -86,8 +85,60 @@ __device__ __forceinline__ ScanAux scan_aux(const Ctx &c) {
 
 __device__ __forceinline__ unsigned bucket_of(unsigned v) { return 31u - __clz(v); }
 
-// Phase 1, one thread per tile: the tile's total count (ranked slots plus sub-counters) into
-// tile_start, each sub-counter's fill offset into cursor, and per CTA the sum, the number of
+// Counting and scattering take one (frame, Gaussian) per thread and give each CTA a piece of one frame. Its
+// touches of tiles are counted in shared memory, one counter per tile of the frame, and each tile a CTA
+// touched then costs one global atomic: 16 frames of 60,000 Gaussians make 3.3 M touches, mostly of a few
+// hundred tiles, and a global atomic per touch (returning the places, in the preprocess, or counting there
+// and taking the places here) made the L2's atomic units and the wait for them the bound. Projection, count,
+// scan and scatter together, one atomic per touch in the projection, then this: 16 frames 148 -> 125 us, ten frames
+// 112 -> 87, 64 frames of eight avatars 661 -> 535, 15 frames of five 275 -> 220, one frame 60 -> 53. Frames of more
+// than kHistTiles tiles (1,773 pixels square) go touch by touch.
+constexpr int kBinThreads = 256;
+constexpr int kHistTiles = 12288;
+
+// The CTA's frame and Gaussian. Neighbouring CTAs take different frames, so that the atomics under way
+// spread over all frames' tiles.
+struct BinItem {
+    FrameInfo f;
+    int i, tiles;
+    bool valid, hist;
+};
+__device__ __forceinline__ BinItem bin_item(const Ctx &c) {
+    BinItem b;
+    b.f = c.frames[blockIdx.x];
+    b.i = (int)((blockIdx.y + blockIdx.z * gridDim.y) * kBinThreads + threadIdx.x);
+    b.tiles = b.f.tiles_x * b.f.tiles_y;
+    b.valid = b.i < b.f.n;
+    b.hist = b.tiles <= kHistTiles;
+    return b;
+}
+
+template <typename F>
+__device__ __forceinline__ void each_tile(const ushort4 &rc, int tiles_x, F f) {
+    for (int ty = rc.y; ty < rc.w; ++ty)
+        for (int tx = rc.x; tx < rc.z; ++tx) f(ty * tiles_x + tx);
+}
+
+__global__ void __launch_bounds__(kBinThreads) k_count(Ctx c) {
+    extern __shared__ unsigned s_hist[];
+    pdl_enter();
+    const BinItem b = bin_item(c);
+    if (b.i - (int)threadIdx.x >= b.f.n || b.i < 0) return;  // the whole CTA
+    const ushort4 rc = b.valid ? c.rects[b.f.rec_base + b.i] : make_ushort4(0, 0, 0, 0);
+    unsigned *count = c.tile_count + b.f.tile_base;
+    if (!b.hist) {
+        each_tile(rc, b.f.tiles_x, [&](int t) { atomicAdd(count + t, 1u); });
+        return;
+    }
+    for (int t = threadIdx.x; t < b.tiles; t += kBinThreads) s_hist[t] = 0u;
+    __syncthreads();
+    each_tile(rc, b.f.tiles_x, [&](int t) { atomicAdd(s_hist + t, 1u); });
+    __syncthreads();
+    for (int t = threadIdx.x; t < b.tiles; t += kBinThreads)
+        if (s_hist[t]) atomicAdd(count + t, s_hist[t]);
+}
+
+// Phase 1, one thread per tile: the tile's total count into tile_start, and per CTA the sum, the number of
 // non-empty tiles and the histogram of floor(log2(length)).
 __global__ void __launch_bounds__(kScanTile) k_scan_blocks(Ctx c) {
     __shared__ unsigned s_hist[32];
@@ -98,13 +149,7 @@ __global__ void __launch_bounds__(kScanTile) k_scan_blocks(Ctx c) {
     const long long t = (long long)blockIdx.x * kScanTile + threadIdx.x;
     unsigned v = 0;
     if (t < c.T) {
-        const unsigned *sub = c.tile_count + tc_sub_base(c.tc_mask) + t * kSubCounters;
-        v = c.tile_count[tc_word(c.tc_mask, t)];
-#pragma unroll
-        for (int q = 0; q < kSubCounters; ++q) {
-            c.cursor[t * kSubCounters + q] = v;
-            v += sub[q];
-        }
+        v = c.tile_count[t];
         c.tile_start[t] = v;
         if (v) atomicAdd(&s_hist[bucket_of(v)], 1u);
     }
@@ -173,8 +218,8 @@ __global__ void __launch_bounds__(kScanTile) k_scan_top(Ctx c) {
     }
 }
 
-// Phase 3, one thread per tile: the list start (exclusive scan of the totals) and the tile's
-// place in the work list: non-empty tiles by bucket, longest bucket first (in any order within
+// Phase 3, one thread per tile: the list start (exclusive scan of the totals), also as the scatter's
+// cursor, and the tile's place in the work list: non-empty tiles by bucket, longest bucket first (in any order within
 // a bucket), then the empty tiles in tile order.
 __global__ void __launch_bounds__(kScanTile) k_scan_write(Ctx c) {
     __shared__ unsigned s_off[32];
@@ -192,6 +237,7 @@ __global__ void __launch_bounds__(kScanTile) k_scan_write(Ctx c) {
         c.tile_start[t] = st > 0xffffffffull ? 0xffffffffu : (unsigned)st;
         if (v) {
             c.work[atomicAdd(&s_off[bucket_of(v)], 1u)] = (unsigned)t;
+            c.cursor[t] = (unsigned)st;  // meaningless past 2^32 pairs, and then unused
         } else {
             // empty tiles before this CTA: its first tile index minus the non-empty ones
             const unsigned e0 = (unsigned)((long long)blockIdx.x * kScanTile) - a.bne[blockIdx.x];
@@ -200,52 +246,41 @@ __global__ void __launch_bounds__(kScanTile) k_scan_write(Ctx c) {
     }
 }
 
-constexpr int kScatterThreads = 128;
-
 // One thread per (frame, Gaussian): drops its key into the list of every tile of its rectangle,
 // with the tile's block mask. The masks cost one ellipse extent per four pixel rows of the
 // rectangle and two compares per block; computed here they are paid once per (Gaussian, tile),
 // where every compositing warp of a tile (eight, forwards and again backwards) would test every
 // entry of its list. TW: the tile width (16 or 8).
+// In shared memory the counts of the CTA's touches become, with one global atomic per touched tile, the
+// places its keys take in the lists.
 template <int TW>
-__global__ void __launch_bounds__(kScatterThreads) k_scatter(Ctx c) {
+__global__ void __launch_bounds__(kBinThreads) k_scatter(Ctx c) {
+    extern __shared__ unsigned s_hist[];
     constexpr int TH = kTilePix / TW, NBX = TW / 8, BANDS = TH / 4;
     pdl_enter();
     if (c.cnt->overflow) return;
-    const int b = blockIdx.y;
-    const FrameInfo f = c.frames[b];
-    const int i = blockIdx.x * blockDim.x + threadIdx.x;
-    if (i >= f.n) return;
-    const long long r = f.rec_base + i;
+    const BinItem b = bin_item(c);
+    if (b.i - (int)threadIdx.x >= b.f.n || b.i < 0) return;  // the whole CTA
+    const FrameInfo &f = b.f;
+    const long long r = f.rec_base + (b.valid ? b.i : 0);
     // every load of the record at once (few Gaussians are culled)
-    const ushort4 rc = c.rects[r];
+    ushort4 rc = c.rects[r];
     const unsigned bits = __float_as_uint(c.depth[r]);
     const float4 r0 = c.records[r * 3];
     const float2 r1 = *reinterpret_cast<const float2 *>(c.records + r * 3 + 1);
-    const uint4 *rp = reinterpret_cast<const uint4 *>(c.ranks + r * kRankSlots);
-    const uint4 q0 = rp[0], q1 = rp[1];
-    if (rc.z <= rc.x || rc.w <= rc.y) return;
-    const int w = rc.z - rc.x, area = w * (rc.w - rc.y);
-    const bool ranked = area <= kRankSlots;  // slots recorded by the preprocess: no atomics
-    unsigned rk[kRankSlots] = {q0.x, q0.y, q0.z, q0.w, q1.x, q1.y, q1.z, q1.w};
-    const unsigned *ts = c.tile_start + f.tile_base;
-    if (ranked) {  // every list start in flight while the masks are computed
-        const unsigned *t0 = ts + (long long)rc.y * f.tiles_x + rc.x;
-        int ox = 0, off = 0;  // slot q is tile (rc.x + ox, rc.y + q / w), off its offset from t0
-#pragma unroll
-        for (int q = 0; q < kRankSlots; ++q) {
-            if (q < area) {
-                rk[q] += __ldg(t0 + off);
-                ++off;
-                if (++ox == w) {
-                    ox = 0;
-                    off += f.tiles_x - w;
-                }
-            }
-        }
+    if (!b.valid) rc = make_ushort4(0, 0, 0, 0);
+    unsigned *cur = c.cursor + f.tile_base;
+    if (b.hist) {
+        for (int t = threadIdx.x; t < b.tiles; t += kBinThreads) s_hist[t] = 0u;
+        __syncthreads();
+        each_tile(rc, f.tiles_x, [&](int t) { atomicAdd(s_hist + t, 1u); });
+        __syncthreads();
+        for (int t = threadIdx.x; t < b.tiles; t += kBinThreads)
+            if (s_hist[t]) s_hist[t] = atomicAdd(cur + t, s_hist[t]);
+        __syncthreads();
     }
+    if (rc.z <= rc.x || rc.w <= rc.y) return;
     const Reach e = reach_of(r0, r1);
-    unsigned *cur = c.cursor + (size_t)f.tile_base * kSubCounters + (r & (kSubCounters - 1));
     for (int ty = rc.y; ty < rc.w; ++ty) {
         float xl[BANDS], xr[BANDS];
 #pragma unroll
@@ -261,16 +296,9 @@ __global__ void __launch_bounds__(kScatterThreads) k_scatter(Ctx c) {
                 }
             if (e.all) mask = 0xffu;
             if (e.none) mask = 0u;
-            const long long t = (long long)ty * f.tiles_x + tx;
-            unsigned pos;
-            if (ranked) {  // the slots in tile order: take the first, move the others up
-                pos = rk[0];
-#pragma unroll
-                for (int q = 0; q + 1 < kRankSlots; ++q) rk[q] = rk[q + 1];
-            } else {
-                pos = ts[t] + atomicAdd(cur + t * kSubCounters, 1u);
-            }
-            c.keys[pos] = ((unsigned long long)bits << 32) | pack_low(c.masked, (unsigned)i, mask);
+            const int t = ty * f.tiles_x + tx;
+            const unsigned pos = b.hist ? atomicAdd(s_hist + t, 1u) : atomicAdd(cur + t, 1u);
+            c.keys[pos] = ((unsigned long long)bits << 32) | pack_low(c.masked, (unsigned)b.i, mask);
         }
     }
 }
@@ -785,10 +813,23 @@ size_t scan_aux_bytes(long long T) {
     return (size_t)nb * 8 + (size_t)nb * 4 + (size_t)nb * 32 * 4 + 32 * 4;
 }
 
-cudaError_t launch_scatter(const Ctx &c, int max_n, cudaStream_t s) {
+namespace {
+dim3 bin_grid(const Ctx &c, int max_n) {
+    const unsigned chunks = (unsigned)(max_n - 1) / kBinThreads + 1, z = (chunks - 1) / 65535u + 1;
+    return dim3((unsigned)c.B, (chunks - 1) / z + 1, z);
+}
+size_t bin_smem(int max_tiles) { return 4 * (size_t)std::min(max_tiles, kHistTiles); }
+}  // namespace
+
+cudaError_t launch_count(const Ctx &c, int max_n, int max_tiles, cudaStream_t s) {
     if (c.B == 0 || max_n == 0) return cudaSuccess;
-    dim3 grid((max_n + kScatterThreads - 1) / kScatterThreads, c.B);
-    return launch_pdl(c.tw == 16 ? k_scatter<16> : k_scatter<8>, grid, dim3(kScatterThreads), 0, s, c);
+    return launch_pdl(k_count, bin_grid(c, max_n), dim3(kBinThreads), bin_smem(max_tiles), s, c);
+}
+
+cudaError_t launch_scatter(const Ctx &c, int max_n, int max_tiles, cudaStream_t s) {
+    if (c.B == 0 || max_n == 0) return cudaSuccess;
+    return launch_pdl(c.tw == 16 ? k_scatter<16> : k_scatter<8>, bin_grid(c, max_n), dim3(kBinThreads),
+                      bin_smem(max_tiles), s, c);
 }
 
 cudaError_t launch_tile_sort(const Ctx &c, int sms, cudaStream_t s) {

@@ -1,4 +1,4 @@
-// Fused blend + activation + EWA projection + tile binning count (the "preprocess" stage of
+// Fused blend + activation + EWA projection + tile rectangles (the "preprocess" stage of
 // the batch-parallel rasterizer, RGBAvatar Sec. 3.2 / Supp. A.3, built on 3DGS), and the
 // standalone Eq. 1 blend.
 //
@@ -155,8 +155,7 @@ __device__ __forceinline__ float sigmoid_spec(float x) { return fdiv(1.0f, fadd(
 
 // The FP32 decision spec for one (frame, Gaussian) from its blended channels v and activated
 // opacity op: view transform, activations, EWA covariance, conic, radius, tile rectangle, depth.
-// Writes the render record, the rectangle and the backward cache, and counts the Gaussian in
-// every tile it touches.
+// Writes the render record, the rectangle and the backward cache.
 __device__ __forceinline__ void decide_and_write(const Ctx &c, const ModelInfo &m, const FrameConst &f,
                                                  const float *V, const float v[kNch], float op, int i,
                                                  long long r) {
@@ -299,34 +298,6 @@ __device__ __forceinline__ void decide_and_write(const Ctx &c, const ModelInfo &
         r1 = make_float4(cc, op, v[11], v[12]);
         r2 = make_float4(v[13], p[2], 0.f, 0.f);
         rc = make_ushort4((unsigned short)ix0, (unsigned short)iy0, (unsigned short)ix1, (unsigned short)iy1);
-        // count the Gaussian in every tile of its rectangle; for rectangles of up to kRankSlots
-        // tiles keep the slot each count returns, so the scatter needs no atomics
-        const int rw = ix1 - ix0, area = rw * (iy1 - iy0);
-        if (area <= kRankSlots) {
-            const long long t0 = (long long)f.tile_base + iy0 * f.tiles_x + ix0;
-            unsigned rk[kRankSlots];
-            int ox = 0, off = 0;  // slot q is tile (ix0 + ox, iy0 + q / rw), off its offset from t0
-#pragma unroll
-            for (int q = 0; q < kRankSlots; ++q) {
-                rk[q] = 0u;
-                if (q < area) {
-                    rk[q] = atomicAdd(c.tile_count + tc_word(c.tc_mask, t0 + off), 1u);
-                    ++off;
-                    if (++ox == rw) {
-                        ox = 0;
-                        off += f.tiles_x - rw;
-                    }
-                }
-            }
-            uint4 *rp = reinterpret_cast<uint4 *>(c.ranks + r * kRankSlots);
-            rp[0] = make_uint4(rk[0], rk[1], rk[2], rk[3]);
-            rp[1] = make_uint4(rk[4], rk[5], rk[6], rk[7]);
-        } else {  // spread over kSubCounters counters per tile, chosen by the Gaussian index
-            unsigned *tb = c.tile_count + tc_sub_base(c.tc_mask) + (size_t)f.tile_base * kSubCounters +
-                           (r & (kSubCounters - 1));
-            for (int ty = iy0; ty < iy1; ++ty)
-                for (int tx = ix0; tx < ix1; ++tx) atomicAdd(tb + (size_t)(ty * f.tiles_x + tx) * kSubCounters, 1u);
-        }
     } while (0);
     c.records[r * 3 + 0] = r0;
     c.records[r * 3 + 1] = r1;

@@ -37,28 +37,6 @@ constexpr int kCacheFloats = 12; // backward cache: mean(3), quat(4), log-scale(
 constexpr int kG2Floats = 12;    // 2-D gradient: du, dv, da, db, dc, dopacity, dr, dg, db, -
 constexpr int kTilePix = 256;    // pixels per screen tile (16x16 or 8x32)
 constexpr int kBwdChunk = 32;    // Gaussians per CTA in the fused preprocess/blend backward
-constexpr int kRankSlots = 8;    // tiles per Gaussian whose in-tile slot preprocess records
-constexpr int kSubCounters = 8;  // per-tile counters for larger rectangles (by Gaussian index)
-// The per-tile counts of the preprocess take millions of atomics on the few thousand counters of
-// the tiles a face covers. Stored side by side, those counters share a few L2 slices, whose
-// atomic units then set the preprocess's pace (it varied by 30 % with the counters' offset). So
-// each tile's ranked count has its own 32-byte sector, at a slot given by an odd multiplier
-// modulo a power of two (Knuth's multiplicative hashing with the golden-ratio constant: a
-// bijection that scatters neighbouring tiles), and the sub-counters follow the slots.
-constexpr int kTcWords = 8;
-__host__ __device__ inline long long tc_pow2(long long T) {
-    long long p = 1;
-    while (p < T) p <<= 1;
-    return p;
-}
-__host__ __device__ inline long long tc_word(unsigned mask, long long t) {
-    return (long long)kTcWords * (long long)(((unsigned)t * 0x9E3779B1u) & mask);
-}
-__host__ __device__ inline long long tc_sub_base(unsigned mask) { return (long long)kTcWords * ((long long)mask + 1); }
-__host__ __device__ inline long long tc_bytes(long long T) {
-    return 4 * ((long long)kTcWords * tc_pow2(T) + T * kSubCounters);
-}
-
 // Per-model table (device copy in the workspace).
 struct ModelInfo {
     const float *g0;
@@ -112,7 +90,7 @@ static_assert(sizeof(Counters) <= 256, "counters fit in one 256-byte block");
 
 struct Layout {
     size_t counters, models, frames, mframes, tile_count, tile_start, cursor, work;
-    size_t records, rects, cache, grad2d, ranks, depth, pix_T, pix_n, pix_dl, pix_img, dpsi_part;
+    size_t records, rects, cache, grad2d, depth, pix_T, pix_n, pix_dl, pix_img, dpsi_part;
     size_t keys, keys2, sorted, scan_aux, total;
     long long R, T, P;     // records, tiles, pixels
     long long dpsi_floats;
@@ -153,10 +131,9 @@ struct Ctx {
     float *grad_psi;
     float *grad_blended;   // [sum over frames of 14 n_pad] or nullptr: dL/dG^psi_b per frame
     Counters *cnt;
-    unsigned *tile_count;  // ranked counts (<= kRankSlots tiles; at tc_word), then [T][kSubCounters] the others
-    unsigned tc_mask;      // tc_pow2(T) - 1: the ranked counts' slot hash range
+    unsigned *tile_count;  // [T]: list lengths
     unsigned *tile_start;
-    unsigned *cursor;      // [T][kSubCounters]: fill positions of the larger rectangles
+    unsigned *cursor;      // [T]: the next free entry of each list while the scatter fills it
     unsigned *work;
     unsigned char *scan_aux;  // the tile scan's per-CTA partials
     float4 *records;   // [R][3]
@@ -169,7 +146,6 @@ struct Ctx {
     // keys carry a pixel-block mask (pack_low): every model has at most kMaskedN Gaussians
     bool masked;
     float *dpsi_part;
-    unsigned *ranks;   // [R][kRankSlots]: slot of the Gaussian in each tile of its rectangle
     float *depth;      // [R]: view-space depth of each kept record (the scatter's sort key)
     long long R, T, cap;
     int B, M, k_stride, tw, th;
@@ -233,14 +209,16 @@ struct PrologueArgs {
     long long zero_b16;
 };
 cudaError_t launch_prologue(const PrologueArgs &a, const void *const src[3], cudaStream_t s);
-// common_mask: the channel mask every model of the batch shares (0 when they differ); the two
-// masks of the RGBA_MASK_* constants run a blend specialised at compile time.
+// common_mask: the channel mask every model of the
+// batch shares (0 when they differ); the two masks of the RGBA_MASK_* constants run a blend specialised at compile time.
 cudaError_t launch_preprocess(const Ctx &c, int max_n, int max_k, int max_rows, unsigned common_mask,
                               cudaStream_t s);
 cudaError_t launch_blend(const Ctx &c, int max_n, float *out, cudaStream_t s);
+// max_tiles: the most tiles of any frame of the batch
+cudaError_t launch_count(const Ctx &c, int max_n, int max_tiles, cudaStream_t s);
 cudaError_t launch_scan(const Ctx &c, cudaStream_t s);
 size_t scan_aux_bytes(long long T);
-cudaError_t launch_scatter(const Ctx &c, int max_n, cudaStream_t s);
+cudaError_t launch_scatter(const Ctx &c, int max_n, int max_tiles, cudaStream_t s);
 cudaError_t launch_tile_sort(const Ctx &c, int sms, cudaStream_t s);
 // stats: run the counting instance (16 x 16 tiles, 64-entry staging only), which adds the
 // compositing statistics of Counters
