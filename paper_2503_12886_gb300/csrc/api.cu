@@ -318,8 +318,10 @@ int memset_async(void *p, size_t bytes, cudaStream_t s, const char *what) {
 
 
 
-int do_preprocess(rgba_ctx_t ctx, Call &k) {
+// zero_g2: a compositing pass of the same call adds to the 2-D gradient slots
+int do_preprocess(rgba_ctx_t ctx, Call &k, bool zero_g2) {
     int rc;
+    k.c.zero_g2 = zero_g2;
     const size_t count_bytes = 4 * (size_t)k.p.L.T;
     {  // tables, counters and tile counts in one launch when the tables fit its parameters
         const Layout &L = k.p.L;
@@ -357,7 +359,7 @@ int do_preprocess(rgba_ctx_t ctx, Call &k) {
         max_rows = std::max(max_rows, kNch + m.k * m.A);
         if (m.mask != common_mask) common_mask = 0u;
     }
-    cudaError_t e = launch_preprocess(k.c, k.p.max_n, k.p.max_k, max_rows, common_mask, k.s);
+    cudaError_t e = launch_preprocess(k.c, k.p.max_n, k.p.max_nb, k.p.max_k, max_rows, common_mask, k.s);
     return e == cudaSuccess ? RGBA_OK : cuda_fail(e, "preprocess");
 }
 
@@ -583,7 +585,7 @@ int rgba_preprocess(rgba_ctx_t ctx, const rgba_batch *batch, void *ws, size_t ws
     Call k;
     int rc = prologue(ctx, batch, ws, ws_bytes, stream, k);
     if (rc || k.p.L.B == 0) return rc;
-    return do_preprocess(ctx, k);
+    return do_preprocess(ctx, k, false);
 }
 
 int rgba_bin_sort(rgba_ctx_t ctx, const rgba_batch *batch, void *ws, size_t ws_bytes, void *stream) {
@@ -647,7 +649,7 @@ int rgba_step_async(rgba_ctx_t ctx, const rgba_batch *batch, void *ws, size_t ws
     float *im = img ? img : reinterpret_cast<float *>(k.ws + L.pix_img);
     float *T = reinterpret_cast<float *>(k.ws + L.pix_T);
     int *n = reinterpret_cast<int *>(k.ws + L.pix_n);
-    if ((rc = do_preprocess(ctx, k))) return rc;
+    if ((rc = do_preprocess(ctx, k, true))) return rc;
     if ((rc = do_bin_sort(ctx, k))) return rc;
     return do_render_step(ctx, k, im, T, n, target, loss_kind);
 }
@@ -687,7 +689,7 @@ int rgba_step_adam_async(rgba_ctx_t ctx, const rgba_batch *batch, void *ws, size
     float *im = img ? img : reinterpret_cast<float *>(k.ws + L.pix_img);
     float *T = reinterpret_cast<float *>(k.ws + L.pix_T);
     int *n = reinterpret_cast<int *>(k.ws + L.pix_n);
-    if ((rc = do_preprocess(ctx, k))) return rc;
+    if ((rc = do_preprocess(ctx, k, true))) return rc;
     if ((rc = do_bin_sort(ctx, k))) return rc;
     return do_render_step(ctx, k, im, T, n, target, loss_kind, &fa);
 }
@@ -875,7 +877,7 @@ int rgba_color_init(rgba_ctx_t ctx, const rgba_batch *batch, void *ws, size_t ws
     if (!target || !done) return fail(RGBA_ERR_INVALID_ARG, "target/done is NULL");
     if (!(delta >= 0.f)) return fail(RGBA_ERR_INVALID_ARG, "delta must be >= 0");
     const Layout &L = k.p.L;
-    if ((rc = do_preprocess(ctx, k))) return rc;
+    if ((rc = do_preprocess(ctx, k, true))) return rc;
     if ((rc = do_bin_sort(ctx, k))) return rc;
     // the accumulators (the records' 2-D gradient slots) were zeroed by the preprocess
     if ((rc = do_render_fwd(ctx, k, reinterpret_cast<float *>(k.ws + L.pix_img), reinterpret_cast<float *>(k.ws + L.pix_T),

@@ -1,4 +1,4 @@
-// Fused blend + activation + EWA projection + tile rectangles (the "preprocess" stage of
+// Fused blend + activation + EWA projection + tile binning count (the "preprocess" stage of
 // the batch-parallel rasterizer, RGBAvatar Sec. 3.2 / Supp. A.3, built on 3DGS), and the
 // standalone Eq. 1 blend.
 //
@@ -161,7 +161,7 @@ __device__ __forceinline__ void decide_and_write(const Ctx &c, const ModelInfo &
                                                  long long r) {
     c.cache[r * 3 + 0] = make_float4(v[0], v[1], v[2], v[3]);
     c.cache[r * 3 + 1] = make_float4(v[4], v[5], v[6], v[7]);
-    {  // the record's 2-D gradient slots start at zero for the compositing backward's atomics
+    if (c.zero_g2) {  // the record's 2-D gradient slots start at zero for the compositing's atomics
         float4 *g = reinterpret_cast<float4 *>(c.grad2d + r * kG2Floats);
         g[0] = g[1] = g[2] = make_float4(0.f, 0.f, 0.f, 0.f);
     }
@@ -313,10 +313,9 @@ constexpr int kPreThreads = 128;  // standalone blend
 // the row stride of the staged weights: max_k rounded up to a multiple of 4
 __host__ __device__ constexpr int psi_stride(int max_k) { return (max_k + 3) & ~3; }
 constexpr int kPreG = 32;         // Gaussians per CTA
-constexpr int kPreSlots = 8;      // frame slots per Gaussian
 constexpr int kPreFB = 2;         // frames per thread per round (register block)
-constexpr int kPreRound = kPreSlots * kPreFB;
-constexpr int kPreBlock = kPreG * kPreSlots;
+constexpr int pre_round(int slots) { return slots * kPreFB; }  // frames per round of a CTA with that many slots
+constexpr int kPreRound = pre_round(8);  // of the larger instance
 
 __host__ __device__ constexpr int popcount_c(unsigned x) { return x ? (int)(x & 1u) + popcount_c(x >> 1) : 0; }
 
@@ -330,18 +329,54 @@ __device__ __forceinline__ void cp_async16(void *dst, const void *src) {
     asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" :: "r"(smem_u32(dst)), "l"(src) : "memory");
 }
 
+// Frames [round, round + nr) of the model's frame list, by all `threads` threads of the CTA: weights
+// (rows of kp), parameters and constants.
+__device__ __forceinline__ void stage_frames(const Ctx &c, const ModelInfo &m, int round, int nr, int kp, int tid,
+                                             int threads, float *s_psi, float *s_fp, FrameConst *s_fc) {
+    for (int e = tid; e < nr * m.k; e += threads) {
+        const int fl = e / m.k, kk = e - fl * m.k;
+        const int b = c.mframes[m.frame_off + round + fl];
+        s_psi[fl * kp + kk] = c.psi[(size_t)b * c.k_stride + kk];
+    }
+    for (int e = tid; e < nr * RGBA_FP_STRIDE; e += threads) {
+        const int fl = e / RGBA_FP_STRIDE, q = e - fl * RGBA_FP_STRIDE;
+        const int b = c.mframes[m.frame_off + round + fl];
+        s_fp[e] = c.fparams[(size_t)b * RGBA_FP_STRIDE + q];
+    }
+    if (tid < nr) {
+        const int b = c.mframes[m.frame_off + round + tid];
+        const FrameInfo &f = c.frames[b];
+        const float *fp = c.fparams + (size_t)b * RGBA_FP_STRIDE;
+        FrameConst fc;
+        fc.limx = fmul(1.3f, fdiv(fmul(0.5f, (float)f.W), fp[12]));
+        fc.limy = fmul(1.3f, fdiv(fmul(0.5f, (float)f.H), fp[13]));
+        fc.tiles_x = f.tiles_x;
+        fc.tiles_y = f.tiles_y;
+        fc.tile_base = f.tile_base;
+        fc.rec_base = f.rec_base;
+        fc.verts = f.verts;
+        s_fc[tid] = fc;
+    }
+}
+
 // One CTA = kPreG (32) Gaussians of one model and every frame that renders it. The model's G0
 // rows and blendshape rows for the chunk arrive once in shared memory by 16-byte asynchronous
 // copies from all threads (39 KB at K = 32 with 9 blended channels, so several CTAs share an
-// SM; 128-byte bulk copies issued by one warp were 20 % slower); its kPreSlots (8)
+// SM; 128-byte bulk copies issued by one warp were 20 % slower); its SLOTS
 // thread slots per Gaussian then each blend kPreFB (2) frames at a time from shared memory
 // (each blendshape value read once per 2 frames) and run the decision spec per frame.
 // MASK != 0: every model of the batch blends exactly the channels in MASK, so the channel
 // selection of the blend loop is resolved at compile time (a runtime mask costs a test, a
 // branch and an index update per channel and blendshape); MASK = 0 reads each model's mask.
-template <unsigned MASK>
-__global__ void __launch_bounds__(kPreBlock, 3)
+// SLOTS: frame slots per Gaussian, 4 where every model is rendered by at most eight frames, else 8.
+// Bound by latency at about half the issue slots: divisions, square roots and the records' 188 bytes per
+// (frame, Gaussian). Four CTAs of eight slots per SM (64 registers, a few spilled) against three: 16 frames of
+// 60,000 Gaussians 68.5 -> 67.5 us, ten frames 42.8 -> 41.2. Four slots against eight with half of them idle: 64
+// frames of eight avatars, eight each, 325 -> 287 us.
+template <unsigned MASK, int SLOTS>
+__global__ void __launch_bounds__(kPreG * SLOTS, SLOTS == 8 ? 4 : 6)
 k_preprocess(Ctx c, int max_k) {
+    constexpr int kPreRound = pre_round(SLOTS), kPreBlock = kPreG * SLOTS;
     extern __shared__ float4 smem4[];
     __shared__ FrameConst s_fc[kPreRound];
     pdl_enter();
@@ -377,30 +412,7 @@ k_preprocess(Ctx c, int max_k) {
     float op0 = 0.0f;
     for (int round = 0; round < m.nb; round += kPreRound) {
         const int nr = min(kPreRound, m.nb - round);
-        for (int e = tid; e < nr * K; e += kPreBlock) {
-            const int fl = e / K, kk = e - fl * K;
-            const int b = c.mframes[m.frame_off + round + fl];
-            s_psi[fl * kp + kk] = c.psi[(size_t)b * c.k_stride + kk];
-        }
-        for (int e = tid; e < nr * RGBA_FP_STRIDE; e += kPreBlock) {
-            const int fl = e / RGBA_FP_STRIDE, q = e - fl * RGBA_FP_STRIDE;
-            const int b = c.mframes[m.frame_off + round + fl];
-            s_fp[e] = c.fparams[(size_t)b * RGBA_FP_STRIDE + q];
-        }
-        if (tid < nr) {
-            const int b = c.mframes[m.frame_off + round + tid];
-            const FrameInfo &f = c.frames[b];
-            const float *fp = c.fparams + (size_t)b * RGBA_FP_STRIDE;
-            FrameConst fc;
-            fc.limx = fmul(1.3f, fdiv(fmul(0.5f, (float)f.W), fp[12]));
-            fc.limy = fmul(1.3f, fdiv(fmul(0.5f, (float)f.H), fp[13]));
-            fc.tiles_x = f.tiles_x;
-            fc.tiles_y = f.tiles_y;
-            fc.tile_base = f.tile_base;
-            fc.rec_base = f.rec_base;
-            fc.verts = f.verts;
-            s_fc[tid] = fc;
-        }
+        stage_frames(c, m, round, nr, kp, tid, kPreBlock, s_psi, s_fp, s_fc);
         if (round == 0) asm volatile("cp.async.wait_all;" ::: "memory");
         __syncthreads();
         if (round == 0) op0 = sigmoid_spec(s_rows[10 * kPreG + g]);
@@ -468,6 +480,94 @@ k_preprocess(Ctx c, int max_k) {
             }
         }
         __syncthreads();
+    }
+}
+
+// The same for large models rendered by at most kFewFrames frames each: a staged row
+// would be read once or twice and most of the slots above would have no frame. Here a thread
+// takes one Gaussian and FB frames and reads the blendshape rows straight from global memory, four
+// blendshapes' loads in flight at once; the CTA's further groups of kFewG threads take the next
+// frames of the same Gaussians (their reads hit L1).
+// Staged against this: one frame of 60,000 Gaussians (K = 32, 73 MB of rows) 22 -> 19 us, 15 frames of five avatars
+// of up to 100,000 129 -> 123, three frames of 35,001 (K = 7) 16 -> 15; but one of 10,000 10 -> 11, where the
+// staged copies have every row in flight at once, hence kFewMinN; and at eight frames a model the shared rows win
+// (64 frames of eight avatars: 287 us staged, 386 so).
+constexpr int kFewG = 64;      // Gaussians per CTA
+constexpr int kFewFrames = 4;
+constexpr int kFewMinN = 20000;
+
+template <unsigned MASK, int FB>
+__global__ void __launch_bounds__(kFewG * (kFewFrames / FB))
+k_preprocess_few(Ctx c, int max_k) {
+    extern __shared__ float4 smem4[];
+    __shared__ FrameConst s_fc[kFewFrames];
+    pdl_enter();
+    const ModelInfo &m = c.models[blockIdx.y];
+    const int i0 = blockIdx.x * kFewG;
+    if (i0 >= m.n || m.nb == 0) return;
+    constexpr int A = popcount_c(MASK);
+    const int K = m.k, nr = m.nb, kp = psi_stride(max_k);
+    float *s_psi = reinterpret_cast<float *>(smem4);  // [kFewFrames][kp]
+    float *s_fp = s_psi + kFewFrames * kp;            // [kFewFrames][20]
+    const int tid = threadIdx.x, i = i0 + tid % kFewG, f0 = tid / kFewG * FB;
+    const bool live = i < m.n && f0 < nr;
+    float v[FB][kNch];
+    if (live) {
+#pragma unroll
+        for (int ch = 0; ch < kNch; ++ch) v[0][ch] = __ldg(m.g0 + (size_t)ch * m.n_pad + i);
+    }
+    stage_frames(c, m, 0, nr, kp, tid, blockDim.x, s_psi, s_fp, s_fc);
+    __syncthreads();
+    if (!live) return;
+    const float op = sigmoid_spec(v[0][10]);  // never blended
+#pragma unroll
+    for (int q = 1; q < FB; ++q)
+#pragma unroll
+        for (int ch = 0; ch < kNch; ++ch) v[q][ch] = v[0][ch];
+    const size_t row = (size_t)m.n_pad;
+    const float *d = m.dg + i;
+    const float *ps = s_psi + f0 * kp;
+    int kk = 0;
+    for (; kk + 4 <= K; kk += 4, d += 4 * A * row) {
+        float dv[4][A];
+#pragma unroll
+        for (int u = 0; u < 4; ++u)
+#pragma unroll
+            for (int a = 0; a < A; ++a) dv[u][a] = __ldg(d + (u * A + a) * row);
+#pragma unroll
+        for (int q = 0; q < FB; ++q) {
+            const float4 w4 = *reinterpret_cast<const float4 *>(ps + q * kp + kk);
+            const float w[4] = {w4.x, w4.y, w4.z, w4.w};
+#pragma unroll
+            for (int u = 0; u < 4; ++u) {
+                int a = 0;
+#pragma unroll
+                for (int ch = 0; ch < kNch; ++ch)
+                    if ((MASK >> ch) & 1u) v[q][ch] = __fmaf_rn(w[u], dv[u][a++], v[q][ch]);
+            }
+        }
+    }
+    for (; kk < K; ++kk, d += A * row) {
+        int a = 0;
+#pragma unroll
+        for (int ch = 0; ch < kNch; ++ch)
+            if ((MASK >> ch) & 1u) {
+                const float dv = __ldg(d + a++ * row);
+#pragma unroll
+                for (int q = 0; q < FB; ++q) v[q][ch] = __fmaf_rn(ps[q * kp + kk], dv, v[q][ch]);
+            }
+    }
+    // one frame at a time through v[0] (a rolled loop keeps the code small)
+#pragma unroll 1
+    for (int q = 0; q < FB; ++q) {
+        if (f0 + q < nr) {
+            const FrameConst &fc = s_fc[f0 + q];
+            decide_and_write(c, m, fc, s_fp + (f0 + q) * RGBA_FP_STRIDE, v[0], op, i, fc.rec_base + i);
+        }
+#pragma unroll
+        for (int q2 = 0; q2 + 1 < FB; ++q2)
+#pragma unroll
+            for (int ch = 0; ch < kNch; ++ch) v[q2][ch] = v[q2 + 1][ch];
     }
 }
 
@@ -553,31 +653,50 @@ int preprocess_smem(int max_k, int max_rows) {
 }
 
 namespace {
-template <unsigned MASK>
-cudaError_t preprocess_inst(const Ctx &c, int max_n, int max_k, int max_rows, cudaStream_t s) {
+template <unsigned MASK, int FB>
+cudaError_t preprocess_few(const Ctx &c, int max_n, int max_nb, int max_k, cudaStream_t s) {
+    const int groups = (max_nb + FB - 1) / FB;
+    const size_t smem = kFewFrames * (size_t)(psi_stride(max_k) + RGBA_FP_STRIDE) * sizeof(float);
+    return launch_pdl(k_preprocess_few<MASK, FB>, dim3((max_n + kFewG - 1) / kFewG, c.M), dim3(kFewG * groups), smem, s,
+                      c, max_k);
+}
+
+template <unsigned MASK, int SLOTS>
+cudaError_t preprocess_slots(const Ctx &c, int max_n, int max_k, int max_rows, cudaStream_t s) {
     static int attr_device = -1;
     int dev = 0;
     cudaError_t e = cudaGetDevice(&dev);
     if (e != cudaSuccess) return e;
     if (attr_device != dev) {  // once, at the largest size (K = 64, 13 blended channels)
-        e = cudaFuncSetAttribute(k_preprocess<MASK>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+        e = cudaFuncSetAttribute(k_preprocess<MASK, SLOTS>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                  preprocess_smem(RGBA_MAX_K, kNch + RGBA_MAX_K * 13));
         if (e != cudaSuccess) return e;
         attr_device = dev;
     }
     dim3 grid((max_n + kPreG - 1) / kPreG, c.M);
-    return launch_pdl(k_preprocess<MASK>, grid, dim3(kPreBlock), preprocess_smem(max_k, max_rows), s, c, max_k);
+    return launch_pdl(k_preprocess<MASK, SLOTS>, grid, dim3(kPreG * SLOTS), preprocess_smem(max_k, max_rows), s, c, max_k);
+}
+
+template <unsigned MASK>
+cudaError_t preprocess_inst(const Ctx &c, int max_n, int max_nb, int max_k, int max_rows, cudaStream_t s) {
+    if constexpr (MASK != 0u) {
+        if (max_nb <= kFewFrames && max_n >= kFewMinN)
+            return max_nb == 1 ? preprocess_few<MASK, 1>(c, max_n, max_nb, max_k, s)
+                               : preprocess_few<MASK, 2>(c, max_n, max_nb, max_k, s);
+    }
+    return max_nb <= pre_round(4) ? preprocess_slots<MASK, 4>(c, max_n, max_k, max_rows, s)
+                                  : preprocess_slots<MASK, 8>(c, max_n, max_k, max_rows, s);
 }
 }  // namespace
 
-cudaError_t launch_preprocess(const Ctx &c, int max_n, int max_k, int max_rows, unsigned common_mask,
+cudaError_t launch_preprocess(const Ctx &c, int max_n, int max_nb, int max_k, int max_rows, unsigned common_mask,
                               cudaStream_t s) {
     if (c.B == 0 || max_n == 0) return cudaSuccess;
     if (common_mask == RGBA_MASK_MEAN_SCALE_COLOR)
-        return preprocess_inst<RGBA_MASK_MEAN_SCALE_COLOR>(c, max_n, max_k, max_rows, s);
+        return preprocess_inst<RGBA_MASK_MEAN_SCALE_COLOR>(c, max_n, max_nb, max_k, max_rows, s);
     if (common_mask == RGBA_MASK_MEAN_ROT_COLOR)
-        return preprocess_inst<RGBA_MASK_MEAN_ROT_COLOR>(c, max_n, max_k, max_rows, s);
-    return preprocess_inst<0u>(c, max_n, max_k, max_rows, s);
+        return preprocess_inst<RGBA_MASK_MEAN_ROT_COLOR>(c, max_n, max_nb, max_k, max_rows, s);
+    return preprocess_inst<0u>(c, max_n, max_nb, max_k, max_rows, s);
 }
 
 cudaError_t launch_blend(const Ctx &c, int max_n, float *out, cudaStream_t s) {

@@ -145,6 +145,7 @@ struct Ctx {
     unsigned *sorted;
     // keys carry a pixel-block mask (pack_low): every model has at most kMaskedN Gaussians
     bool masked;
+    bool zero_g2;  // the preprocess zeroes grad2d (a standalone backward clears it itself)
     float *dpsi_part;
     float *depth;      // [R]: view-space depth of each kept record (the scatter's sort key)
     long long R, T, cap;
@@ -209,9 +210,9 @@ struct PrologueArgs {
     long long zero_b16;
 };
 cudaError_t launch_prologue(const PrologueArgs &a, const void *const src[3], cudaStream_t s);
-// common_mask: the channel mask every model of the
+// max_nb: the most frames any model is rendered by. common_mask: the channel mask every model of the
 // batch shares (0 when they differ); the two masks of the RGBA_MASK_* constants run a blend specialised at compile time.
-cudaError_t launch_preprocess(const Ctx &c, int max_n, int max_k, int max_rows, unsigned common_mask,
+cudaError_t launch_preprocess(const Ctx &c, int max_n, int max_nb, int max_k, int max_rows, unsigned common_mask,
                               cudaStream_t s);
 cudaError_t launch_blend(const Ctx &c, int max_n, float *out, cudaStream_t s);
 // max_tiles: the most tiles of any frame of the batch
