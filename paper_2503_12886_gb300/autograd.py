@@ -80,18 +80,17 @@ class RasterizeBlendFn(torch.autograd.Function):
                                       binding=bd))
         db = _device_batch(ctx.spec, psi.contiguous(), fparams.contiguous(), models, grads=True)
         r: Renderer = ctx.renderer
-        ws = r.ensure_workspace(db)
         b = db.struct()
+        ws = r.ensure_workspace(db, struct=b)
         s = stream_ptr()
         for _ in range(3):  # recompute the splats and tile lists the forward used
             api.rgba_preprocess(r.ctx, b, ws.data_ptr(), ws.numel(), s)
             api.rgba_bin_sort(r.ctx, b, ws.data_ptr(), ws.numel(), s)
-            cnt = r.counters(db)
+            cnt = r.counters(db, b)
             if not cnt["overflow"]:
                 break
-            ws = r.ensure_workspace(db, int(cnt["pairs"] * 1.25) + 4096)
-            b = db.struct()
-        r.backward(db, dl_dimg.contiguous(), T, n)
+            ws = r.ensure_workspace(db, int(cnt["pairs"] * 1.25) + 4096, b)
+        r.backward(db, dl_dimg.contiguous(), T, n, struct=b)
         grads = []
         for m in models:
             grads += [m.grad_g0, m.grad_dg]
