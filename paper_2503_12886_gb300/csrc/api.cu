@@ -366,7 +366,7 @@ int do_preprocess(rgba_ctx_t ctx, Call &k, bool zero_g2) {
 int do_bin_sort(rgba_ctx_t ctx, Call &k) {
     cudaError_t e;
     {
-        StageScope sc(ctx, ST_SCAN, k.s, 4);
+        StageScope sc(ctx, ST_SCAN, k.s, 1 + scan_kernels(k.c.T));
         if ((e = launch_count(k.c, k.p.max_n, k.p.max_tiles, k.s)) != cudaSuccess) return cuda_fail(e, "count");
         if ((e = launch_scan(k.c, k.s)) != cudaSuccess) return cuda_fail(e, "scan");
     }

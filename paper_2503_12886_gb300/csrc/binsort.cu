@@ -246,6 +246,66 @@ __global__ void __launch_bounds__(kScanTile) k_scan_write(Ctx c) {
     }
 }
 
+// The three phases by one CTA, kScanOne / kScanTile tiles per thread, for batches of few tiles, where the
+// launches are most of the phases' time: count and scan 12.2 -> 8.8 us at 64 tiles, 13.7 -> 8.8 at 1,024, 14.1 ->
+// 9.2 at 2,268. With 16 tiles per thread one CTA takes 25 us at 10,240 tiles and the phases 17.
+constexpr int kScanOne = 4 * kScanTile;
+
+__global__ void __launch_bounds__(kScanTile) k_scan_one(Ctx c) {
+    constexpr int PER = kScanOne / kScanTile;
+    __shared__ unsigned s_hist[32], s_off[32];
+    pdl_enter();
+    const int tid = threadIdx.x;
+    if (tid < 32) s_hist[tid] = 0u;
+    __syncthreads();
+    const int t0 = tid * PER, T = (int)c.T;
+    unsigned v[PER], ne = 0u;
+    unsigned long long sum = 0ull;
+#pragma unroll
+    for (int q = 0; q < PER; ++q) {
+        v[q] = t0 + q < T ? c.tile_count[t0 + q] : 0u;
+        sum += v[q];
+        if (v[q]) {
+            ++ne;
+            atomicAdd(&s_hist[bucket_of(v[q])], 1u);
+        }
+    }
+    unsigned long long st, tot;
+    unsigned exe, tote;
+    block_scan(sum, ne, st, exe, tot, tote);  // its syncs also publish s_hist
+    if (tid < 32) {  // bucket offsets, the longest bucket first
+        const unsigned h = s_hist[31 - tid];
+        unsigned x = h;
+#pragma unroll
+        for (int o = 1; o < 32; o <<= 1) {
+            const unsigned y = __shfl_up_sync(0xffffffffu, x, o);
+            if (tid >= o) x += y;
+        }
+        s_off[31 - tid] = x - h;
+    }
+    __syncthreads();
+    unsigned empty = (unsigned)t0 - exe;  // empty tiles before this thread's
+#pragma unroll
+    for (int q = 0; q < PER; ++q) {
+        if (t0 + q >= T) break;
+        const unsigned at = st > 0xffffffffull ? 0xffffffffu : (unsigned)st;
+        c.tile_start[t0 + q] = at;
+        if (v[q]) {
+            c.cursor[t0 + q] = at;
+            c.work[atomicAdd(&s_off[bucket_of(v[q])], 1u)] = (unsigned)(t0 + q);
+        } else {
+            c.work[tote + empty++] = (unsigned)(t0 + q);
+        }
+        st += v[q];
+    }
+    if (tid == 0) {
+        c.tile_start[T] = tot > 0xffffffffull ? 0xffffffffu : (unsigned)tot;
+        c.cnt->pairs = tot > 0xffffffffull ? 0xffffffffu : (unsigned)tot;
+        c.cnt->overflow = tot > (unsigned long long)c.cap ? 1u : 0u;
+        c.cnt->n_work = tote;
+    }
+}
+
 // One thread per (frame, Gaussian): drops its key into the list of every tile of its rectangle,
 // with the tile's block mask. The masks cost one ellipse extent per four pixel rows of the
 // rectangle and two compares per block; computed here they are paid once per (Gaussian, tile),
@@ -801,12 +861,15 @@ __global__ void __launch_bounds__(kSortThreads, 2) k_tile_sort(Ctx c) {
 }  // namespace
 
 cudaError_t launch_scan(const Ctx &c, cudaStream_t s) {
+    if (c.T <= kScanOne) return launch_pdl(k_scan_one, dim3(1), dim3(kScanTile), 0, s, c);
     const unsigned nb = (unsigned)((c.T + kScanTile - 1) / kScanTile);
     cudaError_t e = launch_pdl(k_scan_blocks, dim3(nb), dim3(kScanTile), 0, s, c);
     if (e != cudaSuccess) return e;
     if ((e = launch_pdl(k_scan_top, dim3(1), dim3(kScanTile), 0, s, c)) != cudaSuccess) return e;
     return launch_pdl(k_scan_write, dim3(nb), dim3(kScanTile), 0, s, c);
 }
+
+int scan_kernels(long long T) { return T <= kScanOne ? 1 : 3; }
 
 size_t scan_aux_bytes(long long T) {
     const long long nb = (T + kScanTile - 1) / kScanTile;

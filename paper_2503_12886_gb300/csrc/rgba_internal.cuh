@@ -218,6 +218,7 @@ cudaError_t launch_blend(const Ctx &c, int max_n, float *out, cudaStream_t s);
 // max_tiles: the most tiles of any frame of the batch
 cudaError_t launch_count(const Ctx &c, int max_n, int max_tiles, cudaStream_t s);
 cudaError_t launch_scan(const Ctx &c, cudaStream_t s);
+int scan_kernels(long long T);  // the kernels that launch_scan launches
 size_t scan_aux_bytes(long long T);
 cudaError_t launch_scatter(const Ctx &c, int max_n, int max_tiles, cudaStream_t s);
 cudaError_t launch_tile_sort(const Ctx &c, int sms, cudaStream_t s);

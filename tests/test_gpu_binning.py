@@ -48,3 +48,11 @@ def test_large_frames(renderer, tile, size):
     batch = synth.make_batch([dataclasses.replace(m, g0=g0)], [synth.Frame(0, *size), synth.Frame(0, 64, 48)], seed=103,
                              jitter_deg=10)
     assert check(renderer, batch, tile)["pairs"] > 0
+
+
+@pytest.mark.parametrize("sizes", [[(1024, 1024)], [(1024, 1024), (16, 16)], [(16, 16)], [(1, 1)], [(1024, 1008), (250, 10)]])
+def test_scan_by_one_cta(renderer, sizes):
+    """Up to 4,096 tiles are scanned by one CTA: 4,096, 4,097, 1, 1 and 4,048 tiles."""
+    m = synth.make_model(104, 3000, 3)
+    batch = synth.make_batch([m], [synth.Frame(0, w, h) for w, h in sizes], seed=104, jitter_deg=10)
+    assert check(renderer, batch, (16, 16))["pairs"] > 0
