@@ -622,7 +622,8 @@ __device__ __forceinline__ bool bucket_sort(const unsigned long long *g, int L, 
 
 constexpr int kStreamBits = 14;  // buckets of the sort of long lists
 constexpr int kStreamLoads = 8;  // keys per thread in flight in its sweeps
-static_assert((4 << kStreamBits) <= kSortSmem, "bucket counts fit");
+constexpr int kStreamChunk = kStreamLoads * kSortThreads - 2 * kBucketRun;  // keys ranked at a time
+static_assert((4 << kStreamBits) + 8 * kStreamLoads * kSortThreads <= kSortSmem, "bucket counts and a chunk fit");
 
 // Calls f(key) for the L keys at g, kStreamLoads of each thread's loads in flight at once.
 template <typename F>
@@ -683,14 +684,33 @@ __device__ bool bucket_sort_stream(const unsigned long long *g, unsigned long lo
     __syncthreads();
     sweep(g, L, [&](unsigned long long k) { tmp[atomicAdd(&s_cnt[bucket(k)], 1u)] = k; });
     __syncthreads();  // s_cnt[b] is now the end of bucket b; the keys at g are no longer needed
-    sweep(tmp, L, [&](unsigned long long k) {
-        const unsigned b = bucket(k);
-        const int lo = b ? (int)s_cnt[b - 1] : 0, hi = (int)s_cnt[b];
-        int rank = lo;
-        for (int q = lo; q < hi; ++q) rank += tmp[q] < k;
-        out[rank] = low_index(masked, (unsigned)k);
-        out_mask[rank] = low_mask(masked, (unsigned)k);
-    });
+    // the grouped keys come back to shared memory a chunk at a time, with the keys around it that a bucket
+    // can reach into, the next chunk's loads under way while this one's keys are ranked
+    unsigned long long *s_k = reinterpret_cast<unsigned long long *>(s_cnt + NB);
+    unsigned long long k[kStreamLoads];
+    auto load = [&](int c0) {
+        const int at = max(0, c0 - kBucketRun), n = min(L, c0 + kStreamChunk + kBucketRun) - at;
+#pragma unroll
+        for (int u = 0; u < kStreamLoads; ++u) k[u] = tid + u * kSortThreads < n ? tmp[at + tid + u * kSortThreads] : 0ull;
+    };
+    load(0);
+    for (int c0 = 0; c0 < L; c0 += kStreamChunk) {
+#pragma unroll
+        for (int u = 0; u < kStreamLoads; ++u) s_k[tid + u * kSortThreads] = k[u];
+        __syncthreads();
+        if (c0 + kStreamChunk < L) load(c0 + kStreamChunk);
+        const int at = max(0, c0 - kBucketRun);  // s_k[q - at] is tmp[q]
+        for (int p = c0 + tid; p < min(L, c0 + kStreamChunk); p += kSortThreads) {
+            const unsigned long long key = s_k[p - at];
+            const unsigned b = bucket(key);
+            const int lo = b ? (int)s_cnt[b - 1] : 0, hi = (int)s_cnt[b];
+            int rank = lo;
+            for (int q = lo; q < hi; ++q) rank += s_k[q - at] < key;
+            out[rank] = low_index(masked, (unsigned)key);
+            out_mask[rank] = low_mask(masked, (unsigned)key);
+        }
+        __syncthreads();
+    }
     return true;
 }
 
