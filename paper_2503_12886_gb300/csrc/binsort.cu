@@ -344,7 +344,7 @@ __global__ void __launch_bounds__(kBinThreads) k_scatter(Ctx c) {
     for (int ty = rc.y; ty < rc.w; ++ty) {
         float xl[BANDS], xr[BANDS];
 #pragma unroll
-        for (int k = 0; k < BANDS; ++k) reach_rows(e, (float)(ty * TH + 4 * k) + 0.5f, xl[k], xr[k]);
+        for (int k = 0; k < BANDS; ++k) reach_rows(e, (float)(ty * TH + 4 * k) + 0.5f, (float)(ty * TH + 4 * k) + 3.5f, xl[k], xr[k]);
         for (int tx = rc.x; tx < rc.z; ++tx) {
             unsigned mask = 0u;
 #pragma unroll

@@ -43,10 +43,10 @@ __device__ __forceinline__ Reach reach_of(const float4 &r0, const float2 &r1) {
     return e;
 }
 
-// The x extent [xl, xr] of the ellipse over pixel-centre rows y .. y + 3, widened (empty: xl > xr).
+// The x extent [xl, xr] of the ellipse over pixel-centre rows y0 .. y1, widened (empty: xl > xr).
 // The right end over the rows is where dy is closest to ys, the left end closest to -ys.
-__device__ __forceinline__ void reach_rows(const Reach &e, float y, float &xl, float &xr) {
-    const float d0 = y - 0.05f - e.v, d1 = y + 3.05f - e.v;
+__device__ __forceinline__ void reach_rows(const Reach &e, float y0, float y1, float &xl, float &xr) {
+    const float d0 = y0 - 0.05f - e.v, d1 = y1 + 0.05f - e.v;
     xl = 1.0f;
     xr = -1.0f;
     if (d0 > e.hy || d1 < -e.hy) return;

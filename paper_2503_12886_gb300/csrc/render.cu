@@ -256,13 +256,38 @@ __device__ __forceinline__ void put_slot(WarpMem<S> &m, int h, int k, const floa
     s.idx[i] = idx;
 }
 
-// The staged entries into the slots of the halves they reach, in order; n[h] of half h. A half with
+// The bounding box, in pixel centres, of the pixels of half h that `live` (one bit per lane) holds.
+struct LiveBox {
+    float x0, x1, y0, y1;
+    bool any;
+};
+__device__ __forceinline__ LiveBox live_box(const Walk &w, unsigned live, int h) {
+    const unsigned m = (live >> (16 * h)) & 0xffffu;
+    unsigned col = m | m >> 8;
+    col = (col | col >> 4) & 15u;
+    LiveBox b;
+    b.any = m != 0u;
+    b.x0 = w.bx0 + (float)(4 * h + __ffs((int)col) - 1);
+    b.x1 = w.bx0 + (float)(4 * h + 31 - __clz((int)col));
+    b.y0 = w.by0 + (float)((__ffs((int)m) - 1) >> 2);
+    b.y1 = w.by0 + (float)((31 - __clz((int)m)) >> 2);
+    return b;
+}
+
+// The staged entries into the slots of the halves whose live pixels they can reach (live: one bit per lane for
+// the pixels that can still take one of them), in order; n[h] of half h. Where a block is nearly saturated,
+// or in the backward nearly not reached yet, most of the entries that its mask lets through only touch pixels
+// that are out of the walk: on one 64 x 64 frame of 100,000 Gaussians, where the silhouette's blocks walk lists of
+// 59,000 entries, the forward takes 852 us with this cut and 1,372 without. On 16
+// frames of 512 x 512 it saves 6 us of 121 forwards and 11 of 152 backwards, on 15 frames of five avatars 12 of 160. A half with
 // fewer is filled up, to an even number, with entries that no pixel takes. Returns the slots to walk;
 // reach[h]: the lanes whose (last) entry reaches half h.
 template <int S>
-__device__ __forceinline__ int commit(const Walk &w, const Stage<S> &g, WarpMem<S> &m, int n[2], unsigned reach[2]) {
+__device__ __forceinline__ int commit(const Walk &w, const Stage<S> &g, WarpMem<S> &m, unsigned live, int n[2],
+                                      unsigned reach[2]) {
     const int lane = threadIdx.x & 31;
     const unsigned lt = (1u << lane) - 1u;
+    const LiveBox bl = live_box(w, live, 0), br = live_box(w, live, 1);
     __syncwarp();  // the previous stage's slots are no longer read
     n[0] = n[1] = 0;
 #pragma unroll
@@ -272,19 +297,20 @@ __device__ __forceinline__ int commit(const Walk &w, const Stage<S> &g, WarpMem<
         if (lane + 32 * s < g.id.n) {
             const Reach e = reach_of(g.r0[s], make_float2(g.r1[s].x, g.r1[s].y));
             float xl, xr;
-            reach_rows(e, w.by0, xl, xr);
             tau = alpha_cut(g.r1[s].y);
-            const bool all = e.all || !w.masked, hit = xr >= w.bx0 && xl <= w.bx0 + 7.0f && !e.none;
-            left = all || (hit && xl <= w.bx0 + 3.0f);
-            right = all || (hit && xr >= w.bx0 + 4.0f);
+            const bool all = e.all || !w.masked;
+            reach_rows(e, bl.y0, bl.y1, xl, xr);
+            left = bl.any && (all || (!e.none && xr >= bl.x0 && xl <= bl.x1));
+            reach_rows(e, br.y0, br.y1, xl, xr);
+            right = br.any && (all || (!e.none && xr >= br.x0 && xl <= br.x1));
         }
-        const unsigned bl = __ballot_sync(0xffffffffu, left), br = __ballot_sync(0xffffffffu, right);
-        if (left) put_slot(m, 0, n[0] + __popc(bl & lt), g.r0[s], g.r1[s], g.r2[s], tau, g.id.pos[s], g.id.idx[s]);
-        if (right) put_slot(m, 1, n[1] + __popc(br & lt), g.r0[s], g.r1[s], g.r2[s], tau, g.id.pos[s], g.id.idx[s]);
-        n[0] += __popc(bl);
-        n[1] += __popc(br);
-        reach[0] = bl;
-        reach[1] = br;
+        const unsigned ml = __ballot_sync(0xffffffffu, left), mr = __ballot_sync(0xffffffffu, right);
+        if (left) put_slot(m, 0, n[0] + __popc(ml & lt), g.r0[s], g.r1[s], g.r2[s], tau, g.id.pos[s], g.id.idx[s]);
+        if (right) put_slot(m, 1, n[1] + __popc(mr & lt), g.r0[s], g.r1[s], g.r2[s], tau, g.id.pos[s], g.id.idx[s]);
+        n[0] += __popc(ml);
+        n[1] += __popc(mr);
+        reach[0] = ml;
+        reach[1] = mr;
     }
     const int top = (max(n[0], n[1]) + 1) & ~1;
     const float4 z = make_float4(0.f, 0.f, 0.f, 0.f);
@@ -495,11 +521,12 @@ __device__ __forceinline__ void fwd_walk(const Walk &w, WarpMem<S> &m, PixF &p, 
     load_ids<S>(w, m, f, d);
     while (g.id.n) {
         if (STATS) st.staged += scanned;
-        if (__all_sync(0xffffffffu, p.done)) break;
+        const unsigned live = __ballot_sync(0xffffffffu, !p.done);
+        if (!live) break;
         int n[2];
         unsigned reach[2];
         if (STATS) st.hits += g.id.n;
-        const int top = commit<S>(w, g, m, n, reach);
+        const int top = commit<S>(w, g, m, live, n, reach);
         scanned = f.fill(w, m);
         load_stage<S>(w, d, g);
         load_ids<S>(w, m, f, d);
@@ -652,7 +679,12 @@ __device__ __forceinline__ void bwd_walk(const Walk &w, WarpMem<S> &m, GradMem &
             st.staged += scanned;
             st.hits += g.id.n;
         }
-        const int top = commit<S>(w, g, m, n, reach);
+        // the pixels that blended any of the stage's entries, or any in front of them: those whose contributor
+        // count reaches the stage's last (foremost) entry
+        static_assert(S == 1, "one entry per lane");
+        const int foremost = __shfl_sync(0xffffffffu, (int)g.id.pos[0], g.id.n - 1);
+        const unsigned live = __ballot_sync(0xffffffffu, p.last >= foremost);
+        const int top = commit<S>(w, g, m, live, n, reach);
         scanned = f.fill(w, m);
         load_stage<S>(w, d, g);
         load_ids<S>(w, m, f, d);
