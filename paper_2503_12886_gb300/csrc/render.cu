@@ -109,17 +109,18 @@ struct __align__(16) Pair {
 };
 
 // A warp's shared memory: the queue of list positions that reach its block, and for each half of
-// the block its staged slots, up to 32 S (and a pair past the end for the loop's look-ahead). The
+// the block its staged slots, up to 32 S (the loop looks one pair ahead, past the end at whatever follows). The
 // halves lie 64 bytes apart modulo the banks' 128, so that both halves' reads are one pass.
 template <int S>
 struct WarpMem {
     static constexpr int kQueue = 256;  // holds a stage's worth and one scan
     static_assert(32 * S - 1 + 128 <= kQueue, "queue");
-    static constexpr int kHalf = 16 * S * (int)sizeof(Pair) + 64;
-    __align__(16) unsigned char slots[kHalf + (16 * S + 1) * sizeof(Pair)];
-    unsigned queue[kQueue];
-    __device__ __forceinline__ Pair *half(int h) { return reinterpret_cast<Pair *>(slots + h * kHalf); }
-    __device__ __forceinline__ const Pair *half(int h) const { return reinterpret_cast<const Pair *>(slots + h * kHalf); }
+    static constexpr int kHalf = 16 * S * (int)sizeof(Pair) + 64, kSlots = kHalf + 16 * S * (int)sizeof(Pair);
+    __align__(16) unsigned char mem[kSlots + 4 * kQueue];  // the halves' slots, then the queue
+    __device__ __forceinline__ Pair *half(int h) { return reinterpret_cast<Pair *>(mem + h * kHalf); }
+    __device__ __forceinline__ const Pair *half(int h) const { return reinterpret_cast<const Pair *>(mem + h * kHalf); }
+    __device__ __forceinline__ unsigned &queue(unsigned i) { return reinterpret_cast<unsigned *>(mem + kSlots)[i & (kQueue - 1)]; }
+    __device__ __forceinline__ unsigned queue(unsigned i) const { return reinterpret_cast<const unsigned *>(mem + kSlots)[i & (kQueue - 1)]; }
 };
 
 // One compositing warp's view of a (tile, pixel block) item: the tile's list and the block.
@@ -166,7 +167,6 @@ struct Feed {
     }
     // until the queue holds a stage's worth (or the list is done); returns the entries scanned
     __device__ __forceinline__ int fill(const Walk &w, WarpMem<S> &m) {
-        constexpr unsigned Q = WarpMem<S>::kQueue - 1;
         const int lane = threadIdx.x & 31;
         const unsigned lt = (1u << lane) - 1u;
         int scanned = 0;
@@ -181,7 +181,7 @@ struct Feed {
 #pragma unroll
             for (int i = 0; i < 4; ++i) {
                 const int k = DIR > 0 ? i : 3 - i;
-                if ((hits >> (8 * k)) & 1u) m.queue[at++ & Q] = (unsigned)(e + k + 1);
+                if ((hits >> (8 * k)) & 1u) m.queue(at++) = (unsigned)(e + k + 1);
             }
             count += __popc(b0) + 2u * __popc(b1) + 4u * __popc(b2);
             --left;
@@ -215,7 +215,7 @@ __device__ __forceinline__ void load_ids(const Walk &w, const WarpMem<S> &m, Fee
 #pragma unroll
     for (int s = 0; s < S; ++s) {
         if (lane + 32 * s < d.n) {
-            d.pos[s] = m.queue[(f.head + lane + 32 * s) & (WarpMem<S>::kQueue - 1)];
+            d.pos[s] = m.queue(f.head + lane + 32 * s);
             d.idx[s] = w.list[d.pos[s] - 1u];
         }
     }
@@ -681,8 +681,13 @@ __device__ __forceinline__ void bwd_walk(const Walk &w, WarpMem<S> &m, GradMem &
         }
         // the pixels that blended any of the stage's entries, or any in front of them: those whose contributor
         // count reaches the stage's last (foremost) entry
-        static_assert(S == 1, "one entry per lane");
-        const int foremost = __shfl_sync(0xffffffffu, (int)g.id.pos[0], g.id.n - 1);
+        int foremost = 0;
+#pragma unroll
+        for (int s = 0; s < S; ++s) {
+            const int at = g.id.n - 1 - 32 * s;  // its lane, if it is among these 32
+            const int v = __shfl_sync(0xffffffffu, (int)g.id.pos[s], at & 31);
+            if (at >= 0 && at < 32) foremost = v;
+        }
         const unsigned live = __ballot_sync(0xffffffffu, p.last >= foremost);
         const int top = commit<S>(w, g, m, live, n, reach);
         scanned = f.fill(w, m);
@@ -936,17 +941,26 @@ cudaError_t fwd_inst(const Ctx &c, int grid, float *img, float *T, int *n, const
                       tg, lk, dl, acc_tg);
 }
 
+// Stages of 64 entries instead of 32: in the forward where the caller asks for staging of 128 or 256, and in both
+// directions for batches of at most kFewTiles tiles, whose blocks do not fill the SMs: their time is that of the longest
+// walks, which larger stages shorten (fewer waits for records). With 32 and with 64 entries: one
+// 64 x 64 frame of 100,000 Gaussians 852 against
+// 688 us forwards and 866 against 612 backwards, eight of 128 x 128 272 against 238 and 336 against 270, one of
+// 128 x 128 (N = 10,000) 43 against 37 and 55 against 45; where blocks abound the 32 are better (forward of 15 frames of
+// five avatars 160 against 170 us, of 16 frames 121 against 125).
+constexpr long long kFewTiles = 512;
+
 template <bool ACC>
 cudaError_t fwd_dispatch(const Ctx &c, int grid, int sb, float *img, float *T, int *n, const float *tg,
                          int lk, float *dl, const float *acc_tg, bool stats, cudaStream_t s) {
     if (!ACC && stats && c.tw == 16 && sb == 64)
         return fwd_inst<16, 1, false, true>(c, grid, img, T, n, tg, lk, dl, acc_tg, s);
-    if (c.tw == 16) {
-        if (sb == 64) return fwd_inst<16, 1, ACC>(c, grid, img, T, n, tg, lk, dl, acc_tg, s);
-        return fwd_inst<16, 2, ACC>(c, grid, img, T, n, tg, lk, dl, acc_tg, s);
-    }
-    if (sb == 64) return fwd_inst<8, 1, ACC>(c, grid, img, T, n, tg, lk, dl, acc_tg, s);
-    return fwd_inst<8, 2, ACC>(c, grid, img, T, n, tg, lk, dl, acc_tg, s);
+    const bool large = sb != 64 || c.T <= kFewTiles;
+    if (c.tw == 16)
+        return large ? fwd_inst<16, 2, ACC>(c, grid, img, T, n, tg, lk, dl, acc_tg, s)
+                     : fwd_inst<16, 1, ACC>(c, grid, img, T, n, tg, lk, dl, acc_tg, s);
+    return large ? fwd_inst<8, 2, ACC>(c, grid, img, T, n, tg, lk, dl, acc_tg, s)
+                 : fwd_inst<8, 1, ACC>(c, grid, img, T, n, tg, lk, dl, acc_tg, s);
 }
 
 template <int TW, int S, bool STATS = false>
@@ -969,13 +983,16 @@ cudaError_t launch_render_fwd(const Ctx &c, int grid, int smem_batch, float *img
                                nullptr, stats, s);
 }
 
-// smem_batch: the backward stages 32 entries at a time whatever the staging size (its slots and row sums
-// take 37 KB per CTA; the forward's stages grow to 64 entries at 128 and 256).
+// The backward's stages do not grow with smem_batch: its row sums take the shared memory.
 cudaError_t launch_render_bwd(const Ctx &c, int grid, int smem_batch, const float *dl_dimg,
                               const float *T_final, const int *n_contrib, bool stats, cudaStream_t s) {
     if (stats && c.tw == 16 && smem_batch == 64) return bwd_inst<16, 1, true>(c, grid, dl_dimg, T_final, n_contrib, s);
-    return c.tw == 16 ? bwd_inst<16, 1>(c, grid, dl_dimg, T_final, n_contrib, s)
-                      : bwd_inst<8, 1>(c, grid, dl_dimg, T_final, n_contrib, s);
+    const bool large = c.T <= kFewTiles;
+    if (c.tw == 16)
+        return large ? bwd_inst<16, 2>(c, grid, dl_dimg, T_final, n_contrib, s)
+                     : bwd_inst<16, 1>(c, grid, dl_dimg, T_final, n_contrib, s);
+    return large ? bwd_inst<8, 2>(c, grid, dl_dimg, T_final, n_contrib, s)
+                 : bwd_inst<8, 1>(c, grid, dl_dimg, T_final, n_contrib, s);
 }
 
 }  // namespace rgba
