@@ -150,6 +150,7 @@ __global__ void __launch_bounds__(kScanTile) k_scan_blocks(Ctx c) {
     unsigned v = 0;
     if (t < c.T) {
         v = c.tile_count[t];
+        c.tile_count[t] = 0u;  // the next binning of the same projection counts from zero again
         c.tile_start[t] = v;
         if (v) atomicAdd(&s_hist[bucket_of(v)], 1u);
     }
@@ -263,7 +264,11 @@ __global__ void __launch_bounds__(kScanTile) k_scan_one(Ctx c) {
     unsigned long long sum = 0ull;
 #pragma unroll
     for (int q = 0; q < PER; ++q) {
-        v[q] = t0 + q < T ? c.tile_count[t0 + q] : 0u;
+        v[q] = 0u;
+        if (t0 + q < T) {
+            v[q] = c.tile_count[t0 + q];
+            c.tile_count[t0 + q] = 0u;  // as k_scan_blocks
+        }
         sum += v[q];
         if (v[q]) {
             ++ne;

@@ -6,10 +6,11 @@ import dataclasses
 import math
 
 import pytest
+import torch
 
 import oracle
-from paper_2503_12886_gb300 import synth
-from paper_2503_12886_gb300.rasterizer import Renderer
+from paper_2503_12886_gb300 import api, synth
+from paper_2503_12886_gb300.rasterizer import DeviceBatch, Renderer, stream_ptr
 
 from gpu_helpers import compare_decisions, read_intermediates, run_gpu_forward
 
@@ -56,3 +57,19 @@ def test_scan_by_one_cta(renderer, sizes):
     m = synth.make_model(104, 3000, 3)
     batch = synth.make_batch([m], [synth.Frame(0, w, h) for w, h in sizes], seed=104, jitter_deg=10)
     assert check(renderer, batch, (16, 16))["pairs"] > 0
+
+
+@pytest.mark.parametrize("sizes", [[(200, 150)], [(1024, 1024), (64, 48)], [(2049, 1999)]])
+def test_binning_again_gives_the_same_lists(renderer, sizes):
+    """rgba_bin_sort may run any number of times on one rgba_preprocess."""
+    m = synth.make_model(105, 2000, 3)
+    batch = synth.make_batch([m], [synth.Frame(0, w, h) for w, h in sizes], seed=105, jitter_deg=10)
+    db = DeviceBatch(batch, "cuda:0")
+    first, T, n = renderer.forward(db)
+    ws, b, s = renderer.ws, db.struct(), stream_ptr()
+    for _ in range(2):
+        api.rgba_bin_sort(renderer.ctx, b, ws.data_ptr(), ws.numel(), s)
+    compare_decisions(batch, oracle.forward(batch, do_render=False), read_intermediates(renderer, db), db)
+    img, T2, n2 = torch.empty_like(first), torch.empty_like(T), torch.empty_like(n)
+    api.rgba_render_fwd(renderer.ctx, b, ws.data_ptr(), ws.numel(), img.data_ptr(), T2.data_ptr(), n2.data_ptr(), s)
+    assert torch.equal(img, first) and torch.equal(T2, T) and torch.equal(n2, n)
