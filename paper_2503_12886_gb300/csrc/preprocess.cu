@@ -369,7 +369,7 @@ __device__ __forceinline__ void stage_frames(const Ctx &c, const ModelInfo &m, i
 // selection of the blend loop is resolved at compile time (a runtime mask costs a test, a
 // branch and an index update per channel and blendshape); MASK = 0 reads each model's mask.
 // SLOTS: frame slots per Gaussian, 4 where every model is rendered by at most eight frames, else 8.
-// Bound by latency at about half the issue slots: divisions, square roots and the records' 188 bytes per
+// Bound by latency at about half the issue slots: divisions, square roots and the 156 bytes it writes per
 // (frame, Gaussian). Four CTAs of eight slots per SM (64 registers, a few spilled) against three: 16 frames of
 // 60,000 Gaussians 68.5 -> 67.5 us, ten frames 42.8 -> 41.2. Four slots against eight with half of them idle: 64
 // frames of eight avatars, eight each, 325 -> 287 us.
@@ -489,7 +489,7 @@ k_preprocess(Ctx c, int max_k) {
 // blendshapes' loads in flight at once; the CTA's further groups of kFewG threads take the next
 // frames of the same Gaussians (their reads hit L1).
 // Staged against this: one frame of 60,000 Gaussians (K = 32, 73 MB of rows) 22 -> 19 us, 15 frames of five avatars
-// of up to 100,000 129 -> 123, three frames of 35,001 (K = 7) 16 -> 15; but one of 10,000 10 -> 11, where the
+// of up to 100,000 129 -> 116 (64 registers; 123 to 135 with 80), three frames of 35,001 (K = 7) 16 -> 15; but one of 10,000 10 -> 11, where the
 // staged copies have every row in flight at once, hence kFewMinN; and at eight frames a model the shared rows win
 // (64 frames of eight avatars: 287 us staged, 386 so).
 constexpr int kFewG = 64;      // Gaussians per CTA
@@ -497,7 +497,7 @@ constexpr int kFewFrames = 4;
 constexpr int kFewMinN = 20000;
 
 template <unsigned MASK, int FB>
-__global__ void __launch_bounds__(kFewG * (kFewFrames / FB))
+__global__ void __launch_bounds__(FB == 1 ? kFewG : kFewG * kFewFrames / FB, FB == 1 ? 16 : 8)
 k_preprocess_few(Ctx c, int max_k) {
     extern __shared__ float4 smem4[];
     __shared__ FrameConst s_fc[kFewFrames];
