@@ -462,19 +462,22 @@ def run_ours(args, rank, world, local_rank):
         # from the committed ncu capture: its warp instructions over the visits the counting
         # instances found in the same (seeded) profiled step
         ipv = traffic_for(comp, "render.cu", "warp_instructions_per_visit")
-        roof = {"bound": "alu", "kernel": kname, "achieved": ach,
-                "peak": fp32_peak_tflops, "unit": "TFLOP/s", "frac": ach / fp32_peak_tflops,
+        roof = {"bound": "alu", "kernel": kname, "achieved": useful,
+                "peak": fp32_peak_tflops, "unit": "TFLOP/s", "frac": useful / fp32_peak_tflops,
                 "traffic": traffic_for(comp, "render.cu"),
                 "peak_source": f"FP32 lanes x 2 x {clock_mhz:.0f} MHz (recipe unit counts)",
                 "units": units_bwd, "flops_per_unit": per_unit,
-                "accounting": "units = (pixel, list entry up to the pixel's last contributor), "
-                              f"{per_unit} FLOP each (the hot-path table's per-unit figures: "
-                              f"{FWD_FLOPS_PER_UNIT} forward, {BWD_FLOPS_PER_UNIT} backward)",
+                # most units never reach an instruction (the block masks drop them), so the
+                # table's figure for all of them no longer measures the kernel: it can pass the peak
+                "table_achieved": ach, "table_frac": ach / fp32_peak_tflops,
+                "table_accounting": "units = (pixel, list entry up to the pixel's last contributor), "
+                                    f"{per_unit} FLOP each (the hot-path table's per-unit figures: "
+                                    f"{FWD_FLOPS_PER_UNIT} forward, {BWD_FLOPS_PER_UNIT} backward)",
                 "blend_pairs": blends, "blend_fraction_of_units": blends / max(1, units_bwd),
                 "visits_fwd": rstats["fwd_visits"], "visits_bwd": rstats["bwd_visits"],
                 "lanes_blending_per_visit": blends / max(1, rstats["bwd_visits"]),
                 "useful_achieved": useful, "useful_frac": useful / fp32_peak_tflops,
-                "useful_accounting": f"units x {rej} FLOP (evaluate and cut) + blend pairs x "
+                "accounting": f"units x {rej} FLOP (evaluate and cut) + blend pairs x "
                                      f"{per_unit - rej} FLOP (composite and differentiate a "
                                      "blending entry)",
                 "warp_instructions_per_visit": ipv}
@@ -492,7 +495,7 @@ def run_ours(args, rank, world, local_rank):
     BN = FRAMES * N_GAUSS
     A, K = 9, K_BASES
     pre_bytes = 4 * N_GAUSS * (14 + K * A) + 48 * BN
-    pre_impl = 4 * N_GAUSS * (14 + K * A) + R * (48 + 8 + 48 + 48 + 32 + 4)
+    pre_impl = 4 * N_GAUSS * (14 + K * A) + R * (48 + 8 + 48 + 48 + 4)
     gbwd_bytes = 4 * N_GAUSS * (14 + 2 * K * A) + 36 * BN
     gbwd_impl = 4 * N_GAUSS * (14 + 2 * K * A) + R * (48 + 48) + FRAMES * K * 4
     stages = {k: {"ms": v} for k, v in stage_ms.items()}

@@ -194,7 +194,7 @@ int rgba_workspace_layout(const rgba_batch *batch, size_t ws_bytes, rgba_ws_layo
 int rgba_blend(rgba_ctx_t ctx, const rgba_batch *batch, float *out, void *stream);
 
 /* Fused blend (Eq. 1) + activations (Supp. A.3) + EWA projection + tile rectangle + depth key
- * for every (frame, Gaussian); counts the Gaussians of every (frame, tile). */
+ * for every (frame, Gaussian). */
 int rgba_preprocess(rgba_ctx_t ctx, const rgba_batch *batch, void *ws, size_t ws_bytes,
                     void *stream);
 
