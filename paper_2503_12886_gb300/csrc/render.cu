@@ -784,12 +784,12 @@ __device__ __forceinline__ void flush_loss(const Ctx &c, float loss_acc, float *
 // (flush_acc: one 16-byte reduction per entry and pixel block).
 // STATS (the counting instance): also count the visits that evaluate an entry and the
 // (pixel, entry) pairs that blend, into the compositing statistics of the counters.
-// Bound by instruction issue (67 % of the slots), and by the walks of the heaviest blocks: six CTAs per SM
+// Bound by instruction issue (63 to 67 % of the slots), and by the walks of the heaviest blocks: six CTAs per SM
 // beat eight (more warps, each slower) except where far more blocks have work than fit. Whole-warp
-// entries with a vote per entry, then this: 127 -> 121 us on 16 frames of 512 x 512 (N = 60,000), 248 ->
-// 182 us with the avatar bound to a mesh, 233 -> 160 us on 15 frames of 256 to 1,024 pixels of five
-// avatars, 594 -> 520 us on 64 of eight, 66 -> 49 us on one of 128 x 128, colour initialisation of ten
-// frames 107 -> 98 us. Empty tiles after all blocks instead of among the lighter ones: 559 us on the 64.
+// entries with a vote per entry, then the half blocks with cut entries: 127 -> 115 us on 16 frames of 512 x 512
+// (N = 60,000), 248 -> 182 us with the avatar bound to a mesh, 233 -> 148 us on 15 frames of 256 to 1,024 pixels of
+// five avatars, 594 -> 514 us on 64 of eight, 66 -> 37 us on one of 128 x 128, colour initialisation of ten
+// frames 107 -> 94 us. Empty tiles after all blocks instead of among the lighter ones: 559 us on the 64, before the cut.
 template <int TW, int S, bool ACC, bool STATS = false>
 __global__ void __launch_bounds__(32 * kWarpsPerCta, ACC ? 4 : 6)
 k_render_fwd(Ctx c, float *__restrict__ img, float *__restrict__ T_final, int *__restrict__ n_contrib,
@@ -859,11 +859,11 @@ k_render_fwd(Ctx c, float *__restrict__ img, float *__restrict__ T_final, int *_
 
 // STATS (the counting instance): also count the visits that evaluate an entry and the
 // (pixel, entry) pairs that take a gradient, into the compositing statistics of the counters.
-// Bound by instruction issue (65 % of the slots, 65 instructions per step of the two halves) and by the
+// Bound by instruction issue (66 % of the slots, about 65 instructions per step of the two halves) and by the
 // walks of the heaviest blocks: four CTAs per SM (128 registers) beat five and six. Whole-warp entries with
-// a vote per entry, then this: 16 frames of 512 x 512 of a 60,000-Gaussian avatar, not yet fitted, 170 ->
-// 152 us, bound to a mesh 344 -> 256, 64 frames of eight avatars 644 -> 588; one 128 x 128 frame, where only
-// 80 warps have work and the length of one warp's walk is what counts, 94 -> 53 us.
+// a vote per entry, then the half blocks with cut entries: 16 frames of 512 x 512 of a 60,000-Gaussian avatar, not yet
+// fitted, 170 -> 141 us, bound to a mesh 344 -> 240, 64 frames of eight avatars 644 -> 567; one 128 x 128 frame, where
+// only 96 warps have work and the length of one warp's walk is what counts, 94 -> 45 to 51 us.
 template <int TW, int S, bool STATS = false>
 __global__ void __launch_bounds__(32 * kWarpsPerCta, 4)
 k_render_bwd(Ctx c, const float *__restrict__ dl_dimg, const float *__restrict__ T_final,
