@@ -79,22 +79,23 @@ struct PixF {
 // the pixel: live = the pixel is still compositing and the entry passes the alpha cutoff. A live
 // entry that would take T (1 - alpha) below 1e-4 marks the pixel done without blending;
 // otherwise it blends. Branch-free, so a warp whose lanes disagree runs it once: a lane that is
-// not live keeps its state whatever its exponential gives (alpha is capped at 0.99 and its
-// weight is 0). Returns the splatting weight alpha T at the pixel (0 when the entry does not
-// blend).
+// not live keeps its state whatever its exponential gives. The colour is added under the same
+// condition and not with a weight of 0, which would carry an infinite or undefined colour to
+// every pixel the entry was staged for. Returns the splatting weight alpha T at the pixel (0 when the
+// entry does not blend).
 __device__ __forceinline__ float composite(PixF &p, bool live, float power, const float4 &Cc, int pos) {
     const float alpha = fminf(kAlphaMax, __fmul_rn(Cc.x, exp_ftz(power)));
     const float testT = p.T * (1.0f - alpha);
     const bool sat = testT < kTMin;
     p.done = p.done || (live && sat);
     const bool blend = live && !sat;
-    const float w = blend ? alpha * p.T : 0.0f;
-    p.C0 = fmaf(Cc.y, w, p.C0);
-    p.C1 = fmaf(Cc.z, w, p.C1);
-    p.C2 = fmaf(Cc.w, w, p.C2);
+    const float w = alpha * p.T;
+    p.C0 = blend ? fmaf(Cc.y, w, p.C0) : p.C0;
+    p.C1 = blend ? fmaf(Cc.z, w, p.C1) : p.C1;
+    p.C2 = blend ? fmaf(Cc.w, w, p.C2) : p.C2;
     p.T = blend ? testT : p.T;
     p.last = blend ? pos : p.last;
-    return w;
+    return blend ? w : 0.0f;
 }
 
 constexpr int kWarpsPerCta = 4;  // independent warps per CTA (they share nothing but the loss sum)
