@@ -566,6 +566,8 @@ struct PixB {
     int last;
 };
 
+__device__ __forceinline__ bool is_finite(float x) { return fabsf(x) < __int_as_float(0x7f800000); }
+
 __device__ __forceinline__ float rcp_ftz(float x) {
     float y;
     asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(y) : "f"(x));
@@ -599,11 +601,29 @@ __device__ __forceinline__ void accumulate(PixB &p, bool live, float power, cons
 }
 
 // Shared memory of the backward's gradient sums: per visit and pixel g = dL/dpower and the weight
-// w, and the block's dL/dcolour.
+// w, and the block's dL/dcolour, 0 in place of values that are not finite; odd: the pixels (one bit per
+// lane) that had any.
 struct __align__(16) GradMem {
     float d[kRows * kRowStride], w[kRows * kRowStride];
     float dl[3 * 32];
+    unsigned odd;
 };
+
+// The colour sums' part that is not finite: a pixel whose dL/dcolour is infinite or undefined (this lane's
+// is in g0, g1, g2) adds it only to the entries it blends, where in the products of flush_grads its zero weights
+// would make the sums of every staged entry undefined. dst: this lane's entry's colour sums, or nullptr. Not
+// inlined: it hardly ever runs, and the walk has no registers to spare.
+__device__ __noinline__ void add_odd(const GradMem &r, float g0, float g1, float g2, float *dst) {
+    const int lane = threadIdx.x & 31;
+    for (unsigned odd = r.odd; odd; odd &= odd - 1) {
+        const int q = __ffs((int)odd) - 1;
+        const float g[3] = {__shfl_sync(0xffffffffu, g0, q), __shfl_sync(0xffffffffu, g1, q), __shfl_sync(0xffffffffu, g2, q)};
+        const float w = r.w[(lane & 15) * kRowStride + q];
+        if (!dst || (lane ^ q) & 16 || w == 0.0f) continue;  // w: not in this half, not blended
+        for (int c = 0; c < 3; ++c)
+            if (!is_finite(g[c])) red_add(dst + c, w * g[c]);
+    }
+}
 
 // Adds the gradient sums of the entries in slots slot0 ... slot0 + 15 of each half (n[h] slots in all):
 // the sums over the half's pixels of g (dx, dy, dx^2, dx dy, dy^2, 1), (dx, dy) = pixel centre -
@@ -611,7 +631,7 @@ struct __align__(16) GradMem {
 // one number per pixel row, so the y moments come from the row sums.
 template <int S>
 __device__ __forceinline__ void flush_grads(const GradMem &r, const WarpMem<S> &m, const Walk &w, int slot0,
-                                            const int n[2], float *g2) {
+                                            const int n[2], const PixB &p, float *g2) {
     const int lane = threadIdx.x & 31, h = lane >> 4;
     const bool mine = slot0 + (lane & 15) < (h ? n[1] : n[0]);
     const int slot = mine ? slot0 + (lane & 15) : slot0;  // none: any other, its sums are not added
@@ -654,6 +674,7 @@ __device__ __forceinline__ void flush_grads(const GradMem &r, const WarpMem<S> &
         red_add4(dst + 4, t[4], t[5], t[6], t[7]);
         red_add(dst + 8, t[8]);
     }
+    if (r.odd) add_odd(r, p.g0, p.g1, p.g2, mine ? g2 + (size_t)m.half(h)[slot >> 1].idx[slot & 1] * kG2Floats + 6 : nullptr);
     __syncwarp();
 }
 
@@ -717,7 +738,7 @@ __device__ __forceinline__ void bwd_walk(const Walk &w, WarpMem<S> &m, GradMem &
                 gm.w[(j - j0) * kRowStride + lane] = w0;
                 gm.w[(j - j0 + 1) * kRowStride + lane] = w1;
             }
-            flush_grads<S>(gm, m, w, j0, n, g2);
+            flush_grads<S>(gm, m, w, j0, n, p, g2);
         }
         if (STATS) st.stage(reach);
     }
@@ -901,9 +922,12 @@ k_render_bwd(Ctx c, const float *__restrict__ dl_dimg, const float *__restrict__
             p.g2 = dl[2 * hw];
             p.TB = Tfin * (p.g0 * bgp[0] + p.g1 * bgp[1] + p.g2 * bgp[2]);
         }
-        gm.dl[lane] = p.g0;  // read by flush_grads, after its first __syncwarp
-        gm.dl[32 + lane] = p.g1;
-        gm.dl[64 + lane] = p.g2;
+        // read by flush_grads, after its first __syncwarp
+        gm.dl[lane] = is_finite(p.g0) ? p.g0 : 0.0f;
+        gm.dl[32 + lane] = is_finite(p.g1) ? p.g1 : 0.0f;
+        gm.dl[64 + lane] = is_finite(p.g2) ? p.g2 : 0.0f;
+        const unsigned odd = __ballot_sync(0xffffffffu, !(is_finite(p.g0) && is_finite(p.g1) && is_finite(p.g2)));
+        if (lane == 0) gm.odd = odd;
         int m = p.last;
         for (int o = 16; o > 0; o >>= 1) m = max(m, __shfl_xor_sync(0xffffffffu, m, o));
         // n_contrib comes from the caller: entries past the list's end do not exist

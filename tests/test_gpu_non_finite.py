@@ -1,5 +1,6 @@
 """Infinite and undefined values stay with the pixels and Gaussians they belong to. A Gaussian whose
-colour is not finite changes only the pixels that blend it, whatever else its splat was staged for."""
+colour is not finite changes only the pixels that blend it, whatever else its splat was staged for; a pixel whose
+dL/dimg is not finite makes the sums of the Gaussians that it blends undefined, and no others'."""
 import dataclasses
 
 import numpy as np
@@ -50,3 +51,40 @@ def test_a_colour_reaches_only_the_pixels_that_blend_it(renderer, tile, stage, v
     assert torch.equal(T, T0) and torch.equal(n, n0)
     assert torch.equal(got[:, ~blends], plain[:, ~blends])
     assert not bool(torch.isfinite(got[:, blends]).any())
+
+
+@pytest.mark.parametrize("value", [np.inf, -np.inf, np.nan])
+@pytest.mark.parametrize("channels", [(0,), (0, 1, 2)])
+@pytest.mark.parametrize("tile", [(16, 16), (8, 32)])
+@pytest.mark.parametrize("n", [2000, 30000])
+def test_a_pixel_gradient_reaches_only_what_the_pixel_blends(renderer, n, tile, channels, value):
+    """n: blocks of a few entries, and of several stages. The other Gaussians' sums equal those with 0 at these pixels,
+    up to the order of their additions (at most some 100 partial sums, one per half block, of which
+    the nine sums' magnitudes add: 2 * 100 * 2^-24 of the largest, times ten)."""
+    batch = batch_of(n)
+    db = DeviceBatch(batch, "cuda:0", tile=tile)
+    img, T, k = renderer.forward(db)
+    ys, xs = torch.meshgrid(torch.arange(5, 121, 23, device="cuda:0"), torch.arange(3, 173, 19, device="cuda:0"), indexing="ij")
+    bad = torch.zeros(121, 173, dtype=torch.bool, device="cuda:0")
+    bad[ys, xs] = True
+    clean = 1.0 + (torch.arange(img.numel(), device="cuda:0") % 7).view(3, 121, 173)
+
+    def sums(dl):
+        renderer.backward(db, dl.contiguous(), T, k)
+        lay = renderer.layout(db)
+        return renderer.ws[lay.grad2d: lay.grad2d + 48 * db.total_rec].view(torch.float32).view(-1, 12)[:, :9].clone()
+
+    owned = sums(bad.float().expand(3, -1, -1))[:, 6] > 0  # w times 1: what the pixels blend
+    assert 20 < int(owned.sum()) < n - 20
+    odd, ref = clean.clone(), clean.clone()
+    for c in range(3):
+        ref[c][bad] = 0.0
+        odd[c][bad] = value if c in channels else 0.0
+    got, want = sums(odd), sums(ref)
+    assert bool(torch.isfinite(got[~owned]).all()) and int((want[~owned] != 0).sum()) > 0
+    assert bool(((got - want)[~owned].abs() <= 1e-4 * want.abs().amax(0)).all())
+    for c in range(3):  # the channels whose gradient is finite keep their colour sums
+        if c in channels:
+            assert not bool(torch.isfinite(got[owned, 6 + c]).any())
+        else:
+            assert bool(((got - want)[:, 6 + c].abs() <= 1e-4 * want[:, 6 + c].abs().max()).all())
