@@ -8,7 +8,7 @@ namespace rgba {
 // The region where a splat reaches alpha 1/255: the ellipse a dx^2 + 2 b dx dy + c dy^2 <= s,
 // s = -2 alpha_cut(o), around (u, v).
 struct Reach {
-    bool none, all;  // never reaches it; too elongated to bound tightly
+    bool none, all;  // never reaches it (decides over all); too elongated to bound tightly
     float u, v, ia, b, det, as, ys, hy;
 };
 
@@ -27,7 +27,8 @@ __device__ __forceinline__ float sqrt_fast(float x) {
 __device__ __forceinline__ Reach reach_of(const float4 &r0, const float2 &r1) {
     Reach e;
     const float a = r0.z, b = r0.w, c = r1.x, tau = alpha_cut(r1.y);
-    const float det = a * c - b * b;
+    // by fixed operations, so that whoever asks gets the same none
+    const float det = __fmaf_rn(a, c, -__fmul_rn(b, b));
     e.none = !(tau < 0.0f && det > 0.0f);
     e.all = !(a * c < 1e4f * det);
     const float s = -2.04f * tau, id = __fdividef(1.0f, det);

@@ -299,11 +299,11 @@ __device__ __forceinline__ int commit(const Walk &w, const Stage<S> &g, WarpMem<
             const Reach e = reach_of(g.r0[s], make_float2(g.r1[s].x, g.r1[s].y));
             float xl, xr;
             tau = alpha_cut(g.r1[s].y);
-            const bool all = e.all || !w.masked;
+            const bool all = e.all || !w.masked;  // lists without masks are not cut, but for what reaches no pixel
             reach_rows(e, bl.y0, bl.y1, xl, xr);
-            left = bl.any && (all || (!e.none && xr >= bl.x0 && xl <= bl.x1));
+            left = bl.any && !e.none && (all || (xr >= bl.x0 && xl <= bl.x1));
             reach_rows(e, br.y0, br.y1, xl, xr);
-            right = br.any && (all || (!e.none && xr >= br.x0 && xl <= br.x1));
+            right = br.any && !e.none && (all || (xr >= br.x0 && xl <= br.x1));
         }
         const unsigned ml = __ballot_sync(0xffffffffu, left), mr = __ballot_sync(0xffffffffu, right);
         if (left) put_slot(m, 0, n[0] + __popc(ml & lt), g.r0[s], g.r1[s], g.r2[s], tau, g.id.pos[s], g.id.idx[s]);
