@@ -92,7 +92,9 @@ __device__ __forceinline__ unsigned bucket_of(unsigned v) { return 31u - __clz(v
 // and taking the places here) made the L2's atomic units and the wait for them the bound. Projection, count,
 // scan and scatter together, one atomic per touch in the projection, then this: 16 frames 148 -> 125 us, ten frames
 // 112 -> 87, 64 frames of eight avatars 661 -> 535, 15 frames of five 275 -> 220, one frame 60 -> 53. Frames of more
-// than kHistTiles tiles (1,773 pixels square) go touch by touch.
+// than kHistTiles tiles (1,773 pixels square) are taken in windows of whole tile rows, one after the other. Touch by
+// touch with global atomics, then this, count, scan and scatter: one frame of 1,800 x 1,800 (N = 60,000) 128 -> 41 us,
+// of 4,096 x 4,096 223 -> 143, of 2,048 x 2,048 under 2,000 splats of its size 14.2 -> 2.4 ms.
 constexpr int kBinThreads = 256;
 constexpr int kHistTiles = 12288;
 
@@ -100,42 +102,58 @@ constexpr int kHistTiles = 12288;
 // spread over all frames' tiles.
 struct BinItem {
     FrameInfo f;
-    int i, tiles;
-    bool valid, hist;
+    int i;
+    bool valid;
 };
 __device__ __forceinline__ BinItem bin_item(const Ctx &c) {
     BinItem b;
     b.f = c.frames[blockIdx.x];
     b.i = (int)((blockIdx.y + blockIdx.z * gridDim.y) * kBinThreads + threadIdx.x);
-    b.tiles = b.f.tiles_x * b.f.tiles_y;
     b.valid = b.i < b.f.n;
-    b.hist = b.tiles <= kHistTiles;
     return b;
 }
 
+// Calls f(y0, y1, tiles) for every window of the frame's tile rows, [y0, y1), whose tiles have a counter each, by the
+// whole CTA. WINDOWS: some frame of the batch has more than kHistTiles tiles (a row has at most 512); of several
+// windows those that no rectangle of the CTA meets are passed over, and the barrier in the vote keeps a window's
+// counters from the next one's. Otherwise the only window is the frame, and its bounds are compiled out: they cost
+// the scatter up to 15 registers, and 477 us instead of 448 on one frame of 1,024 x 1,024 with 64 splats of its size.
+template <bool WINDOWS, typename F>
+__device__ __forceinline__ void each_window(const FrameInfo &fr, const ushort4 &rc, F f) {
+    const int all = fr.tiles_x * fr.tiles_y;
+    if (!WINDOWS) return f(0, 0x7fffffff, all);
+    const int rows = all <= kHistTiles ? fr.tiles_y : kHistTiles / fr.tiles_x;
+    for (int y0 = 0; y0 < fr.tiles_y; y0 += rows) {
+        const int y1 = min(fr.tiles_y, y0 + rows);
+        if (rows < fr.tiles_y && !__syncthreads_or(rc.y < y1 && rc.w > y0 && rc.x < rc.z)) continue;
+        f(y0, y1, (y1 - y0) * fr.tiles_x);
+    }
+}
+static_assert(RGBA_MAX_DIM / 8 <= kHistTiles, "a window holds a row of tiles");
+
+// Calls f(t) for the rectangle's tiles in rows [y0, y1), t counted from row y0.
 template <typename F>
-__device__ __forceinline__ void each_tile(const ushort4 &rc, int tiles_x, F f) {
-    for (int ty = rc.y; ty < rc.w; ++ty)
-        for (int tx = rc.x; tx < rc.z; ++tx) f(ty * tiles_x + tx);
+__device__ __forceinline__ void each_tile(const ushort4 &rc, int tiles_x, int y0, int y1, F f) {
+    for (int ty = max((int)rc.y, y0); ty < min((int)rc.w, y1); ++ty)
+        for (int tx = rc.x; tx < rc.z; ++tx) f((ty - y0) * tiles_x + tx);
 }
 
+template <bool WINDOWS>
 __global__ void __launch_bounds__(kBinThreads) k_count(Ctx c) {
     extern __shared__ unsigned s_hist[];
     pdl_enter();
     const BinItem b = bin_item(c);
     if (b.i - (int)threadIdx.x >= b.f.n || b.i < 0) return;  // the whole CTA
     const ushort4 rc = b.valid ? c.rects[b.f.rec_base + b.i] : make_ushort4(0, 0, 0, 0);
-    unsigned *count = c.tile_count + b.f.tile_base;
-    if (!b.hist) {
-        each_tile(rc, b.f.tiles_x, [&](int t) { atomicAdd(count + t, 1u); });
-        return;
-    }
-    for (int t = threadIdx.x; t < b.tiles; t += kBinThreads) s_hist[t] = 0u;
-    __syncthreads();
-    each_tile(rc, b.f.tiles_x, [&](int t) { atomicAdd(s_hist + t, 1u); });
-    __syncthreads();
-    for (int t = threadIdx.x; t < b.tiles; t += kBinThreads)
-        if (s_hist[t]) atomicAdd(count + t, s_hist[t]);
+    each_window<WINDOWS>(b.f, rc, [&](int y0, int y1, int tiles) {
+        unsigned *count = c.tile_count + b.f.tile_base + y0 * b.f.tiles_x;
+        for (int t = threadIdx.x; t < tiles; t += kBinThreads) s_hist[t] = 0u;
+        __syncthreads();
+        each_tile(rc, b.f.tiles_x, y0, y1, [&](int t) { atomicAdd(s_hist + t, 1u); });
+        __syncthreads();
+        for (int t = threadIdx.x; t < tiles; t += kBinThreads)
+            if (s_hist[t]) atomicAdd(count + t, s_hist[t]);
+    });
 }
 
 // Phase 1, one thread per tile: the tile's total count into tile_start, and per CTA the sum, the number of
@@ -318,7 +336,7 @@ __global__ void __launch_bounds__(kScanTile) k_scan_one(Ctx c) {
 // entry of its list. TW: the tile width (16 or 8).
 // In shared memory the counts of the CTA's touches become, with one global atomic per touched tile, the
 // places its keys take in the lists.
-template <int TW>
+template <int TW, bool WINDOWS>
 __global__ void __launch_bounds__(kBinThreads) k_scatter(Ctx c) {
     extern __shared__ unsigned s_hist[];
     constexpr int TH = kTilePix / TW, NBX = TW / 8, BANDS = TH / 4;
@@ -334,38 +352,38 @@ __global__ void __launch_bounds__(kBinThreads) k_scatter(Ctx c) {
     const float4 r0 = c.records[r * 3];
     const float2 r1 = *reinterpret_cast<const float2 *>(c.records + r * 3 + 1);
     if (!b.valid) rc = make_ushort4(0, 0, 0, 0);
-    unsigned *cur = c.cursor + f.tile_base;
-    if (b.hist) {
-        for (int t = threadIdx.x; t < b.tiles; t += kBinThreads) s_hist[t] = 0u;
+    const Reach e = reach_of(r0, r1);
+    each_window<WINDOWS>(f, rc, [&](int y0, int y1, int tiles) {
+        unsigned *cur = c.cursor + f.tile_base + y0 * f.tiles_x;
+        for (int t = threadIdx.x; t < tiles; t += kBinThreads) s_hist[t] = 0u;
         __syncthreads();
-        each_tile(rc, f.tiles_x, [&](int t) { atomicAdd(s_hist + t, 1u); });
+        each_tile(rc, f.tiles_x, y0, y1, [&](int t) { atomicAdd(s_hist + t, 1u); });
         __syncthreads();
-        for (int t = threadIdx.x; t < b.tiles; t += kBinThreads)
+        for (int t = threadIdx.x; t < tiles; t += kBinThreads)
             if (s_hist[t]) s_hist[t] = atomicAdd(cur + t, s_hist[t]);
         __syncthreads();
-    }
-    if (rc.z <= rc.x || rc.w <= rc.y) return;
-    const Reach e = reach_of(r0, r1);
-    for (int ty = rc.y; ty < rc.w; ++ty) {
-        float xl[BANDS], xr[BANDS];
+        if (rc.z <= rc.x) return;
+        for (int ty = max((int)rc.y, y0); ty < min((int)rc.w, y1); ++ty) {
+            float xl[BANDS], xr[BANDS];
 #pragma unroll
-        for (int k = 0; k < BANDS; ++k) reach_rows(e, (float)(ty * TH + 4 * k) + 0.5f, (float)(ty * TH + 4 * k) + 3.5f, xl[k], xr[k]);
-        for (int tx = rc.x; tx < rc.z; ++tx) {
-            unsigned mask = 0u;
+            for (int k = 0; k < BANDS; ++k) reach_rows(e, (float)(ty * TH + 4 * k) + 0.5f, (float)(ty * TH + 4 * k) + 3.5f, xl[k], xr[k]);
+            unsigned *place = s_hist + (ty - y0) * f.tiles_x;
+            for (int tx = rc.x; tx < rc.z; ++tx) {
+                unsigned mask = 0u;
 #pragma unroll
-            for (int k = 0; k < BANDS; ++k)
+                for (int k = 0; k < BANDS; ++k)
 #pragma unroll
-                for (int q = 0; q < NBX; ++q) {
-                    const float x0 = (float)(tx * TW + 8 * q) + 0.5f;
-                    if (xr[k] >= x0 && xl[k] <= x0 + 7.0f) mask |= 1u << (k * NBX + q);
-                }
-            if (e.all) mask = 0xffu;
-            if (e.none) mask = 0u;
-            const int t = ty * f.tiles_x + tx;
-            const unsigned pos = b.hist ? atomicAdd(s_hist + t, 1u) : atomicAdd(cur + t, 1u);
-            c.keys[pos] = ((unsigned long long)bits << 32) | pack_low(c.masked, (unsigned)b.i, mask);
+                    for (int q = 0; q < NBX; ++q) {
+                        const float x0 = (float)(tx * TW + 8 * q) + 0.5f;
+                        if (xr[k] >= x0 && xl[k] <= x0 + 7.0f) mask |= 1u << (k * NBX + q);
+                    }
+                if (e.all) mask = 0xffu;
+                if (e.none) mask = 0u;
+                const unsigned pos = atomicAdd(place + tx, 1u);
+                c.keys[pos] = ((unsigned long long)bits << 32) | pack_low(c.masked, (unsigned)b.i, mask);
+            }
         }
-    }
+    });
 }
 
 constexpr int kSortThreads = 512;
@@ -911,13 +929,14 @@ size_t bin_smem(int max_tiles) { return 4 * (size_t)std::min(max_tiles, kHistTil
 
 cudaError_t launch_count(const Ctx &c, int max_n, int max_tiles, cudaStream_t s) {
     if (c.B == 0 || max_n == 0) return cudaSuccess;
-    return launch_pdl(k_count, bin_grid(c, max_n), dim3(kBinThreads), bin_smem(max_tiles), s, c);
+    return launch_pdl(max_tiles > kHistTiles ? k_count<true> : k_count<false>, bin_grid(c, max_n), dim3(kBinThreads), bin_smem(max_tiles), s, c);
 }
 
 cudaError_t launch_scatter(const Ctx &c, int max_n, int max_tiles, cudaStream_t s) {
     if (c.B == 0 || max_n == 0) return cudaSuccess;
-    return launch_pdl(c.tw == 16 ? k_scatter<16> : k_scatter<8>, bin_grid(c, max_n), dim3(kBinThreads),
-                      bin_smem(max_tiles), s, c);
+    const bool w = max_tiles > kHistTiles;
+    return launch_pdl(c.tw == 16 ? (w ? k_scatter<16, true> : k_scatter<16, false>) : (w ? k_scatter<8, true> : k_scatter<8, false>),
+                      bin_grid(c, max_n), dim3(kBinThreads), bin_smem(max_tiles), s, c);
 }
 
 cudaError_t launch_tile_sort(const Ctx &c, int sms, cudaStream_t s) {
