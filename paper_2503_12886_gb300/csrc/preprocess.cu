@@ -368,13 +368,13 @@ __device__ __forceinline__ void stage_frames(const Ctx &c, const ModelInfo &m, i
 // MASK != 0: every model of the batch blends exactly the channels in MASK, so the channel
 // selection of the blend loop is resolved at compile time (a runtime mask costs a test, a
 // branch and an index update per channel and blendshape); MASK = 0 reads each model's mask.
-// SLOTS: frame slots per Gaussian, 4 where every model is rendered by at most eight frames, else 8.
+// SLOTS: frame slots per Gaussian, 4 where every model is rendered by at most eight frames, else 8. CTAS: resident
+// CTAs per SM that the registers allow (preprocess_inst).
 // Bound by latency at about half the issue slots: divisions, square roots and the 156 bytes it writes per
-// (frame, Gaussian). Four CTAs of eight slots per SM (64 registers, a few spilled) against three: 16 frames of
-// 60,000 Gaussians 68.5 -> 67.5 us, ten frames 42.8 -> 41.2. Four slots against eight with half of them idle: 64
-// frames of eight avatars, eight each, 325 -> 287 us.
-template <unsigned MASK, int SLOTS>
-__global__ void __launch_bounds__(kPreG * SLOTS, SLOTS == 8 ? 4 : 6)
+// (frame, Gaussian). Four slots against eight with half of them idle: 64 frames of eight avatars, eight each,
+// 325 -> 287 us.
+template <unsigned MASK, int SLOTS, int CTAS>
+__global__ void __launch_bounds__(kPreG * SLOTS, CTAS)
 k_preprocess(Ctx c, int max_k) {
     constexpr int kPreRound = pre_round(SLOTS), kPreBlock = kPreG * SLOTS;
     extern __shared__ float4 smem4[];
@@ -661,42 +661,58 @@ cudaError_t preprocess_few(const Ctx &c, int max_n, int max_nb, int max_k, cudaS
                       c, max_k);
 }
 
-template <unsigned MASK, int SLOTS>
+template <unsigned MASK, int SLOTS, int CTAS>
 cudaError_t preprocess_slots(const Ctx &c, int max_n, int max_k, int max_rows, cudaStream_t s) {
     static int attr_device = -1;
     int dev = 0;
     cudaError_t e = cudaGetDevice(&dev);
     if (e != cudaSuccess) return e;
     if (attr_device != dev) {  // once, at the largest size (K = 64, 13 blended channels)
-        e = cudaFuncSetAttribute(k_preprocess<MASK, SLOTS>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+        e = cudaFuncSetAttribute(k_preprocess<MASK, SLOTS, CTAS>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                  preprocess_smem(RGBA_MAX_K, kNch + RGBA_MAX_K * 13));
         if (e != cudaSuccess) return e;
         attr_device = dev;
     }
     dim3 grid((max_n + kPreG - 1) / kPreG, c.M);
-    return launch_pdl(k_preprocess<MASK, SLOTS>, grid, dim3(kPreG * SLOTS), preprocess_smem(max_k, max_rows), s, c, max_k);
+    return launch_pdl(k_preprocess<MASK, SLOTS, CTAS>, grid, dim3(kPreG * SLOTS), preprocess_smem(max_k, max_rows), s, c, max_k);
 }
 
+// Registers of the staged instances (projection times of 60,000 Gaussians):
+// - Channel masks compiled in: four CTAs of eight slots per SM (64 registers, 32 or 74 bytes spilled) against three,
+//   16 frames (K = 32) 68.5 -> 67.5 us, ten frames 42.8 -> 41.2; six CTAs of four slots (80 registers).
+// - Batches with a bound model: three. The mapping through the TBN frame has more values live, and four never won:
+//   16 frames with K = 32 94 us with four and 91 with three, with K = 40 120 and 100.
+// - A mask read at run time needs the registers in the loop over the blendshapes, where spills cost most: two CTAs of
+//   eight slots or five of four. 13 channels with four or six, three of eight, and this: 16 frames (K = 32) 147, 116
+//   and 86 us, 17 frames (K = 64) 580, 421 and 184, one frame (K = 64) 202, 198 and 75. Up to kFewRows blendshape
+//   rows the loop is short and four of eight slots stay: 24 frames (K = 4, three channels) 75 and not 83 us.
+constexpr int kFewRows = 64;
+
 template <unsigned MASK>
-cudaError_t preprocess_inst(const Ctx &c, int max_n, int max_nb, int max_k, int max_rows, cudaStream_t s) {
+cudaError_t preprocess_inst(const Ctx &c, int max_n, int max_nb, int max_k, int max_rows, bool any_bound, cudaStream_t s) {
+    const bool few_frames = max_nb <= pre_round(4);
     if constexpr (MASK != 0u) {
         if (max_nb <= kFewFrames && max_n >= kFewMinN)
             return max_nb == 1 ? preprocess_few<MASK, 1>(c, max_n, max_nb, max_k, s)
                                : preprocess_few<MASK, 2>(c, max_n, max_nb, max_k, s);
+        if (few_frames) return preprocess_slots<MASK, 4, 6>(c, max_n, max_k, max_rows, s);
+        if (any_bound) return preprocess_slots<MASK, 8, 3>(c, max_n, max_k, max_rows, s);
+    } else {
+        if (few_frames) return preprocess_slots<MASK, 4, 5>(c, max_n, max_k, max_rows, s);
+        if (max_rows > kNch + kFewRows) return preprocess_slots<MASK, 8, 2>(c, max_n, max_k, max_rows, s);
     }
-    return max_nb <= pre_round(4) ? preprocess_slots<MASK, 4>(c, max_n, max_k, max_rows, s)
-                                  : preprocess_slots<MASK, 8>(c, max_n, max_k, max_rows, s);
+    return preprocess_slots<MASK, 8, 4>(c, max_n, max_k, max_rows, s);
 }
 }  // namespace
 
 cudaError_t launch_preprocess(const Ctx &c, int max_n, int max_nb, int max_k, int max_rows, unsigned common_mask,
-                              cudaStream_t s) {
+                              bool any_bound, cudaStream_t s) {
     if (c.B == 0 || max_n == 0) return cudaSuccess;
     if (common_mask == RGBA_MASK_MEAN_SCALE_COLOR)
-        return preprocess_inst<RGBA_MASK_MEAN_SCALE_COLOR>(c, max_n, max_nb, max_k, max_rows, s);
+        return preprocess_inst<RGBA_MASK_MEAN_SCALE_COLOR>(c, max_n, max_nb, max_k, max_rows, any_bound, s);
     if (common_mask == RGBA_MASK_MEAN_ROT_COLOR)
-        return preprocess_inst<RGBA_MASK_MEAN_ROT_COLOR>(c, max_n, max_nb, max_k, max_rows, s);
-    return preprocess_inst<0u>(c, max_n, max_nb, max_k, max_rows, s);
+        return preprocess_inst<RGBA_MASK_MEAN_ROT_COLOR>(c, max_n, max_nb, max_k, max_rows, any_bound, s);
+    return preprocess_inst<0u>(c, max_n, max_nb, max_k, max_rows, any_bound, s);
 }
 
 cudaError_t launch_blend(const Ctx &c, int max_n, float *out, cudaStream_t s) {

@@ -212,8 +212,9 @@ struct PrologueArgs {
 cudaError_t launch_prologue(const PrologueArgs &a, const void *const src[3], cudaStream_t s);
 // max_nb: the most frames any model is rendered by. common_mask: the channel mask every model of the
 // batch shares (0 when they differ); the two masks of the RGBA_MASK_* constants run a blend specialised at compile time.
+// any_bound: some model has a tangent-space binding.
 cudaError_t launch_preprocess(const Ctx &c, int max_n, int max_nb, int max_k, int max_rows, unsigned common_mask,
-                              cudaStream_t s);
+                              bool any_bound, cudaStream_t s);
 cudaError_t launch_blend(const Ctx &c, int max_n, float *out, cudaStream_t s);
 // max_tiles: the most tiles of any frame of the batch
 cudaError_t launch_count(const Ctx &c, int max_n, int max_tiles, cudaStream_t s);
