@@ -389,13 +389,12 @@ __global__ void __launch_bounds__(kBinThreads) k_scatter(Ctx c) {
 constexpr int kSortThreads = 512;
 constexpr int kSortWarps = kSortThreads / 32;
 // Shared memory of the sort: 96 KB, so that two CTAs share an SM. The bucket sort takes kSmemCap keys
-// and 2^kMaxBits 2-byte bucket counts; the radix sort kRadixCap keys twice, their ranks and the digit counts;
+// and 2^kMaxBits 2-byte bucket counts; the radix sort kSmemCap keys, their ranks and the digit counts;
 // the sort of long lists 2^kStreamBits 4-byte bucket counts.
 constexpr int kSmemCap = 16 * kSortThreads;
 constexpr int kMaxBits = 14;
-constexpr int kRadixCap = 4544;
 constexpr int kSortSmem = kSmemCap * 8 + (2 << kMaxBits) + 16;
-static_assert(kRadixCap * (2 * 8 + 2) + (kSortWarps * 256 + kSortWarps) * 4 <= kSortSmem, "radix sort fits");
+static_assert(kSmemCap * (8 + 2) + kSortWarps * 256 * 4 <= kSortSmem, "radix sort fits");
 constexpr int kDigitParts = kSortThreads / 256;  // threads sharing one digit's column of warp counts
 static_assert(kSortThreads % 256 == 0 && 32 % kDigitParts == 0, "whole digits per warp");
 
@@ -413,24 +412,25 @@ __device__ __forceinline__ unsigned digit_peers(unsigned act, unsigned d) {
 }
 
 // Stable LSD radix sort of L keys on the bits [shift0, shift_end), 8-bit digits; a and b are both in
-// shared memory or both in global memory. Warp w owns the contiguous run [w S, (w+1) S) of the
+// global memory, or a is in shared memory and b unused (kInPlace, L <= kSmemCap). Warp w owns the contiguous run [w S, (w+1) S) of the
 // input; within a warp, rounds of 32 keys go in order and lanes are ranked by lane index among
 // equal digits (digit_peers), so the order of equal digits is kept and the result after the
-// last pass is fully sorted. With kCacheRanks each key's rank within its warp's run of equal
-// digits is kept from the counting sweep (s_rank, L entries) and the scatter sweep only adds the
-// digit base; without it the scatter sweep ranks again. Returns the buffer holding the result.
+// last pass is fully sorted. In place, each key's rank within its warp's run of equal digits is kept from
+// the counting sweep (s_rank, L entries); the scatter sweep takes the keys into registers, all of the CTA's
+// before any is written, and only adds the digit base. Otherwise it ranks again. Returns the buffer
+// holding the result. A second shared-memory buffer in place of the registers holds 4,544 keys beside two CTAs
+// per SM; longer crowded lists then sort in global memory: one list of 8,192 keys, 900 of them at one depth,
+// 133 us, of 4,545 86, 300 lists of 6,000 172; in place 55, 35 and 70.
 constexpr int kRounds = 4;  // rounds of 32 keys whose loads the radix sweeps issue together
 
-template <bool kCacheRanks>
+template <bool kInPlace>
 __device__ unsigned long long *radix_sort(unsigned long long *a, unsigned long long *b, int L,
-                                          int shift0, int shift_end,
-                                          unsigned *s_cnt /* [warps][256] + [warps] */,
-                                          unsigned short *s_rank) {
+                                          int shift0, int shift_end, unsigned *s_cnt /* [kSortWarps][256] */,
+                                          unsigned *s_sum /* [kSortWarps] */, unsigned short *s_rank) {
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     const int S = ((L + kSortWarps - 1) / kSortWarps + 31) & ~31;
     const int lo = warp * S, hi = min(L, lo + S);
     unsigned *cnt = s_cnt + warp * 256;
-    unsigned *wsum = s_cnt + kSortWarps * 256;
     const unsigned lt_mask = (1u << lane) - 1u;
     // thread (digit d, part q) owns the counts of digit d in warps [q W/P, (q+1) W/P)
     const int d_own = threadIdx.x / kDigitParts, w_own = (threadIdx.x % kDigitParts) * (kSortWarps / kDigitParts);
@@ -458,7 +458,7 @@ __device__ unsigned long long *radix_sort(unsigned long long *a, unsigned long l
                     d = (unsigned)(kk[u] >> shift) & 255u;
                     peers = digit_peers(act, d);
                     before = cnt[d];
-                    if (kCacheRanks) s_rank[e] = (unsigned short)(before + __popc(peers & lt_mask));
+                    if (kInPlace) s_rank[e] = (unsigned short)(before + __popc(peers & lt_mask));
                 }
                 __syncwarp();
                 if (ok && (peers & lt_mask) == 0) cnt[d] = before + __popc(peers);
@@ -483,20 +483,31 @@ __device__ unsigned long long *radix_sort(unsigned long long *a, unsigned long l
                 const unsigned y = __shfl_up_sync(0xffffffffu, x, o);
                 if (lane >= o) x += y;
             }
-            if (lane == 31) wsum[warp] = x;
+            if (lane == 31) s_sum[warp] = x;
             __syncthreads();
             unsigned off = x - run;
 #pragma unroll
-            for (int q = 0; q < kSortWarps; ++q) off += q < warp ? wsum[q] : 0u;
+            for (int q = 0; q < kSortWarps; ++q) off += q < warp ? s_sum[q] : 0u;
 #pragma unroll
             for (int w = w_own; w < w_own + kSortWarps / kDigitParts; ++w) s_cnt[w * 256 + d_own] += off;
         }
         __syncthreads();
-        if (kCacheRanks) {
-            for (int e = lo + lane; e < hi; e += 32) {
-                const unsigned long long k = a[e];
-                b[cnt[(unsigned)(k >> shift) & 255u] + s_rank[e]] = k;
+        if (kInPlace) {
+            constexpr int KPT = kSmemCap / kSortThreads;
+            unsigned long long k[KPT];
+#pragma unroll
+            for (int u = 0; u < KPT; ++u) {
+                const int e = lo + 32 * u + lane;
+                k[u] = e < hi ? a[e] : 0ull;
             }
+            __syncthreads();
+#pragma unroll
+            for (int u = 0; u < KPT; ++u) {
+                const int e = lo + 32 * u + lane;
+                if (e < hi) a[cnt[(unsigned)(k[u] >> shift) & 255u] + s_rank[e]] = k[u];
+            }
+            __syncthreads();
+            continue;
         } else {
             for (int base0 = lo; base0 < hi; base0 += kRounds * 32) {
                 unsigned long long kk[kRounds];
@@ -741,7 +752,7 @@ __device__ bool bucket_sort_stream(const unsigned long long *g, unsigned long lo
 // (depth, Gaussian index), "index" standing here for the word that also holds the block mask below
 // the index. A segment of up to kSmemCap keys is sorted by bucket_sort, with more keys per thread and
 // more buckets the longer it is, a longer one by bucket_sort_stream with its keys in
-// global memory (mostly L2). A bucket longer than kBucketRun sends a segment of up to kRadixCap keys to a
+// global memory (mostly L2). A bucket longer than kBucketRun sends a segment of up to kSmemCap keys to a
 // full-key radix sort in shared memory (index bits, then depth bits), and a longer one to a radix sort in
 // global memory on the depth bits only, which leaves runs of equal depth in list order; a tie pass orders
 // each such run by index (insertion sort by the run's first thread), a run longer than kTieRun the full key.
@@ -825,10 +836,10 @@ __global__ void __launch_bounds__(kSortThreads, 2) k_tile_sort(Ctx c) {
             if ((threadIdx.x & 31) == 0) atomicMax(&s_imax, imax);
             const unsigned d0 = s_dmin;
             const int db = 32 - __clz(s_dmax - d0);  // bits of the depth spread
-            const bool radix_smem = L <= (unsigned)kRadixCap;
-            unsigned long long *a = radix_smem ? s_keys : c.keys2 + st, *bb = radix_smem ? s_keys + kRadixCap : c.keys + st;
-            unsigned short *rank = reinterpret_cast<unsigned short *>(s_keys + 2 * kRadixCap);
-            unsigned *cnt = reinterpret_cast<unsigned *>(rank + kRadixCap);
+            unsigned long long *a = in_smem ? s_keys : c.keys2 + st, *bb = in_smem ? nullptr : c.keys + st;
+            unsigned short *rank = reinterpret_cast<unsigned short *>(s_keys + kSmemCap);
+            unsigned *cnt = reinterpret_cast<unsigned *>(rank + kSmemCap);
+            const int shift0 = c.masked ? 8 : 0;  // of the index below its mask
             for (unsigned e = threadIdx.x; e < L; e += blockDim.x) {
                 const unsigned long long k = g[e];
                 a[e] = ((unsigned long long)((unsigned)(k >> 32) - d0) << 32) | (unsigned)k;
@@ -836,11 +847,11 @@ __global__ void __launch_bounds__(kSortThreads, 2) k_tile_sort(Ctx c) {
             __syncthreads();
             const int ib = 32 - __clz(s_imax);  // bits of the largest index (0 if 0)
             unsigned long long *res;
-            if (radix_smem) {
-                res = radix_sort<true>(a, bb, (int)L, 0, ib, cnt, rank);
-                res = radix_sort<true>(res, res == a ? bb : a, (int)L, 32, 32 + db, cnt, rank);
+            if (in_smem) {
+                res = radix_sort<true>(a, bb, (int)L, shift0, ib, cnt, s_sum, rank);
+                res = radix_sort<true>(a, bb, (int)L, 32, 32 + db, cnt, s_sum, rank);
             } else {
-                res = radix_sort<false>(a, bb, (int)L, 32, 32 + db, cnt, nullptr);
+                res = radix_sort<false>(a, bb, (int)L, 32, 32 + db, cnt, s_sum, nullptr);
                 // ties: a run keeps its depth under any reordering, so run starts found by other
                 // threads do not change while a run is being ordered
                 for (unsigned e = threadIdx.x; e + 1 < L; e += blockDim.x) {
@@ -863,9 +874,9 @@ __global__ void __launch_bounds__(kSortThreads, 2) k_tile_sort(Ctx c) {
                 __syncthreads();
                 if (s_long) {
                     unsigned long long *other = res == a ? bb : a;
-                    res = radix_sort<false>(res, other, (int)L, 0, ib, cnt, nullptr);
+                    res = radix_sort<false>(res, other, (int)L, shift0, ib, cnt, s_sum, nullptr);
                     other = res == a ? bb : a;
-                    res = radix_sort<false>(res, other, (int)L, 32, 32 + db, cnt, nullptr);
+                    res = radix_sort<false>(res, other, (int)L, 32, 32 + db, cnt, s_sum, nullptr);
                 }
             }
             if (res == g) {  // the masks go over this buffer: finish from the other one
