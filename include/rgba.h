@@ -121,8 +121,10 @@ typedef struct {
     const float *fparams;       /* device [n_frames][RGBA_FP_STRIDE] */
     float *grad_psi;            /* device [n_frames][k_stride] or NULL, overwritten */
     int32_t tile_w, tile_h;     /* screen tile shape: 16x16 or 8x32 (tile_w * tile_h == 256) */
-    int32_t smem_batch;         /* staging size of a compositing warp: 64, 128 or 256 (0: 64) stage 32, 64
-                                   or 96 of the entries that reach its pixel block at a time */
+    int32_t smem_batch;         /* staging size of a compositing warp, 64, 128 or 256 (0: 64): in the forward
+                                   64 stages 32 of the entries that reach its pixel block at a time, 128 and
+                                   256 stage 64. The backward stages 32 whatever the value, and batches of at
+                                   most 512 tiles stage 64 in both. Results do not depend on it */
     int32_t loss_frames;        /* frames the batch loss is averaged over: 0 = n_frames; a rank of
                                    a frame-sharded data-parallel step passes the global batch size
                                    (>= n_frames), so that its loss and gradients are its share of

@@ -95,6 +95,12 @@ TILES = ((16, 16), (8, 32))
 SMEM_BATCHES = (64, 128, 256)
 
 
+def _kernels_of(smem_batch: int) -> int:
+    """The staging size of the kernels that a value of rgba_batch.smem_batch selects: 0 means 64, and 256
+    selects what 128 does."""
+    return min(smem_batch or 64, 128)
+
+
 def workload_signature(batch: synth.Batch) -> str:
     ns = sorted({(m.n, m.k) for m in batch.models})
     res = sorted({(f.width, f.height) for f in batch.frames})
@@ -106,7 +112,8 @@ def autotune(renderer: Renderer, batch: synth.Batch, targets, steps: int = 5,
     """Times the whole training step for every (tile shape, staging size) and keeps the fastest.
 
     Each candidate builds its own device batch (the tile shape changes the binning), runs one
-    sizing step, then `steps` timed steps with CUDA events. Results are cached per workload
+    sizing step, then `steps` timed steps with CUDA events. Staging sizes that select the same
+    kernels share one timing, and of those the first wins. Results are cached per workload
     signature in cache_path (JSON) when given."""
     sig = workload_signature(batch)
     if cache_path and os.path.exists(cache_path):
@@ -118,7 +125,12 @@ def autotune(renderer: Renderer, batch: synth.Batch, targets, steps: int = 5,
     table = {}
     models = None
     for tile in tiles:
+        timed = {}
         for sb in smem_batches:
+            key = f"{tile[0]}x{tile[1]}/{sb}"
+            if _kernels_of(sb) in timed:
+                table[key] = timed[_kernels_of(sb)]
+                continue
             db = DeviceBatch(batch, f"cuda:{renderer.device}", tile=tile, smem_batch=sb,
                              models=models)
             models = db.models
@@ -132,7 +144,7 @@ def autotune(renderer: Renderer, batch: synth.Batch, targets, steps: int = 5,
                 renderer.step(db, tg, api.RGBA_LOSS_L1, img)
             e1.record()
             torch.cuda.synchronize()
-            table[f"{tile[0]}x{tile[1]}/{sb}"] = e0.elapsed_time(e1) / steps
+            table[key] = timed[_kernels_of(sb)] = e0.elapsed_time(e1) / steps
     best = min(table, key=table.get)
     tw, th = (int(x) for x in best.split("/")[0].split("x"))
     res = TuneResult((tw, th), int(best.split("/")[1]), table[best], table)
