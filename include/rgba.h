@@ -305,7 +305,7 @@ int rgba_debug_keys(rgba_ctx_t ctx, const rgba_batch *batch, const void *ws, siz
                     void *stream);
 
 /* Per-stage device timing with CUDA events on the call's stream (off by default). Stages, in
- * launch order: 0 table upload, 1 preprocess (fused blend + projection), 2 tile-count scan,
+ * launch order: 0 table upload, 1 preprocess (fused blend + projection), 2 tile counts and scan,
  * 3 pair scatter, 4 per-tile depth sort, 5 compositing forward (+ fused loss), 6 compositing
  * backward, 7 projection + blend backward, 8 weight-gradient reduction. Do not enable it while
  * capturing a CUDA graph. */
@@ -367,11 +367,11 @@ int rgba_color_init(rgba_ctx_t ctx, const rgba_batch *batch, void *ws, size_t ws
  *    in the layouts of rgba_render_fwd; out (host) receives the pair count.
  *  - Limits: a batch whose workspace (rgba_workspace_size with capacity = the batch's total
  *    Gaussian records) does not fit the block returns RGBA_ERR_INVALID_ARG before anything is
- *    enqueued. The block holds the full rgba_step layout, so roughly 208 bytes per Gaussian
+ *    enqueued. The block holds the full rgba_step layout, so roughly 176 bytes per Gaussian
  *    record (a frame's record count is its model's n_pad; 20 of them are the one pair per record
- *    that must fit) + 32 bytes per pixel + 110-140 bytes per tile must fit in 64 MiB: one 512x512
- *    frame of a 100,000-Gaussian avatar (about 29 MB) or two of them fit, three do not; 16
- *    frames of 512x512 of a 60,000-Gaussian avatar need about 335 MB and are rejected. More
+ *    that must fit) and K / 8 + 32 bytes per pixel + 16 bytes per tile must fit in 64 MiB: one 512x512
+ *    frame of a 100,000-Gaussian avatar (about 26 MB) or two of them fit, three do not; 16
+ *    frames of 512x512 of a 60,000-Gaussian avatar need about 307 MB and are rejected. More
  *    pairs than fit in what is left return RGBA_ERR_CAPACITY with out->pairs_needed set (the
  *    outputs are then not written), and an out-of-range tangent-space binding index returns
  *    RGBA_ERR_INVALID_ARG, both after the call's one synchronisation. A NULL img, T_final or

@@ -144,7 +144,7 @@ __device__ __forceinline__ void chain(const float v[10], float op, const float *
 }
 
 // TBN matrix and barycentric point of Gaussian i in one frame (the same definitions as the
-// preprocess, fp32 without its fixed rounding order): out[12] as recompute() reads it.
+// preprocess, fp32 without its fixed rounding order): out[12] as chain() reads it.
 __device__ __forceinline__ bool tbn_fast(const ModelInfo &m, const float *__restrict__ verts, int i, float out[12]) {
     const int f = __ldg(m.face_of + i);
     if ((unsigned)f >= (unsigned)m.n_faces) return false;
@@ -283,7 +283,6 @@ k_gauss_bwd(Ctx c, int max_k, int max_ka, AdamArg<ADAM> fa) {
     if (i0 >= m.n_pad || m.nb == 0) return;
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     const int i = i0 + lane;
-    const bool valid = i < m.n;      // real Gaussian
     const bool in_pad = i < m.n_pad; // row slot (padding slots receive zeros)
     const int K = m.k, A = m.A;
     float ibc1 = 0.f, ibc2 = 0.f;

@@ -3,7 +3,7 @@
 // tile of its rectangle and each (frame, tile) list is ordered by (depth bits, Gaussian index).
 //
 // Design: a kernel counts the rectangles' tiles, a three-phase scan (per-CTA
-// partials, one CTA over the partials, per-CTA writes) turns the counts into list offsets and a work list, a scatter
+// partials, one CTA over the partials, per-CTA writes; one CTA in all for few tiles) turns the counts into list offsets and a work list, a scatter
 // kernel drops (depth << 32 | index) keys, with a mask of the pixel blocks each splat reaches in
 // the low byte of the index word, into their tile's segment, and
 // one CTA per non-empty tile sorts its list: in shared memory by one bucket pass on the top depth bits and a placement of every key by its rank in its bucket,
@@ -758,7 +758,7 @@ __device__ bool bucket_sort_stream(const unsigned long long *g, unsigned long lo
 // each such run by index (insertion sort by the run's first thread), a run longer than kTieRun the full key.
 // The radix sorts take keys compressed to (depth - min depth) << 32 | index.
 // Bound by the shared-memory passes over the keys and, for short lists, by the load and the barriers
-// between them, so two CTAs share an SM. Keys moved between two shared-memory buffers with 2^12 buckets
+// between them, so two CTAs share an SM, at 64 registers with 136 bytes spilled. Keys moved between two shared-memory buffers with 2^12 buckets
 // whatever the length (one CTA per SM, lists of 8,193 to 12,288 keys by positions), then this: one frame with lists
 // of up to 6,321 keys 35 -> 16 us, 15 frames of five avatars 145 -> 80, 16 frames 55 -> 43, ten frames 43 -> 31,
 // 64 frames of eight avatars with lists of up to 24,552 keys 268 -> 188. The same with one CTA of 1,024

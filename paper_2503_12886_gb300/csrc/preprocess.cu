@@ -1,5 +1,5 @@
-// Fused blend + activation + EWA projection + tile binning count (the "preprocess" stage of
-// the batch-parallel rasterizer, RGBAvatar Sec. 3.2 / Supp. A.3, built on 3DGS), and the
+// Fused blend + activation + EWA projection to tile rectangles and depths (the "preprocess" stage
+// of the batch-parallel rasterizer, RGBAvatar Sec. 3.2 / Supp. A.3, built on 3DGS), and the
 // standalone Eq. 1 blend.
 //
 // The base Gaussians and blendshapes are read from HBM once per step: a CTA stages its chunk's
@@ -56,7 +56,7 @@ struct UploadBlob {
 
 // The step's prologue in one launch: CTA 0 copies up to three host tables (packed in the blob
 // at 16-byte offsets) to the workspace and zeroes the counters; every CTA zeroes its share of
-// the per-tile counts, which the preprocess then counts into.
+// the per-tile counts, which the binning then counts into.
 __global__ void k_prologue(PrologueArgs a, UploadBlob blob) {
     pdl_enter();  // the previous step's kernels may still read the tables and counts
     const uint4 z = make_uint4(0u, 0u, 0u, 0u);
@@ -99,7 +99,7 @@ __device__ __forceinline__ void blend14(const ModelInfo &m, const float *__restr
 // per-Gaussian spec would use, so staging them changes no bit.
 struct FrameConst {
     float limx, limy;
-    int tiles_x, tiles_y, tile_base, rec_base;
+    int tiles_x, tiles_y, rec_base;
     const float *verts;  // the frame's deformed mesh (bound models)
 };
 
@@ -352,7 +352,6 @@ __device__ __forceinline__ void stage_frames(const Ctx &c, const ModelInfo &m, i
         fc.limy = fmul(1.3f, fdiv(fmul(0.5f, (float)f.H), fp[13]));
         fc.tiles_x = f.tiles_x;
         fc.tiles_y = f.tiles_y;
-        fc.tile_base = f.tile_base;
         fc.rec_base = f.rec_base;
         fc.verts = f.verts;
         s_fc[tid] = fc;
@@ -489,7 +488,8 @@ k_preprocess(Ctx c, int max_k) {
 // blendshapes' loads in flight at once; the CTA's further groups of kFewG threads take the next
 // frames of the same Gaussians (their reads hit L1).
 // Staged against this: one frame of 60,000 Gaussians (K = 32, 73 MB of rows) 22 -> 19 us, 15 frames of five avatars
-// of up to 100,000 129 -> 116 (64 registers; 123 to 135 with 80), three frames of 35,001 (K = 7) 16 -> 15; but one of 10,000 10 -> 11, where the
+// of up to 100,000 129 -> 116 (64 registers, two frames per thread with 112 or 156 bytes spilled; 123 to 135 us with
+// 80 registers), three frames of 35,001 (K = 7) 16 -> 15; but one of 10,000 10 -> 11, where the
 // staged copies have every row in flight at once, hence kFewMinN; and at eight frames a model the shared rows win
 // (64 frames of eight avatars: 287 us staged, 386 so).
 constexpr int kFewG = 64;      // Gaussians per CTA

@@ -61,8 +61,7 @@ __device__ __forceinline__ float2 power_of(float pxc, float pyc, const float4 &A
 __device__ __forceinline__ bool skip(float power, float tau) { return power > 0.0f || power < tau; }
 
 // e^x for the compositing, as 2^(x log2 e) on the hardware's base-2 exponential in its
-// flush-to-zero form: the general form guards against subnormal results with three more
-// instructions, and no weight that counts (alpha >= 1/255) is near that range.
+// flush-to-zero form: no weight that counts (alpha >= 1/255) is near the subnormal range.
 __device__ __forceinline__ float exp_ftz(float x) {
     float y;
     asm("ex2.approx.ftz.f32 %0, %1;" : "=f"(y) : "f"(__fmul_rn(x, 1.44269504088896341f)));
@@ -967,7 +966,8 @@ cudaError_t fwd_inst(const Ctx &c, int grid, float *img, float *T, int *n, const
 }
 
 // Stages of 64 entries instead of 32: in the forward where the caller asks for staging of 128 or 256, and in both
-// directions for batches of at most kFewTiles tiles, whose blocks do not fill the SMs: their time is that of the longest
+// directions for batches of at most kFewTiles tiles, whose blocks do not fill the SMs (a larger batch of mostly empty
+// tiles may not fill them either, but how many are empty is known on the device only): their time is that of the longest
 // walks, which larger stages shorten (fewer waits for records). With 32 and with 64 entries: one
 // 64 x 64 frame of 100,000 Gaussians 852 against
 // 688 us forwards and 866 against 612 backwards, eight of 128 x 128 272 against 238 and 336 against 270, one of
