@@ -600,29 +600,11 @@ __device__ __forceinline__ void accumulate(PixB &p, bool live, float power, cons
 }
 
 // Shared memory of the backward's gradient sums: per visit and pixel g = dL/dpower and the weight
-// w, and the block's dL/dcolour, 0 in place of values that are not finite; odd: the pixels (one bit per
-// lane) that had any.
+// w, and the block's dL/dcolour, 0 in place of values that are not finite.
 struct __align__(16) GradMem {
     float d[kRows * kRowStride], w[kRows * kRowStride];
     float dl[3 * 32];
-    unsigned odd;
 };
-
-// The colour sums' part that is not finite: a pixel whose dL/dcolour is infinite or undefined (this lane's
-// is in g0, g1, g2) adds it only to the entries it blends, where in the products of flush_grads its zero weights
-// would make the sums of every staged entry undefined. dst: this lane's entry's colour sums, or nullptr. Not
-// inlined: it hardly ever runs, and the walk has no registers to spare.
-__device__ __noinline__ void add_odd(const GradMem &r, float g0, float g1, float g2, float *dst) {
-    const int lane = threadIdx.x & 31;
-    for (unsigned odd = r.odd; odd; odd &= odd - 1) {
-        const int q = __ffs((int)odd) - 1;
-        const float g[3] = {__shfl_sync(0xffffffffu, g0, q), __shfl_sync(0xffffffffu, g1, q), __shfl_sync(0xffffffffu, g2, q)};
-        const float w = r.w[(lane & 15) * kRowStride + q];
-        if (!dst || (lane ^ q) & 16 || w == 0.0f) continue;  // w: not in this half, not blended
-        for (int c = 0; c < 3; ++c)
-            if (!is_finite(g[c])) red_add(dst + c, w * g[c]);
-    }
-}
 
 // Adds the gradient sums of the entries in slots slot0 ... slot0 + 15 of each half (n[h] slots in all):
 // the sums over the half's pixels of g (dx, dy, dx^2, dx dy, dy^2, 1), (dx, dy) = pixel centre -
@@ -630,7 +612,7 @@ __device__ __noinline__ void add_odd(const GradMem &r, float g0, float g1, float
 // one number per pixel row, so the y moments come from the row sums.
 template <int S>
 __device__ __forceinline__ void flush_grads(const GradMem &r, const WarpMem<S> &m, const Walk &w, int slot0,
-                                            const int n[2], const PixB &p, float *g2) {
+                                            const int n[2], float *g2) {
     const int lane = threadIdx.x & 31, h = lane >> 4;
     const bool mine = slot0 + (lane & 15) < (h ? n[1] : n[0]);
     const int slot = mine ? slot0 + (lane & 15) : slot0;  // none: any other, its sums are not added
@@ -673,8 +655,27 @@ __device__ __forceinline__ void flush_grads(const GradMem &r, const WarpMem<S> &
         red_add4(dst + 4, t[4], t[5], t[6], t[7]);
         red_add(dst + 8, t[8]);
     }
-    if (r.odd) add_odd(r, p.g0, p.g1, p.g2, mine ? g2 + (size_t)m.half(h)[slot >> 1].idx[slot & 1] * kG2Floats + 6 : nullptr);
     __syncwarp();
+}
+
+// The colour gradients of a pixel whose dL/dcolour is infinite or undefined, over list positions [0, top): those values,
+// which no weight changes, go to the entries that the pixel blends and to no others. In flush_grads, which takes 0 in
+// their place, the zero weights of the other entries staged for the block would make their sums undefined.
+__device__ __forceinline__ void odd_colours(const Walk &w, const PixB &p, int top, float *g2) {
+#pragma unroll 1
+    for (int k = min(p.last, top); k > 0; --k) {
+        if (!((w.masks[k - 1] >> w.blk) & 1u)) continue;
+        const size_t i = w.list[k - 1];
+        const float4 r0 = w.rec[i * 3], r1 = w.rec[i * 3 + 1];
+        const float hc = -0.5f * r1.x;
+        const float power = power_of(p.pxc, p.pyc, make_float4(-r0.x, -r0.x, -r0.y, -r0.y),
+                                     make_float4(-0.5f * r0.z, -0.5f * r0.z, -r0.w, -r0.w), make_float2(hc, hc)).x;
+        if (skip(power, alpha_cut(r1.y)) || reach_of(r0, make_float2(r1.x, r1.y)).none) continue;
+        float *dst = g2 + i * kG2Floats + 6;
+        if (!is_finite(p.g0)) red_add(dst, p.g0);
+        if (!is_finite(p.g1)) red_add(dst + 1, p.g1);
+        if (!is_finite(p.g2)) red_add(dst + 2, p.g2);
+    }
 }
 
 // The reverse walk of one pixel block over list positions [0, top), top the block's largest
@@ -737,10 +738,13 @@ __device__ __forceinline__ void bwd_walk(const Walk &w, WarpMem<S> &m, GradMem &
                 gm.w[(j - j0) * kRowStride + lane] = w0;
                 gm.w[(j - j0 + 1) * kRowStride + lane] = w1;
             }
-            flush_grads<S>(gm, m, w, j0, n, p, g2);
+            flush_grads<S>(gm, m, w, j0, n, g2);
         }
         if (STATS) st.stage(reach);
     }
+    // hardly ever true, and after the walk, which must not pay for it: tested in every flush, the heaviest blocks took
+    // 10 % longer (one 64 x 64 frame of 100,000 Gaussians 603 -> 660 us), tested before the walk, 5 us at 128 x 128
+    if (!(is_finite(p.g0) && is_finite(p.g1) && is_finite(p.g2))) odd_colours(w, p, last, g2);
 }
 
 // A (tile, pixel block) item: its frame, the block's pixel (one per lane: the block's left 4 x 4 pixels
@@ -925,12 +929,12 @@ k_render_bwd(Ctx c, const float *__restrict__ dl_dimg, const float *__restrict__
         gm.dl[lane] = is_finite(p.g0) ? p.g0 : 0.0f;
         gm.dl[32 + lane] = is_finite(p.g1) ? p.g1 : 0.0f;
         gm.dl[64 + lane] = is_finite(p.g2) ? p.g2 : 0.0f;
-        const unsigned odd = __ballot_sync(0xffffffffu, !(is_finite(p.g0) && is_finite(p.g1) && is_finite(p.g2)));
-        if (lane == 0) gm.odd = odd;
         int m = p.last;
         for (int o = 16; o > 0; o >>= 1) m = max(m, __shfl_xor_sync(0xffffffffu, m, o));
         // n_contrib comes from the caller: entries past the list's end do not exist
-        bwd_walk<S, STATS>(w, s_m[wid], gm, p, c.grad2d + (size_t)f.rec_base * kG2Floats, min(m, w.len), st);
+        const int top = min(m, w.len);
+        float *g2 = c.grad2d + (size_t)f.rec_base * kG2Floats;
+        bwd_walk<S, STATS>(w, s_m[wid], gm, p, g2, top, st);
     }
     if (STATS) flush_stats(c.cnt->st_bwd, st);
     // the last warp out puts the work counter back to zero for the next launch
